@@ -292,7 +292,8 @@ size_t sd_verify_layer_workspace(int B, int R, int Hq, int Hkv, int D, int capac
  *   SD_ATTN_BLOCK_MASK of sd_verify_attention_ex).
  * For head_dim 128 this is one kernel: the tcgen05 kernel for G * R <= 128
  * and R <= 31 (R <= 16 when a causal layer has G * R <= 32: its 32-row tile
- * is causal only, so block-masked layers always take the 64-row tile);
+ * holds 16 new rows and is causal only, so block-masked layers always take the
+ * wider tiles);
  * other shapes run the three kernels in sequence (sd_verify_kernel names the
  * choice). A scene whose append would pass the
  * capacity sets SD_DEVERR_KV_OVERFLOW and is left untouched.

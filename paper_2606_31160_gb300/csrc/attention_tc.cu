@@ -9,8 +9,10 @@
 // MMA's M side and no padding waste:
 //     S^T[128 keys][kR rows] = K_tile[128 keys][128 d] . Q^T      (K-major A, B)
 //     O^T[128 d][kR rows]   += V_tile^T[128 d][128 keys] . P^T     (MN-major A, B)
-// kR = 32 (G*R <= 32) or 64 (G*R <= 64, and m-blocks of 64 rows up to 128);
-// an N = 64 product costs about what an N = 32 one does. Both accumulators
+// kR = 32 (G*R <= 32). More rows, and block-masked layers, take the wide tiles of
+// attention_wide.cu; with more new rows than either holds beside its prefix
+// loop (17 to 128, few query heads a KV head) the attention runs here with every
+// key in the loop, on 32 rows or m-blocks of kR = 64. Both accumulators
 // live in tensor memory, S triple-buffered: 4 kR columns.
 //
 // Warp roles in a CTA (352 threads). The issuing warps run converged: every
@@ -47,9 +49,7 @@
 // shared memory, never re-read from the cache) enter as one more partial that
 // each CTA forms on the CUDA cores for the rows it merges. Every wait is
 // bounded (SD_DEVERR_TIMEOUT instead of a hang).
-#include "common.cuh"
-
-#include <cuda.h>
+#include "tc_common.cuh"
 
 #include <math.h>
 #include <stdlib.h>
@@ -60,7 +60,6 @@ SD_DEFINE_ERROR_ACCESSOR(sd_take_error_attention_tc)
 
 namespace {
 
-constexpr int kD = 128;         // head dim
 constexpr int kStageKeys = 128; // M of S^T
 constexpr int kHalf = kStageKeys * 128;     // one 64-column half of a 128-key tile (16 KB)
 constexpr int kKV = 2 * kHalf;              // one K (or V) tile of 128 keys (32 KB)
@@ -69,7 +68,6 @@ constexpr int kSoftWarps = 8;
 constexpr int kSoftThreads = 32 * kSoftWarps;
 constexpr int kPvWarp = 2 + kSoftWarps;        // the warp after the softmax warps issues PV
 constexpr int kThreads = 96 + kSoftThreads;
-constexpr uint32_t kSpinLimit = 1u << 20;
 constexpr float kSlack = 64.f;              // log2 units a score may exceed its reference by
 // a partial row sent to its owner is [O(128) | l by TMEM lane quarter (4) | m |
 // 3 pad] fp32 = 544 bytes (16-byte multiple: one bulk copy per peer)
@@ -77,7 +75,6 @@ constexpr int kRowF = kD + 8;
 constexpr int kRowL = kD;       // the four l terms (float4)
 constexpr int kRowM = kD + 4;   // the row's reference m
 constexpr int kRowBytes = kRowF * 4;
-constexpr int round_up(int x, int m) { return (x + m - 1) / m * m; }
 
 // Everything that depends on the packed query rows per CTA (kR = 32 or 64:
 // the N of both MMAs). A softmax thread owns kR / 2 rows of one key lane.
@@ -85,7 +82,7 @@ template <int kR>
 struct Cfg {
   static_assert(kR == 32 || kR == 64, "row tile");
   static constexpr int kRpt = kR / 2;                       // rows per softmax thread
-  static constexpr int kMaxNew = kR == 32 ? 16 : 32;        // new rows the fused kernel takes
+  static constexpr int kMaxNew = 16;                        // new rows beside the loop (32-row tile)
   // K and V rings of kStages tiles each: a K slot is free once its S product
   // is done, a V slot once its PV product is
   static constexpr int kStages = kR == 32 ? 3 : 2;
@@ -114,9 +111,9 @@ struct Cfg {
   // barriers: full_k[S] full_v[S] p_full[2] s_ready[3] pv_done[S] q_full recv
   // decide s_free[3] tmem_done
   static constexpr int kNumBars = 3 * kStages + 12;
-  // tmem slot, (unused), decision, len (and, 64 rows, the last reader of the new key rows)
+  // tmem slot, (unused), decision, len
   static constexpr int kOffMisc = round_up(kOffBar + kNumBars * 8, 16);
-  static constexpr int kOffRowA = kOffMisc + (kR == 32 ? 16 : 32);  // [kR] per-row results (reductions)
+  static constexpr int kOffRowA = kOffMisc + 16;            // [kR] per-row results (reductions)
   static constexpr int kOffRef = kOffRowA + kR * 4;         // [kR] per-row references
   static constexpr int kOffLim = kOffRef + kR * 4;          // [kR] per-row causal key limits
   static constexpr int kSmemBytes = kOffLim + kR * 4 + 1024;
@@ -135,99 +132,6 @@ struct Cfg {
   static_assert(kNewS + kR * kMaxNew * 4 <= kRing, "merge buffers");
 };
 
-__device__ __forceinline__ uint32_t smem_addr(const void* p) {
-  return static_cast<uint32_t>(__cvta_generic_to_shared(p));
-}
-__device__ __forceinline__ void mbar_init(uint32_t bar, uint32_t count) {
-  asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(bar), "r"(count) : "memory");
-}
-__device__ __forceinline__ void mbar_expect_tx(uint32_t bar, uint32_t bytes) {
-  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes)
-               : "memory");
-}
-__device__ __forceinline__ void mbar_arrive(uint32_t bar) {
-  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
-}
-__device__ __forceinline__ bool mbar_try_wait(uint32_t bar, uint32_t parity) {
-  uint32_t ok;
-  asm volatile(
-      "{\n\t.reg .pred p;\n\t"
-      "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
-      "selp.u32 %0, 1, 0, p;\n\t}"
-      : "=r"(ok)
-      : "r"(bar), "r"(parity)
-      : "memory");
-  return ok != 0;
-}
-__device__ __noinline__ void mbar_timed_out() { sd_set_error(SD_DEVERR_TIMEOUT); }
-// One small loop per call site (the timeout report is out of line): the code
-// that the warps run at the same time must stay inside the instruction cache.
-__device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity) {
-#pragma unroll 1
-  for (uint32_t i = 0; i < kSpinLimit; ++i)
-    if (mbar_try_wait(bar, parity)) return true;
-  mbar_timed_out();
-  return false;
-}
-__device__ __forceinline__ void tma_load_3d(uint32_t dst, const CUtensorMap* map, uint32_t bar,
-                                            int x, int y, int z) {
-  asm volatile(
-      "cp.async.bulk.tensor.3d.shared::cluster.global.tile.mbarrier::complete_tx::bytes"
-      " [%0], [%1, {%3, %4, %5}], [%2];" ::"r"(dst),
-      "l"(reinterpret_cast<uint64_t>(map)), "r"(bar), "r"(x), "r"(y), "r"(z)
-      : "memory");
-}
-// The same load with an L2 eviction policy (createpolicy): the cached prefix is
-// read once per step, so its lines go first and the code and the per-step rows
-// stay in L2 (an instruction fetch that misses L2 waits behind the stream).
-__device__ __forceinline__ void tma_load_3d_hint(uint32_t dst, const CUtensorMap* map, uint32_t bar, int x, int y,
-                                                 int z, uint64_t policy) {
-  asm volatile(
-      "cp.async.bulk.tensor.3d.shared::cluster.global.tile.mbarrier::complete_tx::bytes.L2::cache_hint"
-      " [%0], [%1, {%3, %4, %5}], [%2], %6;" ::"r"(dst),
-      "l"(reinterpret_cast<uint64_t>(map)), "r"(bar), "r"(x), "r"(y), "r"(z), "l"(policy)
-      : "memory");
-}
-__device__ __forceinline__ uint64_t l2_evict_first_policy() {
-  uint64_t p;
-  asm volatile("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(p));
-  return p;
-}
-__device__ __forceinline__ void tma_prefetch_3d(const CUtensorMap* map, int x, int y, int z) {
-  asm volatile("cp.async.bulk.prefetch.tensor.3d.L2.global.tile [%0, {%1, %2, %3}];" ::"l"(
-                   reinterpret_cast<uint64_t>(map)),
-               "r"(x), "r"(y), "r"(z)
-               : "memory");
-}
-__device__ __forceinline__ void bulk_prefetch_l2(const void* p, uint32_t bytes) {
-  asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(reinterpret_cast<uint64_t>(p)), "r"(bytes)
-               : "memory");
-}
-__device__ __forceinline__ float ex2(float x) {
-  float y;
-  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
-  return y;
-}
-// two floats -> bf16x2 (round to nearest even), lo in the low half
-__device__ __forceinline__ uint32_t cvt_bf16x2(float lo, float hi) {
-  uint32_t r;
-  asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(r) : "f"(hi), "f"(lo));
-  return r;
-}
-__device__ __forceinline__ void named_bar_sync(int id, int threads) {
-  asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(threads) : "memory");
-}
-// bar.sync over `threads` threads that also ORs a predicate across them
-__device__ __forceinline__ bool named_bar_or(int id, int threads, bool p) {
-  uint32_t r;
-  asm volatile(
-      "{\n\t.reg .pred pi, po;\n\tsetp.ne.u32 pi, %1, 0;\n\t"
-      "bar.red.or.pred po, %2, %3, pi;\n\tselp.u32 %0, 1, 0, po;\n\t}"
-      : "=r"(r)
-      : "r"(static_cast<uint32_t>(p)), "r"(id), "r"(threads)
-      : "memory");
-  return r != 0;
-}
 // Sum over the 32 lanes of a warp of each of kN per-lane values (kN = 16 or
 // 32), by a butterfly reduce-scatter: at the step of stride s a lane keeps the
 // half of its values selected by its bit s and adds its partner's copy of that
@@ -256,94 +160,6 @@ __device__ __forceinline__ float warp_rows_sum(const float (&v0)[kN], int lane, 
   row = r;
   return x;
 }
-// an arrival that orders nothing: no data passes through the barrier
-__device__ __forceinline__ void cluster_arrive_relaxed() {
-  asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");
-}
-__device__ __forceinline__ void cluster_wait() {
-  asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
-}
-// shared::cta -> shared::cluster bulk copy, completing on the destination's mbarrier
-__device__ __forceinline__ void bulk_copy_s2s(uint32_t dst_cluster, uint32_t src_cta, uint32_t bytes,
-                                              uint32_t bar_cluster) {
-  asm volatile(
-      "cp.async.bulk.shared::cluster.shared::cta.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
-          dst_cluster),
-      "r"(src_cta), "r"(bytes), "r"(bar_cluster)
-      : "memory");
-}
-__device__ __forceinline__ uint32_t cluster_map(uint32_t addr, uint32_t rank) {
-  uint32_t r;
-  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
-  return r;
-}
-__device__ __forceinline__ void st_shared_v4(uint32_t addr, uint32_t x, uint32_t y, uint32_t z,
-                                             uint32_t w) {
-  asm volatile("st.shared.v4.u32 [%0], {%1,%2,%3,%4};" ::"r"(addr), "r"(x), "r"(y), "r"(z), "r"(w)
-               : "memory");
-}
-// ---------------------------------------------------------------- tcgen05
-// Shared-memory matrix descriptor (sm_100 family format): start address,
-// leading / stride byte offsets (>> 4), version 1, layout type (2 = 128-byte
-// swizzle, 4 = 64-byte swizzle).
-__device__ __forceinline__ uint64_t umma_desc(uint32_t addr, uint32_t lbo, uint32_t sbo,
-                                              uint64_t layout = 2) {
-  return static_cast<uint64_t>((addr >> 4) & 0x3FFF) |
-         (static_cast<uint64_t>((lbo >> 4) & 0x3FFF) << 16) |
-         (static_cast<uint64_t>((sbo >> 4) & 0x3FFF) << 32) | (1ull << 46) | (layout << 61);
-}
-// Instruction descriptor, kind::f16: fp32 accumulate, bf16 A and B.
-constexpr uint32_t umma_idesc(int M, int N, int a_mn_major, int b_mn_major) {
-  return (1u << 4) | (1u << 7) | (1u << 10) | (static_cast<uint32_t>(a_mn_major) << 15) |
-         (static_cast<uint32_t>(b_mn_major) << 16) | (static_cast<uint32_t>(N >> 3) << 17) |
-         (static_cast<uint32_t>(M >> 4) << 24);
-}
-
-__device__ __forceinline__ void umma(uint32_t d_tmem, uint64_t a, uint64_t b, uint32_t idesc,
-                                     int accumulate) {
-  asm volatile(
-      "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(d_tmem),
-      "l"(a), "l"(b), "r"(idesc), "r"(accumulate)
-      : "memory");
-}
-__device__ __forceinline__ __nv_bfloat162 as_bf162(uint32_t w) {
-  __nv_bfloat162 v;
-  memcpy(&v, &w, 4);
-  return v;
-}
-// one lane of the (converged) warp
-__device__ __forceinline__ bool elect_one() {
-  uint32_t pred = 0;
-  asm volatile(
-      "{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}"
-      : "=r"(pred));
-  return pred != 0;
-}
-__device__ __forceinline__ void umma_commit(uint32_t bar) {
-  asm volatile(
-      "tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar)
-      : "memory");
-}
-__device__ __forceinline__ void tc_fence_before() {
-  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-}
-__device__ __forceinline__ void tc_fence_after() {
-  asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-}
-
-// 16 consecutive fp32 columns of this warp's 32 TMEM lanes -> 16 registers
-__device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t (&r)[16]) {
-  asm volatile(
-      "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,"
-      "%14,%15}, [%16];"
-      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]),
-        "=r"(r[7]), "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]),
-        "=r"(r[14]), "=r"(r[15])
-      : "r"(taddr));
-  asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-}
-
 // Per-row reduction (max or sum) over the 128 key lanes of a CTA, for the 256
 // softmax threads: thread (key lane kl, rows row0 .. row0 + kN - 1) contributes
 // v[j] to row row0 + j. The values pass through buf ([2 kN rows][128] fp32,
@@ -407,33 +223,6 @@ __device__ __noinline__ void redo_references(int kl, int row0, int st, int quart
   asm volatile("bar.sync 2, 256;" ::: "memory");
 }
 
-struct TcArgs {
-  const __nv_bfloat16* q;   // rotated q rows (standalone attention)
-  __nv_bfloat16* out;
-  int32_t* len;
-  // fused verify layer only
-  __nv_bfloat16* qw;        // raw q rows, rotated in place
-  __nv_bfloat16* k_new;     // raw new key rows [B][R][Hkv][D], rotated in place
-  const __nv_bfloat16* v_new;
-  __nv_bfloat16* kc;        // cache K / V [B][Hkv][cap][D] (append target)
-  __nv_bfloat16* vc;
-  const int32_t* pos;       // [B][R][3]
-  uint32_t* ticket;         // [B] per-scene CTA tickets (zeroed, re-armed)
-  uint32_t* kv_ticket;      // [B][Hkv] read-before-write-back tickets (several m-blocks)
-  // kernels whose new keys enter as S_new: bit 0 = prefix, len (and pos) may
-  // be read before the dependency wait, bit 1 = the block mask (every new row
-  // sees all R new rows); the all-keys kernel: nonzero = the block mask
-  int early;
-  int R, Hq, Hkv, G, M, cap, n_mblocks;
-  float inv_g;              // 1 / G: p / G == int((p + 0.5) / G) exactly for the p < 128 used here
-  float scale_log2;
-};
-
-__device__ __forceinline__ void griddep_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
-__device__ __forceinline__ void griddep_launch() {
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-}
-
 // ------------------------------------------------------------------ kernel
 // kMode 0: attention over a cache that already holds the R new rows, every
 // key in the tensor-core loop, the rotated query rows read from a.q.
@@ -458,10 +247,10 @@ __global__ void __launch_bounds__(kThreads, 1)
   constexpr bool kNew = kMode != 0;  // the R new keys enter as S_new, not as tiles
   // prefix (and len) before the dependency wait; the block mask
   const bool early = kMode == 1 || (kMode == 2 && (a.early & 1) != 0);
-  // (the fused layer's 32-row tile takes no block mask: its callers are the
-  // target's causal verify steps; the host sends block-masked layers of up to
-  // 32 packed rows to the 64-row tile)
-  const bool block = kMode == 0 ? a.early != 0 : ((kMode == 2 || kR == 64) && (a.early & 2) != 0);
+  // (the fused layer takes no block mask here: its callers are the target's
+  // causal verify steps; the host sends block-masked layers of up to 32 packed
+  // rows to the wide tiles)
+  const bool block = kMode == 0 ? a.early != 0 : (kMode == 2 && (a.early & 2) != 0);
   constexpr int kS = C::kStages;
   constexpr int kRpt = C::kRpt;
   constexpr uint32_t kIdescS = umma_idesc(128, kR, 0, 0);
@@ -498,7 +287,6 @@ __global__ void __launch_bounds__(kThreads, 1)
   constexpr int kSB = C::kSBuf;
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(smem + C::kOffMisc);
   int* s_redo = reinterpret_cast<int*>(smem + C::kOffMisc + 8);
-  int* s_kvlast = reinterpret_cast<int*>(smem + C::kOffMisc + 16);  // 64 rows only
   float* row_a = reinterpret_cast<float*>(smem + C::kOffRowA);  // [kR] reduction results
   float* row_ref = reinterpret_cast<float*>(smem + C::kOffRef); // [kR] references
   int* row_lim = reinterpret_cast<int*>(smem + C::kOffLim);      // [kR] last key a row sees
@@ -814,8 +602,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                    ((static_cast<long long>(b) * a.R + i) * a.Hq + kvh * a.G + (p - i * a.G)) * kD + c * 8;
         q_cs[u] = i * 64 + c * 4;
       }
-      // new key / value rows: chunk st + u * 256 (row >> 4, 16-byte chunk & 15);
-      // one chunk a thread with 32 rows (16 new rows), two with 64 (32)
+      // new key / value rows: chunk st (row >> 4, 16-byte chunk & 15), one a thread
       const bool append = kFused && valid && rank == csize - 1 && mblock == 0;
       bool has_kv[kKvc];
       long long kv_src[kKvc];
@@ -908,20 +695,6 @@ __global__ void __launch_bounds__(kThreads, 1)
         mbar_arrive(QFULL);
         // every older kernel has finished: the next layer may launch
         if (kNew) griddep_launch();
-        // with several m-blocks the head's raw key rows are read by several
-        // clusters: the last of the head's CTAs to have read them writes the
-        // rotated rows back (the fence orders this CTA's reads before its ticket)
-        if constexpr (kR == 64) {
-          if (kFused && valid) {
-            if (a.n_mblocks > 1) {
-              __threadfence();
-              *s_kvlast = atomicAdd(&a.kv_ticket[b * a.Hkv + kvh], 1u) ==
-                          static_cast<uint32_t>(csize * a.n_mblocks - 1);
-            } else {
-              *s_kvlast = rank == csize - 1;
-            }
-          }
-        }
       }
     }
 
@@ -1258,8 +1031,8 @@ __global__ void __launch_bounds__(kThreads, 1)
     if (kFused && valid) {
       // while the partials travel: every CTA of the cluster read the raw rows
       // before its tiles (the cluster barrier above is behind all of them), so
-      // the rotated query rows this CTA merges go back to q, and the head's
-      // last reader of the raw key rows writes the rotated ones back to k_new
+      // the rotated query rows this CTA merges go back to q, and the last rank
+      // writes the rotated key rows back to k_new
 #pragma unroll 1
       for (int idx = st; idx < my_rows * 16; idx += kSoftThreads) {
         const int row = mrow0 + idx / 16, c = idx % 16;
@@ -1270,10 +1043,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         *reinterpret_cast<uint4*>(a.qw + ((static_cast<long long>(b) * a.R + gdiv(p)) * a.Hq + kvh * a.G +
                                           (p - gdiv(p) * a.G)) * kD + c * 8) = v;
       }
-      // 32 rows: one m-block, one cluster, so its last rank
-      bool write_k = rank == csize - 1 && mblock == 0;
-      if constexpr (kR == 64) write_k = *s_kvlast != 0;
-      if (write_k) {
+      if (rank == csize - 1) {  // one m-block: one cluster reads the head's raw key rows
 #pragma unroll 1
         for (int idx = st; idx < a.R * 16; idx += kSoftThreads) {
           const int i = idx / 16, c = idx % 16;
@@ -1281,7 +1051,6 @@ __global__ void __launch_bounds__(kThreads, 1)
           *reinterpret_cast<uint4*>(a.k_new + src) =
               *reinterpret_cast<const uint4*>(smem + C::kOffNewK + i * kNewRow + c * 16);
         }
-        if (kR == 64 && a.n_mblocks > 1 && st == 0) a.kv_ticket[b * a.Hkv + kvh] = 0;  // re-armed
       }
     }
     // ---- merge of the rows this CTA owns; slot c * rpc + rr came from rank c.
@@ -1320,33 +1089,16 @@ __global__ void __launch_bounds__(kThreads, 1)
         mloc = rref;
         nx = ny = nl = 0.f;
         const float* sn = s_new + r * a.R;
-        if constexpr (kR == 64) {
-          // unrolled: the shared-memory loads of several keys issue together
-          // (a rolled loop waits on each in turn, ~0.03 us a row and key: up
-          // to 64 rows x 17 keys of a K = 16 block on one CTA)
-#pragma unroll 4
-          for (int n = 0; n < n_new; ++n) mloc = fmaxf(mloc, sn[n]);
-          const float msub = mloc == -INFINITY ? 0.f : mloc;
-#pragma unroll 4
-          for (int n = 0; n < n_new; ++n) {
-            const float w = ex2(sn[n] - msub);
-            const uint32_t v2 = *reinterpret_cast<const uint32_t*>(smem + C::kOffNewV + n * kNewRow + d * 2);
-            nl += w;
-            nx = fmaf(w, sd_bf16_lo(v2), nx);
-            ny = fmaf(w, sd_bf16_hi(v2), ny);
-          }
-        } else {
 #pragma unroll 1
-          for (int n = 0; n < n_new; ++n) mloc = fmaxf(mloc, sn[n]);
-          const float msub = mloc == -INFINITY ? 0.f : mloc;
+        for (int n = 0; n < n_new; ++n) mloc = fmaxf(mloc, sn[n]);
+        const float msub = mloc == -INFINITY ? 0.f : mloc;
 #pragma unroll 1
-          for (int n = 0; n < n_new; ++n) {
-            const float w = ex2(sn[n] - msub);
-            const uint32_t v2 = *reinterpret_cast<const uint32_t*>(smem + C::kOffNewV + n * kNewRow + d * 2);
-            nl += w;
-            nx = fmaf(w, sd_bf16_lo(v2), nx);
-            ny = fmaf(w, sd_bf16_hi(v2), ny);
-          }
+        for (int n = 0; n < n_new; ++n) {
+          const float w = ex2(sn[n] - msub);
+          const uint32_t v2 = *reinterpret_cast<const uint32_t*>(smem + C::kOffNewV + n * kNewRow + d * 2);
+          nl += w;
+          nx = fmaf(w, sd_bf16_lo(v2), nx);
+          ny = fmaf(w, sd_bf16_hi(v2), ny);
         }
       }
       const float* part = recv + r * kRowF;  // rank c's partial at part + c * rpc * kRowF
@@ -1404,68 +1156,27 @@ __global__ void __launch_bounds__(kThreads, 1)
 }
 
 // ------------------------------------------------------------------ host
-typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*,
-                                  const cuuint64_t*, const cuuint64_t*, const cuuint32_t*,
-                                  const cuuint32_t*, CUtensorMapInterleave, CUtensorMapSwizzle,
-                                  CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
-
-EncodeTiledFn encode_fn() {
-  static EncodeTiledFn fn = nullptr;
-  static std::once_flag once;
-  std::call_once(once, [] {
-    void* p = nullptr;
-    cudaDriverEntryPointQueryResult qres;
-    if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &p, 12000, cudaEnableDefault,
-                                         &qres) == cudaSuccess &&
-        qres == cudaDriverEntryPointSuccess)
-      fn = reinterpret_cast<EncodeTiledFn>(p);
-  });
-  return fn;
-}
-
-bool make_map(CUtensorMap* map, void* base, int cap, int planes, int box_rows) {
-  EncodeTiledFn fn = encode_fn();
-  if (!fn) return false;
-  cuuint64_t dims[3] = {static_cast<cuuint64_t>(kD), static_cast<cuuint64_t>(cap),
-                        static_cast<cuuint64_t>(planes)};
-  cuuint64_t strides[2] = {static_cast<cuuint64_t>(kD) * 2,
-                           static_cast<cuuint64_t>(cap) * static_cast<cuuint64_t>(kD) * 2};
-  cuuint32_t box[3] = {64, static_cast<cuuint32_t>(box_rows), 1};
-  cuuint32_t estr[3] = {1, 1, 1};
-  return fn(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, base, dims, strides, box, estr,
-            CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
-            CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
-}
-
 constexpr int kNumClusterSizes = 6;
 constexpr int kClusterSizes[kNumClusterSizes] = {1, 2, 4, 6, 8, 16};
 
+// The row tiles: 32 and 64 packed rows of this file's kernel (the 64-row one
+// only with every key in the loop), 48, 64 and 80 of attention_wide.cu's.
+enum Tile { kTile32 = 0, kTile64All, kWide48, kWide64, kWide80, kNumTiles };
+
 // per device: how many clusters of each size fit at once, for each row tile
-// (index 0: 32 rows, 1: 64 rows)
 struct DevState {
   bool ready = false;
   bool ok = false;
-  int active[2][kNumClusterSizes] = {};
+  int active[kNumTiles][kNumClusterSizes] = {};
 };
 
-template <int kR>
-bool set_attributes(int* active) {
-  auto kern = verify_attn_tc_kernel<kR, 0>;
-  auto kern_f = verify_attn_tc_kernel<kR, 1>;
-  auto kern_n = verify_attn_tc_kernel<kR, 2>;
-  auto kern_p = verify_attn_tc_kernel<kR, 3>;
-  constexpr int smem = Cfg<kR>::kSmemBytes;
-  if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess ||
-      cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess ||
-      cudaFuncSetAttribute(kern_f, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess ||
-      cudaFuncSetAttribute(kern_f, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess ||
-      cudaFuncSetAttribute(kern_n, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess ||
-      cudaFuncSetAttribute(kern_n, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess ||
-      cudaFuncSetAttribute(kern_p, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess ||
-      cudaFuncSetAttribute(kern_p, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) {
-    (void)cudaGetLastError();
-    return false;
-  }
+bool set_attributes(const void* const* kerns, int n_kerns, int smem, int* active) {
+  for (int i = 0; i < n_kerns; ++i)
+    if (cudaFuncSetAttribute(kerns[i], cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess ||
+        cudaFuncSetAttribute(kerns[i], cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) {
+      (void)cudaGetLastError();
+      return false;
+    }
   for (int i = 0; i < kNumClusterSizes; ++i) {
     cudaLaunchConfig_t cfg = {};
     cudaLaunchAttribute attr[1];
@@ -1479,7 +1190,7 @@ bool set_attributes(int* active) {
     cfg.attrs = attr;
     cfg.numAttrs = 1;
     int n = 0;
-    if (cudaOccupancyMaxActiveClusters(&n, reinterpret_cast<const void*>(kern), &cfg) != cudaSuccess) {
+    if (cudaOccupancyMaxActiveClusters(&n, kerns[0], &cfg) != cudaSuccess) {
       (void)cudaGetLastError();
       n = 0;
     }
@@ -1498,7 +1209,16 @@ DevState* state() {
   DevState& s = st[dev];
   if (!s.ready) {
     s.ready = true;
-    s.ok = set_attributes<32>(s.active[0]) && set_attributes<64>(s.active[1]);
+    const void* k32[4] = {reinterpret_cast<const void*>(verify_attn_tc_kernel<32, 0>),
+                          reinterpret_cast<const void*>(verify_attn_tc_kernel<32, 1>),
+                          reinterpret_cast<const void*>(verify_attn_tc_kernel<32, 2>),
+                          reinterpret_cast<const void*>(verify_attn_tc_kernel<32, 3>)};
+    const void* k64[1] = {reinterpret_cast<const void*>(verify_attn_tc_kernel<64, 0>)};
+    s.ok = set_attributes(k32, 4, Cfg<32>::kSmemBytes, s.active[kTile32]) &&
+           set_attributes(k64, 1, Cfg<64>::kSmemBytes, s.active[kTile64All]) &&
+           sd_internal_wide_active(48, kClusterSizes, kNumClusterSizes, s.active[kWide48]) &&
+           sd_internal_wide_active(64, kClusterSizes, kNumClusterSizes, s.active[kWide64]) &&
+           sd_internal_wide_active(80, kClusterSizes, kNumClusterSizes, s.active[kWide80]);
   }
   return &s;
 }
@@ -1534,9 +1254,10 @@ static bool tc_enabled() {
   return on;
 }
 
-// How the tcgen05 path runs a shape: row tile (32 or 64 packed query rows),
-// m-blocks (row tiles per KV head) and cluster size; cs == 0: not served.
+// How the tcgen05 path runs a shape: row tile, its packed rows, m-blocks (row
+// tiles per KV head) and cluster size; cs == 0: not served.
 struct TcPlan {
+  Tile tile = kTile32;
   int rows = 0, mblocks = 0, cs = 0;
 };
 
@@ -1556,23 +1277,37 @@ extern "C" sd_status sd_set_cluster_size(int cluster_size) {
   return SD_ERR_INVALID_ARG;
 }
 
-// rows64: the 64-row tile even for G * R <= 32 (the block-masked fused layer:
-// the 32-row fused kernel is compiled causal only, and an N = 64 product
-// costs about what an N = 32 one does)
-static TcPlan tc_plan(int B, int R, int Hq, int Hkv, int D, int cap, int max_cs = 16, bool rows64 = false) {
+// The tile and cluster size of a shape whose new rows enter beside the prefix
+// loop (all_keys false: up to 16 new rows on the 32-row tile, 31 on the wide
+// ones) or with every key in the loop (all_keys). wide: a wide tile even for G * R
+// <= 32 (the block-masked fused layer: the 32-row fused kernel is causal only).
+static TcPlan tc_plan(int B, int R, int Hq, int Hkv, int D, int cap, bool all_keys, bool wide = false) {
   TcPlan p;
   if (!tc_enabled() || D != kD || Hkv <= 0 || Hq % Hkv || R <= 0) return p;
   const int M = (Hq / Hkv) * R;
   if (M > 2 * 64) return p;
+  int max_cs = 16;
+  if (all_keys) {
+    p.tile = M <= 32 ? kTile32 : kTile64All;
+    p.rows = M <= 32 ? 32 : 64;
+  } else if (M <= 32 && !wide) {
+    if (R > Cfg<32>::kMaxNew) return p;
+    // the 32-row tile's merge holds csize partials and R new keys in the lanes of one warp
+    max_cs = 32 - R;
+    p.tile = kTile32;
+    p.rows = 32;
+  } else {
+    if (R > 31) return p;
+    // the smallest tile that holds the rows in one m-block (every key read
+    // once), above 80 rows in two
+    p.tile = M <= 48 ? kWide48 : (M <= 64 ? kWide64 : (M <= 80 ? kWide80 : (M <= 96 ? kWide48 : kWide64)));
+    p.rows = p.tile == kWide48 ? 48 : (p.tile == kWide64 ? 64 : 80);
+  }
   DevState* s = state();
   if (!s || !s->ok) return p;
-  p.rows = M <= 32 && !rows64 ? 32 : 64;
   p.mblocks = (M + p.rows - 1) / p.rows;
-  const int* active = s->active[p.rows == 32 ? 0 : 1];
-  // sizes above max_cs are not used (the fused merge holds csize partials and
-  // R new keys in the lanes of one warp)
   int capped[kNumClusterSizes];
-  for (int i = 0; i < kNumClusterSizes; ++i) capped[i] = kClusterSizes[i] <= max_cs ? active[i] : 0;
+  for (int i = 0; i < kNumClusterSizes; ++i) capped[i] = kClusterSizes[i] <= max_cs ? s->active[p.tile][i] : 0;
   const int forced = g_forced_cluster.load();
   for (int i = 0; i < kNumClusterSizes && forced > 0; ++i)
     if (kClusterSizes[i] == forced && capped[i] > 0) p.cs = forced;
@@ -1581,13 +1316,11 @@ static TcPlan tc_plan(int B, int R, int Hq, int Hkv, int D, int cap, int max_cs 
 }
 
 bool sd_internal_tc_serves(int B, int R, int Hq, int Hkv, int D, int cap) {
-  return tc_plan(B, R, Hq, Hkv, D, cap).cs > 0;
+  return tc_plan(B, R, Hq, Hkv, D, cap, true).cs > 0;
 }
 
 bool sd_internal_tc_serves_layer(int B, int R, int Hq, int Hkv, int D, int cap, bool block) {
-  if (R > 32) return false;
-  const TcPlan plan = tc_plan(B, R, Hq, Hkv, D, cap, 32 - R, block);
-  return plan.cs > 0 && R <= (plan.rows == 32 ? Cfg<32>::kMaxNew : Cfg<64>::kMaxNew);
+  return tc_plan(B, R, Hq, Hkv, D, cap, false, block).cs > 0;
 }
 
 template <int kR, int kMode>
@@ -1618,32 +1351,28 @@ static sd_status launch_tc(const sd_kv_cache* cache, const TcArgs& a, const Rope
   return SD_OK;
 }
 
+// Modes 1 to 3 (the new rows beside the prefix loop) on the plan's tile.
 template <int kMode>
-static sd_status launch_plan(const sd_kv_cache* cache, const TcArgs& a, const RopeTable& tab,
-                             const TcPlan& plan, bool pdl, cudaStream_t stream) {
-  return plan.rows == 32 ? launch_tc<32, kMode>(cache, a, tab, plan, pdl, stream)
-                         : launch_tc<64, kMode>(cache, a, tab, plan, pdl, stream);
+static sd_status launch_new(const sd_kv_cache* cache, const TcArgs& a, const RopeTable& tab, const TcPlan& plan,
+                            cudaStream_t stream) {
+  if (plan.tile == kTile32) return launch_tc<32, kMode>(cache, a, tab, plan, true, stream);
+  return sd_internal_wide_launch(cache, a, tab, plan.rows, plan.cs, kMode, stream);
 }
 
 // Routed here by sd_verify_attention for head_dim 128 and G * R <= 128. Up to
-// kMaxNew new rows (and cluster sizes with csize + R <= 32) take the kernel
-// whose tensor-core loop covers the prefix only and whose new rows enter as
-// S_new (as in the fused layer), with the prefix optionally streamed before
-// the dependency wait (SD_ATTN_PREFIX_EARLY); other shapes take the kernel
-// whose loop covers every key (the flag is then a promise it does not need).
+// 16 (32-row tile) or 31 new rows take the kernels whose loop covers the prefix
+// only, with the prefix optionally streamed before the dependency wait
+// (SD_ATTN_PREFIX_EARLY); other shapes take the kernel whose loop covers every
+// key (the flag is then a promise it does not need).
 sd_status sd_internal_verify_attention_tc(const void* q, const sd_kv_cache* cache, void* out,
                                           int R, int Hq, float scale_log2, int flags, cudaStream_t stream,
                                           bool* handled) {
   *handled = false;
   const int B = cache->batch, Hkv = cache->n_kv_heads;
   const bool block = (flags & SD_ATTN_BLOCK_MASK) != 0, early = (flags & SD_ATTN_PREFIX_EARLY) != 0;
-  TcPlan plan;
-  int mode = 0;
-  if (R <= 32) {
-    plan = tc_plan(B, R, Hq, Hkv, cache->head_dim, cache->capacity, 32 - R);
-    if (plan.cs > 0 && R <= (plan.rows == 32 ? Cfg<32>::kMaxNew : Cfg<64>::kMaxNew)) mode = 2;
-  }
-  if (mode == 0) plan = tc_plan(B, R, Hq, Hkv, cache->head_dim, cache->capacity);
+  TcPlan plan = tc_plan(B, R, Hq, Hkv, cache->head_dim, cache->capacity, false);
+  const bool all_keys = plan.cs <= 0;
+  if (all_keys) plan = tc_plan(B, R, Hq, Hkv, cache->head_dim, cache->capacity, true);
   if (plan.cs <= 0) return SD_OK;
   TcArgs a = {};
   a.q = static_cast<const __nv_bfloat16*>(q);
@@ -1662,15 +1391,16 @@ sd_status sd_internal_verify_attention_tc(const void* q, const sd_kv_cache* cach
   a.scale_log2 = scale_log2;
   RopeTable tab = {};
   *handled = true;
-  if (mode == 2) {
+  if (!all_keys) {
     a.early = (early ? 1 : 0) | (block ? 2 : 0);
     // a programmatic dependent launch either way: without the flag the kernel
     // waits before its first global access, so only its launch and set-up
     // (barriers, tensor memory) overlap the kernel before it
-    return launch_plan<2>(cache, a, tab, plan, true, stream);
+    return launch_new<2>(cache, a, tab, plan, stream);
   }
   a.early = block ? 1 : 0;  // the all-keys kernel's block mask
-  return launch_plan<0>(cache, a, tab, plan, false, stream);
+  return plan.rows == 32 ? launch_tc<32, 0>(cache, a, tab, plan, false, stream)
+                         : launch_tc<64, 0>(cache, a, tab, plan, false, stream);
 }
 
 // The fused verify layer (rope + append + attention) on the tcgen05 path.
@@ -1680,13 +1410,9 @@ sd_status sd_internal_verify_layer_tc(void* q, void* k_new, const void* v_new, c
                                       int block, cudaStream_t stream, bool* handled) {
   *handled = false;
   const int B = cache->batch, Hkv = cache->n_kv_heads;
-  // the new rows are held in shared memory (16 with the 32-row tile, 32 with
-  // the 64-row tile) and merged in the lanes of one warp with the partials
-  if (R > 32) return SD_OK;
-  // block-masked layers take the 64-row tile (the 32-row fused kernel is causal only)
-  const TcPlan plan = tc_plan(B, R, Hq, Hkv, cache->head_dim, cache->capacity, 32 - R, block != 0);
+  // the new rows are held in shared memory (16 with the 32-row tile, 32 with the wide ones)
+  const TcPlan plan = tc_plan(B, R, Hq, Hkv, cache->head_dim, cache->capacity, false, block != 0);
   if (plan.cs <= 0) return SD_OK;
-  if (R > (plan.rows == 32 ? Cfg<32>::kMaxNew : Cfg<64>::kMaxNew)) return SD_OK;
   TcArgs a = {};
   a.q = static_cast<const __nv_bfloat16*>(q);
   a.out = static_cast<__nv_bfloat16*>(out);
@@ -1710,8 +1436,8 @@ sd_status sd_internal_verify_layer_tc(void* q, void* k_new, const void* v_new, c
   a.n_mblocks = plan.mblocks;
   a.scale_log2 = scale_log2;
   *handled = true;
-  if (early) return launch_plan<1>(cache, a, tab, plan, true, stream);
+  if (early) return launch_new<1>(cache, a, tab, plan, stream);
   // dependent as well: the wait comes before any global access (the draft's
   // single-row steps, each reading the length the step before advanced)
-  return launch_plan<3>(cache, a, tab, plan, true, stream);
+  return launch_new<3>(cache, a, tab, plan, stream);
 }

@@ -14,8 +14,7 @@
 
 namespace {
 // per-scene tickets [B], then per-(scene, KV head) tickets [B][Hkv] (the
-// tcgen05 kernel's read-before-write-back count when a head spans several
-// clusters)
+// wide tiles' read-before-write-back count when a head spans several clusters)
 constexpr size_t kTicketBytes(int B, int Hkv) {
   return (static_cast<size_t>(B) * (1 + static_cast<size_t>(Hkv)) * 4 + 255) / 256 * 256;
 }

@@ -1,0 +1,84 @@
+"""The wide row tiles (48, 64 and 80 packed query rows per KV head, two m-blocks
+above 80) against the float64 oracle: every edge of the tile choice, prefixes
+around the 32-key split and the 128-key tile, causal and block masks, the fused
+layer and the attention; and the second pass of a CTA whose row sums leave the
+range of weights taken without a reference (2^-80 .. 2^64)."""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+from paper_2606_31160_gb300 import sd, workloads
+from tests.helpers import attn_within, ensure_lib, to64
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _lib():
+    ensure_lib()
+
+
+def _run(q, k, v, k_new, v_new, prefix, fused, block):
+    """Position-0 new rows (an identity rotation) through the layer or the attention."""
+    B, R, Hq, D = q.shape
+    bf = workloads.to_bf16
+    kc, vc = np.full_like(k, np.nan), np.full_like(v, np.nan)  # stale rows hold NaN
+    for b, n in enumerate(prefix):
+        kc[b, :, :n], vc[b, :, :n] = k[b, :, :n], v[b, :, :n]
+        if not fused:
+            kc[b, :, n:n + R] = k_new[b].transpose(1, 0, 2)
+            vc[b, :, n:n + R] = v_new[b].transpose(1, 0, 2)
+    lens = torch.tensor([n + (0 if fused else R) for n in prefix], dtype=torch.int32).cuda()
+    cache = sd.KVCache(bf(kc).cuda(), bf(vc).cuda(), lens)
+    qd = bf(q).cuda()
+    if fused:
+        pos = torch.zeros((B, R, 3), dtype=torch.int32).cuda()
+        out = sd.verify_layer(qd, bf(k_new).cuda(), bf(v_new).cuda(), pos, (16, 24, 24), cache, 0, 1e6, block=block)
+    else:
+        out = sd.verify_attention(qd, cache, block=block)
+    torch.cuda.synchronize()
+    assert sd.get_device_error() == 0
+    ref = oracle.verify_attention(to64(qd), to64(cache.k), to64(cache.v), cache.len.cpu().numpy(), block=block)
+    assert np.isfinite(to64(out)).all() and attn_within(to64(out), ref), np.abs(to64(out) - ref).max()
+
+
+# (G, R): 33, 48 | 49, 64 | 65, 68, 80 | 81, 96 | 98, 128 packed rows, up to 31 new rows
+@pytest.mark.parametrize("G,R", [(11, 3), (4, 12), (7, 7), (4, 16), (5, 13), (4, 17), (16, 5), (27, 3), (6, 16), (7, 14),
+                                 (4, 31), (8, 16)])
+@pytest.mark.parametrize("fused,block", [(True, False), (True, True), (False, False)])
+def test_tile_edges(G, R, fused, block):
+    prefix = [0, 1, 31, 127, 128, 129, 700]
+    B, Hkv, D, cap = len(prefix), 2, 128, 760
+    rng = np.random.default_rng(100 * G + R)
+    draw = lambda *s: rng.standard_normal(s).astype(np.float32)  # noqa: E731
+    _run(draw(B, R, Hkv * G, D), draw(B, Hkv, cap, D), draw(B, Hkv, cap, D), draw(B, R, Hkv, D), draw(B, R, Hkv, D),
+         prefix, fused, block)
+
+
+# the score (log2) around which a third of the keys, or all, lie: far outside the
+# range on either side, and just inside it
+@pytest.mark.parametrize("G,R", [(6, 8), (8, 8), (4, 17)])
+@pytest.mark.parametrize("level", [-150.0, 100.0, -70.0, 55.0])
+@pytest.mark.parametrize("part", [1, 3])
+@pytest.mark.parametrize("cluster", [0, 1, 4])
+def test_row_sums_out_of_range(G, R, level, part, cluster):
+    prefix = [1500, 40]
+    B, Hkv, D, cap = len(prefix), 1, 128, 1540
+    rng = np.random.default_rng(int(1000 + level + 10 * G + R))
+    draw = lambda *s: rng.standard_normal(s).astype(np.float32)  # noqa: E731
+    u = np.zeros(D, dtype=np.float32)
+    u[5] = 1.0
+    q = draw(B, R, Hkv * G, D)
+    q[..., 5] = 8.0
+    k, k_new = draw(B, Hkv, cap, D), draw(B, R, Hkv, D)
+    beta = level / (8.0 * 1.4426950408889634 / np.sqrt(D))
+    k[:, :, :, 5] = 0.0
+    k[:, :, : cap // part, 5] += beta
+    k_new[..., 5] = beta if part == 1 else 0.0
+    sd.set_cluster_size(cluster)
+    try:
+        _run(q, k, draw(B, Hkv, cap, D), k_new, draw(B, R, Hkv, D), prefix, True, False)
+        _run(q, k, draw(B, Hkv, cap, D), k_new, draw(B, R, Hkv, D), prefix, False, False)
+    finally:
+        sd.set_cluster_size(0)
