@@ -194,3 +194,38 @@ def test_sample_output_law_by_enumeration_on_gpu(V):
     p /= p.sum()
     dist = sum(q[x] * np.bincount(first[x], minlength=V) / n for x in range(V))
     np.testing.assert_allclose(dist, p, atol=2.0 / N + 1e-6)
+
+
+@pytest.mark.parametrize("dtype", [torch.bfloat16, torch.float32])
+@pytest.mark.parametrize("B,R,V", [(1, 1, 1), (2, 3, 7), (3, 2, 8), (1, 9, 255), (2, 2, 4096), (1, 2, 8191), (2, 1, 8192),
+                                   (1, 3, 8193), (2, 2, 32768), (33, 8, 16385), (1, 128, 1000), (300, 2, 130)])
+@pytest.mark.parametrize("shift", [0, 1])
+def test_greedy_scan_edges(dtype, B, R, V, shift):
+    # few distinct values, so every row has many equal maxima in different
+    # vectors, steps and segments; rows of -inf, of the lowest finite value and of
+    # signed zeros; bases and rows off the 16-byte boundary. Whole numbers: exact.
+    g = torch.Generator().manual_seed(B * 1000 + V)
+    z = torch.randint(-3, 4, (B, R, V), generator=g).float()
+    z[-1, -1] = torch.where(torch.arange(V) % 3 == 1, 0.0, -0.0)
+    z[0, 0] = -float("inf")
+    if B > 1:
+        z[0, 0, V // 2:] = float(torch.finfo(dtype).min)
+    flat = torch.zeros(z.numel() + shift, dtype=dtype, device="cuda")
+    flat[shift:] = z.flatten().to(dtype)
+    logits = flat[shift:].view(B, R, V)
+    star = np.argmax(logits.float().cpu().numpy(), axis=-1)
+    draft = torch.from_numpy(star[:, : R - 1].astype(np.int32)).cuda().contiguous()
+    if R > 2 and V > 1:
+        draft[0, 1] = (draft[0, 1] + 1) % V
+    ws = sd.workspace(sd.greedy_workspace_bytes(B, R - 1, V))
+    for _ in range(2):  # the workspace is left zeroed
+        n_emit, tokens, argmax = sd.accept_greedy(logits, draft, ws=ws)
+        assert np.array_equal(argmax.cpu().numpy(), star)
+        ell = np.full(B, R - 1)
+        if R > 2 and V > 1:
+            ell[0] = 1
+        assert np.array_equal(n_emit.cpu().numpy(), ell + 1)
+        want = np.where(np.arange(R)[None] <= ell[:, None], star, -1)
+        assert np.array_equal(tokens.cpu().numpy(), want)
+        assert int(ws.count_nonzero()) == 0
+    assert sd.get_device_error() == 0
