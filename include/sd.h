@@ -188,8 +188,8 @@ sd_status sd_verify_attention(const void* q, const sd_kv_cache* cache, void* out
  * SD_ATTN_PREFIX_EARLY declares that the kernel issued just before this call
  * on the stream writes neither this cache (its K / V rows, the new rows
  * included) nor its len (true when a step's layers are issued back to back
- * after their appends). For head_dim 128 and up to 16 new rows (32 when
- * G * R > 32) the call is then a programmatic dependent launch that reads len
+ * after their appends). For head_dim 128 and up to 31 new rows
+ * the call is then a programmatic dependent launch that reads len
  * and streams the whole cache while its predecessor still runs, and reads q
  * only after the predecessor has completed; other shapes ignore the flag.
  * Without the flag those shapes are programmatic dependent launches too, but
@@ -291,9 +291,7 @@ size_t sd_verify_layer_workspace(int B, int R, int Hq, int Hkv, int D, int capac
  *   SD_LAYER_BLOCK_MASK: the attention uses the block mask (as
  *   SD_ATTN_BLOCK_MASK of sd_verify_attention_ex).
  * For head_dim 128 this is one kernel: the tcgen05 kernel for G * R <= 128
- * and R <= 31 (R <= 16 when a causal layer has G * R <= 32: its 32-row tile
- * holds 16 new rows and is causal only, so block-masked layers always take the
- * wider tiles);
+ * and R <= 31;
  * other shapes run the three kernels in sequence (sd_verify_kernel names the
  * choice). A scene whose append would pass the
  * capacity sets SD_DEVERR_KV_OVERFLOW and is left untouched.

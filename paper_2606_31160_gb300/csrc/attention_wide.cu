@@ -1,35 +1,44 @@
-// K3 / the fused verify layer for more than 32 packed query rows per KV head
-// (Eq. verify, Sec. 3.2; drafts of K = 8 and the K = 16 blocks of Sec. 5), head
-// dim 128, up to 31 new rows, on the 5th-generation tensor cores.
+// The verify attention and the fused verify layer (Eq. verify, Sec. 3.2; the
+// rotations of Sec. 3.3 / 4.2, the append of Eq. commit) for head dim 128 and up to
+// 31 new rows, on the 5th-generation tensor cores (tcgen05 + TMEM).
 //
-// As in attention_tc.cu both products run transposed, the 128-wide dimension
-// on the MMA's M side:
+// The packed query rows of a KV head (G * R) are few, so both products run
+// transposed, the 128-wide dimension on the MMA's M side:
 //     S^T[128 keys][kR rows] = K_tile . Q^T,   O^T[128 d][kR rows] += V_tile^T . P^T
-// with kR = 48, 64 or 80 packed rows, the smallest that holds the rows of a KV
-// head (two m-blocks of 48 or 64 above 80): a K = 16 block of the 8B target
-// (68 rows) is one tile and reads every key once.
+// with kR = 32, 48, 64 or 80, the smallest that holds the rows in one tile (two
+// m-blocks of 48 or 64 above 80): a K = 16 block of the 8B target (68 rows) reads
+// every key once. One cluster per (scene, KV head, m-block); its CTAs take
+// contiguous ranges of the prefix and merge their partials through distributed
+// shared memory.
 //
-// The new rows are one more tile: the cluster's last rank holds the R (rotated)
-// new keys and values in shared memory in the operands' own layout, so their
-// scores and values are products like every other tile's (32 keys, the causal
-// limit per row). Scored on the CUDA cores instead, rows x new keys on the
-// rows a CTA merges, they took 26 us a launch at one CTA a head and K = 16.
+// What bounds it. With many scenes the stream of K and V (32 scenes, L = 8192: K = 7
+// 153 -> 142 us, K = 8 165 -> 146, 1.0 of the measured copy). With one scene the
+// dependent path behind the previous kernel: rows, rotation, S(0), the tiles at
+// ~0.4 us of products each, the exchange (~0.7 us), the merge (target layer
+// 6.77 -> 6.27 us, K = 8 10.0 -> 7.8, K = 16 block 15.9 -> 11.4, draft step 6.8 -> 6.1
+// on one cache).
 //
-// Fixed reference. Weights are 2^(score * scale) with no reference subtracted:
-// a floating-point weight keeps its relative precision at any size, so only
-// overflow and underflow would matter. A row sum above 2^kHigh or, over a
-// warp's keys, below 2^kLow (log2) sends the CTA through its range again with
-// each row's exact maximum as its reference: one pass for the maxima, one for
-// the weights. No reduction and no reference product stands between S and P.
+// The new rows stay out of the loop: the cluster's last rank holds the R (rotated)
+// new keys and values in shared memory, scores them by mma.sync, 8 rows by 16 keys a
+// warp, and adds one PV product of 16 or 32 keys. Scored on the CUDA cores by the
+// rows a CTA merges instead, rows x new keys took 26 us a launch at one CTA a head
+// and K = 16.
 //
-// Warps (608 threads): 0 the TMA producer, 1 issues S and owns tensor memory, 2
-// issues PV, 3..18 two softmax groups of eight. Group g takes tiles T with
-// T % 2 == g and P buffer g, so a group has two tiles' time for its tile's
-// dependent chain (barrier wake-up, tensor-memory load, exponentials, stores)
-// while the other group's tile is in the products. With one group of eight on
-// every tile that chain set the pace: ~1.1 us a 128-key tile of 64 rows against
-// ~0.45 us of products. Products of pairs (fma / add f32x2) and a select on the
-// packed weights take 4 issue slots a weight instead of ~9.5.
+// Fixed reference. Weights are 2^(score * scale) with no reference subtracted: a
+// floating-point weight keeps its relative precision at any size, so only overflow
+// and underflow matter. A row sum above 2^64, or no lane of a warp with every sum
+// above 2^-80, sends the CTA through its range again with each row's exact maximum
+// as its reference: one pass for the maxima, one for the weights. No reduction and
+// no reference product stands between S and P.
+//
+// Warps (608 threads): 0 the TMA producer, whose first tiles go out before the CTA's
+// set-up is over; 1 issues S and owns tensor memory; 2 issues PV; 3..18 two softmax
+// groups of eight. Group g takes tiles T with T % 2 == g and P buffer g, so a group
+// has two tiles' time for its tile's dependent chain (barrier wake-up,
+// tensor-memory load, exponentials, stores: ~800 cycles on 32 rows) while the other
+// group's tile is in the products. With one group of eight on every tile that chain
+// set the pace: ~1.1 us a 128-key tile of 64 rows. fma on pairs (f32x2) and a select
+// on the packed weights take about 5 issue slots a weight instead of ~9.5.
 #include "tc_common.cuh"
 
 #include <math.h>
@@ -48,12 +57,10 @@ constexpr int kSoftThreads = 32 * kSoftWarps;
 constexpr int kFirstSoft = 3;            // the first softmax warp
 constexpr int kSoft0 = 32 * kFirstSoft;  // the first softmax thread
 constexpr int kThreads = kSoft0 + kSoftThreads;
-constexpr int kMaxNew = 32;              // new rows held in shared memory
-constexpr int kNewHalf = kMaxNew * 128;  // one 64-column half of the new key (value) rows
 constexpr float kHigh = 18446744073709551616.f;          // 2^64: a larger row sum runs the range again
 constexpr float kLow = 8.271806125530277e-25f;           // 2^-80: a smaller one too
-// a partial row sent to its owner: [O(128) | l by softmax group and lane
-// quarter (8) | reference | 3 pad] fp32 (560 bytes)
+// a partial row sent to its owner: [O(128) | prefix row sums by softmax group and
+// lane quarter (8) | reference | new keys' row sum | 2 pad] fp32 (560 bytes)
 constexpr int kRowL = kD;
 constexpr int kRowM = kD + 8;
 constexpr int kRowF = kD + 12;
@@ -61,9 +68,11 @@ constexpr int kRowBytes = kRowF * 4;
 
 template <int kR>
 struct Cfg {
-  static_assert(kR == 48 || kR == 64 || kR == 80, "row tile");
-  static constexpr int kRpt = kR / 2;   // rows of a softmax thread in its tile
-  static constexpr int kStages = 2;     // K slots, and V slots
+  static_assert(kR == 32 || kR == 48 || kR == 64 || kR == 80, "row tile");
+  static constexpr int kRpt = kR / 2;                   // rows of a softmax thread in its tile
+  static constexpr int kStages = kR == 32 ? 3 : 2;      // K slots, and V slots
+  static constexpr int kMaxNew = kR == 32 ? 16 : 32;    // new rows held in shared memory
+  static constexpr int kNewHalf = kMaxNew * 128;        // one 64-column half of the new key (value) rows
   static constexpr int kRingV = kStages * kKV;
   static constexpr int kRing = 2 * kStages * kKV;
   static constexpr int kQHalf = kR * 128;
@@ -71,26 +80,28 @@ struct Cfg {
   // 16-row groups kPGroup apart
   static constexpr int kPGroup = kStageKeys * 32;
   static constexpr int kP = (kR / 16) * kPGroup;
-  static constexpr int kSStride = kR == 48 ? 64 : (kR == 64 ? 64 : 128);  // columns between S0 | S1 | S2 | O
+  static constexpr int kSStride = kR == 32 ? 32 : (kR <= 64 ? 64 : 128);  // columns between S0 | S1 | S2 | O
   static constexpr int kTmemCols = 4 * kSStride;
-  // shared memory (offsets from the 1024-aligned base). The new-key tile's S
-  // product reads 128 rows from each half of kOffNewK: rows past kMaxNew are
-  // the regions behind it, their scores are never used.
+  // shared memory (offsets from the 1024-aligned base)
   static constexpr int kOffNewK = kRing;
   static constexpr int kOffNewV = kOffNewK + 2 * kNewHalf;
   static constexpr int kOffQ = kOffNewV + 2 * kNewHalf;
   static constexpr int kOffP = kOffQ + 2 * kQHalf;
-  static constexpr int kOffBar = kOffP + 2 * kP;
-  // full_k[2] full_v[2] p_full[2] s_ready[3] s_free[3] pv_done[2] q_full recv decide tmem_done
-  static constexpr int kNumBars = 3 * kStages + 12;
+  // the new keys' weights: on the 32-row tile, which has no room for more, in P
+  // buffer 1 ahead of its first tile; on the others beside it, in the same layout
+  static constexpr bool kNewFirst = kR == 32;
+  static constexpr int kOffPNew = kNewFirst ? kOffP + kP : kOffP + 2 * kP;
+  static constexpr int kPNewGroup = kNewFirst ? kPGroup : kMaxNew * 32;
+  static constexpr int kOffBar = kNewFirst ? kOffP + 2 * kP : kOffPNew + (kR / 16) * kPNewGroup;
+  // full_k[S] full_v[S] p_full[2] s_ready[3] s_free[3] pv_done[S] p_new new_done recv decide maxima tmem_done
+  static constexpr int kNumBars = 3 * kStages + 14;
   static constexpr int kOffMisc = round_up(kOffBar + kNumBars * 8, 16);
-  static constexpr int kOffRef = kOffMisc + 32;       // [kR] negated references
-  static constexpr int kOffLim = kOffRef + kR * 4;    // [kR] last new key a row sees
-  static constexpr int kOffSum = kOffLim + kR * 4;    // [kR][8] row sums by group and lane quarter
+  static constexpr int kOffRef = kOffMisc + 16;        // [kR] negated references
+  static constexpr int kOffNewSum = kOffRef + kR * 4;  // [kR] row sums of the new keys
+  static constexpr int kOffSum = kOffNewSum + kR * 4;  // [kR][8] row sums by group and lane quarter
   static constexpr int kSmemBytes = kOffSum + kR * 32 + 1024;
   static_assert(kSmemBytes <= 227 * 1024, "shared memory budget");
   static_assert(kOffNewV % 1024 == 0 && kOffQ % 1024 == 0 && kOffP % 1024 == 0 && kQHalf % 1024 == 0, "swizzle atoms");
-  static_assert(kOffNewK + kNewHalf + kHalf <= kOffBar, "the new-key tile's product stays inside");
   static_assert(kMaxNew * 64 * 8 <= 2 * kP, "rotation table fits the P buffers");
   static_assert(kR * 128 * 4 <= 2 * kP, "row maxima fit the P buffers");
   // cluster merge: incoming rows in the K ring (free after the last S), this
@@ -137,11 +148,11 @@ __device__ __forceinline__ uint64_t add2(uint64_t a, uint64_t b) {
   return d;
 }
 
-// Weights of kN rows of one key: P = 2^(S * scale - ref) in bf16, the row sums
-// advanced by the same rounded weights, stored to the key's P^T chunks. keep
-// masks each packed pair (0 drops a weight whatever its score, NaN included).
-template <int kN, typename Keep>
-__device__ __forceinline__ void weights_to_p(const uint32_t (&r)[kN], const float* nref, uint64_t sl2, Keep keep,
+// Weights of kN rows of one key: P = 2^(S * scale - ref) in bf16 (0 for a key out
+// of the range, whatever its score, NaN included), the row sums advanced by the
+// same rounded weights.
+template <int kN>
+__device__ __forceinline__ void weights_to_p(const uint32_t (&r)[kN], const float* nref, uint64_t sl2, bool key_ok,
                                              uint64_t* lp2, uint32_t (&pw)[kN / 2]) {
 #pragma unroll
   for (int j = 0; j < kN; j += 4) {
@@ -150,7 +161,7 @@ __device__ __forceinline__ void weights_to_p(const uint32_t (&r)[kN], const floa
     for (int e = 0; e < 2; ++e) {
       float y0, y1;
       unpack2(fma2(pack2(r[j + 2 * e], r[j + 2 * e + 1]), sl2, e == 0 ? pack2f(nr.x, nr.y) : pack2f(nr.z, nr.w)), y0, y1);
-      const uint32_t w = keep(j + 2 * e, cvt_bf16x2(ex2(y0), ex2(y1)));
+      const uint32_t w = key_ok ? cvt_bf16x2(ex2(y0), ex2(y1)) : 0u;
       pw[j / 2 + e] = w;
       lp2[j / 2 + e] = add2(lp2[j / 2 + e], pack2(w << 16, w & 0xffff0000u));
     }
@@ -179,25 +190,59 @@ __device__ __forceinline__ float warp_sum8(const float (&v0)[8], int lane) {
   return x;
 }
 
+// C += A . B of one m16n8k16 bf16 product
+__device__ __forceinline__ void mma_bf16(float (&c)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1) {
+  asm("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
+      : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
+      : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
+}
+__device__ __forceinline__ void ldmatrix4(uint32_t addr, uint32_t (&r)[4]) {
+  asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+               : "r"(addr)
+               : "memory");
+}
+// Byte offset of 16-byte chunk c of row r in a 128-byte-swizzled pair of
+// 64-column halves, `half` bytes each.
+__device__ __forceinline__ uint32_t swz(int r, int c, int half) {
+  return (c >> 3) * half + r * 128 + (((c & 7) ^ (r & 7)) << 4);
+}
+
+// A row's largest score against the new keys it sees (the range is run again:
+// out of line). One warp; qrow / krow0: the packed query row and new key row 0.
+__device__ __noinline__ float new_key_max(const uint8_t* q, int row, int q_half, const uint8_t* k, int k_half, int last,
+                                          float sl, int lane) {
+  const int c = lane >> 1, e = (lane & 1) * 8;  // 4 d a lane
+  const uint2 qw = *reinterpret_cast<const uint2*>(q + swz(row, c, q_half) + e);
+  float m = -INFINITY;
+  for (int n = 0; n <= last; ++n) {
+    const uint2 kw = *reinterpret_cast<const uint2*>(k + swz(n, c, k_half) + e);
+    float x = sd_bf16_lo(qw.x) * sd_bf16_lo(kw.x);
+    x = fmaf(sd_bf16_hi(qw.x), sd_bf16_hi(kw.x), x);
+    x = fmaf(sd_bf16_lo(qw.y), sd_bf16_lo(kw.y), x);
+    x = fmaf(sd_bf16_hi(qw.y), sd_bf16_hi(kw.y), x);
+    for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
+    m = fmaxf(m, x * sl);
+  }
+  return m;
+}
+
 // ------------------------------------------------------------------ kernel
-// kMode 1: the verify layer (M-RoPE, append, attention) whose prefix, len and
-// pos are read before the dependency wait; 3: the same, everything after the
-// wait; 2: the attention over a cache that already holds the R new rows
-// (prefix before the wait when bit 0 of a.early is set). Bit 1 of a.early: the
-// block mask. Grid: (cluster size, Hkv * n_mblocks, B); m-block mb takes packed
-// rows mb * kR .. mb * kR + kR - 1.
-template <int kR, int kMode>
+// kFused: the verify layer (M-RoPE, append, attention); otherwise the attention
+// over a cache that already holds the R new rows. Bit 0 of a.early: prefix, len
+// and pos may be read before the dependency wait; bit 1: the block mask. Grid:
+// (cluster size, Hkv * n_mblocks, B); m-block mb takes packed rows mb * kR ..
+// mb * kR + kR - 1.
+template <int kR, bool kFused>
 __global__ void __launch_bounds__(kThreads, 1)
     verify_wide_kernel(const __grid_constant__ CUtensorMap tm_k128, const __grid_constant__ CUtensorMap tm_v128,
                        const TcArgs a, const RopeTable tab) {
   using C = Cfg<kR>;
-  constexpr bool kFused = kMode != 2;
-  constexpr bool rows_first = kMode == 3;
   constexpr int kS = C::kStages;
   constexpr int kRpt = C::kRpt;
   constexpr uint32_t kIdescS = umma_idesc(128, kR, 0, 0);
   constexpr uint32_t kIdescO = umma_idesc(128, kR, 1, 1);
-  const bool early = kMode == 1 || (kMode == 2 && (a.early & 1) != 0);
+  const bool early = (a.early & 1) != 0;
   const bool block = (a.early & 2) != 0;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) &
@@ -205,22 +250,25 @@ __global__ void __launch_bounds__(kThreads, 1)
   const uint32_t base = smem_addr(smem);
   const uint32_t qs = base + C::kOffQ;
   auto bar = [&](int i) { return base + C::kOffBar + 8u * i; };
-  // T counts the tiles of all passes (the new-key tile included), TL those the
-  // producer loads. A barrier's next phase never completes before its waiters
-  // have seen the current one: S(T + 3) and P(T + 2) follow the softmax's waits
-  // for S(T) and PV(T), and a K (V) slot's next tile the producer's wait for
-  // its S (PV). A waiter that skips phases of a slot (a group sees every second
-  // tile) knows the skipped ones complete: products complete in order.
+  // T counts the prefix tiles of all passes. A wait names a phase by its parity,
+  // so a waiter has to know that the phase before has completed, and the next one
+  // must not complete before it has looked: S(T + 3) and P(T + 2) follow the
+  // softmax's waits for S(T) and PV(T), a K (V) slot's next tile the producer's
+  // wait for its S (PV); a group that skips phases of a ring (it sees every second
+  // tile) knows the skipped ones complete, as products complete in order; and
+  // between passes everything is complete.
   auto FULLK = [&](int s) { return bar(s); };
   auto FULLV = [&](int s) { return bar(kS + s); };
   auto PFULL = [&](int T) { return bar(2 * kS + (T & 1)); };
-  auto SREADY = [&](int T) { return bar(2 * kS + 2 + T % 3); };
-  auto SFREE = [&](int T) { return bar(2 * kS + 5 + T % 3); };
-  auto PVDONE = [&](int T) { return bar(2 * kS + 8 + T % kS); };
-  const uint32_t QFULL = bar(3 * kS + 8);
-  const uint32_t RECV = bar(3 * kS + 9);
-  const uint32_t DECIDE = bar(3 * kS + 10);  // phase 0: whether the range runs again; phase 1: the maxima are in
-  const uint32_t TMEMDONE = bar(3 * kS + 11);
+  auto SREADY = [&](int i) { return bar(2 * kS + 2 + i); };  // i = T % 3
+  auto SFREE = [&](int i) { return bar(2 * kS + 5 + i); };
+  auto PVDONE = [&](int i) { return bar(2 * kS + 8 + i); };  // i = T % kS
+  const uint32_t PNEW = bar(3 * kS + 8);      // the new keys' weights are stored
+  const uint32_t NEWDONE = bar(3 * kS + 9);   // their product is done
+  const uint32_t RECV = bar(3 * kS + 10);
+  const uint32_t DECIDE = bar(3 * kS + 11);   // whether the range runs again
+  const uint32_t MAXIMA = bar(3 * kS + 12);   // pass 1 is over
+  const uint32_t TMEMDONE = bar(3 * kS + 13);
   auto par3 = [](int T) { return static_cast<uint32_t>((T / 3) & 1); };
   auto parS = [](int T) { return static_cast<uint32_t>((T / kS) & 1); };
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(smem + C::kOffMisc);
@@ -228,7 +276,7 @@ __global__ void __launch_bounds__(kThreads, 1)
   int* s_len = reinterpret_cast<int*>(smem + C::kOffMisc + 8);
   int* s_kvlast = reinterpret_cast<int*>(smem + C::kOffMisc + 12);
   float* row_nref = reinterpret_cast<float*>(smem + C::kOffRef);
-  int* row_lim = reinterpret_cast<int*>(smem + C::kOffLim);
+  float* row_new = reinterpret_cast<float*>(smem + C::kOffNewSum);
   float* row_sum = reinterpret_cast<float*>(smem + C::kOffSum);
 
   auto gdiv = [&](int p) { return __float2int_rz((static_cast<float>(p) + 0.5f) * a.inv_g); };
@@ -239,118 +287,83 @@ __global__ void __launch_bounds__(kThreads, 1)
   const int b = blockIdx.z;
   const int warp = threadIdx.x >> 5;
   const int lane = threadIdx.x & 31;
+  // the launch's arguments come into the constant cache here, ahead of the wait
+  // (a first touch behind it costs a round trip to L2 on the critical path)
+  const float sl = a.scale_log2;
+  asm volatile("" ::"f"(sl), "l"(a.out), "l"(a.ticket), "r"(a.cap), "r"(a.M));
+  const bool last_rank = rank == csize - 1;
+  // the cluster launched last starts when the previous kernel is nearly done
+  const bool last_cluster = blockIdx.y == gridDim.y - 1 && blockIdx.z == gridDim.z - 1;
 
-  if (threadIdx.x == 0) {
-    for (int s = 0; s < kS; ++s) {
-      mbar_init(FULLK(s), 1);
-      mbar_init(FULLV(s), 1);
-      mbar_init(PVDONE(s), 1);
-    }
-    for (int i = 0; i < 2; ++i) mbar_init(PFULL(i), kSoftWarps / 2);
-    for (int i = 0; i < 3; ++i) {
-      mbar_init(SREADY(i), 1);
-      mbar_init(SFREE(i), kSoftWarps / 2);
-    }
-    mbar_init(QFULL, 1);
-    mbar_init(RECV, 1);
-    mbar_init(DECIDE, 1);
-    mbar_init(TMEMDONE, kSoftWarps);
-    *s_redo = 0;
-    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-  }
-  if (warp == 1) {
-    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_addr(tmem_slot)),
-                 "r"(C::kTmemCols)
-                 : "memory");
-    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
-  }
+  // this CTA's share of a scene with len0 cached rows: the prefix in 32-key
+  // blocks, split over the cluster's ranks
+  int L_pre, key_begin, key_end, n_pre;
+  bool valid;
+  auto ranges = [&](int len0) {
+    L_pre = kFused ? len0 : len0 - a.R;
+    valid = L_pre >= 0 && L_pre + a.R <= a.cap;
+    const int nblk = valid ? (L_pre + 31) / 32 : 0;
+    const int blk_begin = static_cast<int>((static_cast<uint32_t>(rank) * nblk) / static_cast<uint32_t>(csize));
+    const int blk_end = static_cast<int>((static_cast<uint32_t>(rank + 1) * nblk) / static_cast<uint32_t>(csize));
+    key_begin = blk_begin * 32;
+    key_end = min(blk_end * 32, valid ? L_pre : 0);
+    n_pre = (blk_end - blk_begin + 3) / 4;  // prefix tiles
+  };
+  // keys of tile t that its PV product reads: whole 16-key steps up to the last key
+  auto pv_keys = [&](int t) { return min(kStageKeys, (key_end - key_begin - t * kStageKeys + 15) & ~15); };
+
   // a launch without the early prefix waits here, before any global access
   if (!early) griddep_wait();
-  if (threadIdx.x == 0) *s_len = a.len[b];  // the scene's length advances at the producer's end
-  const bool last_rank = rank == csize - 1;
-  // this thread's 16-byte chunks: of the packed query tile (row idx >> 4, chunk
-  // idx & 15, rows past M zero) and, in the cluster's last rank, of the new key
-  // and value rows
-  constexpr int kQc = (kR * 16 + kSoftThreads - 1) / kSoftThreads;
-  const int st = static_cast<int>(threadIdx.x) - kSoft0;  // softmax threads: 0 .. 511
-  auto q_off = [&](int p) {
-    const int i = gdiv(p);
-    return ((static_cast<long long>(b) * a.R + i) * a.Hq + kvh * a.G + (p - i * a.G)) * kD;
-  };
-  const bool raw_kv = last_rank && st < a.R * 16;
-  const long long kv_row = ((static_cast<long long>(b) * a.R + (st >> 4)) * a.Hkv + kvh) * kD + (st & 15) * 8;
-  uint4 pre_q[kQc], pre_k = make_uint4(0, 0, 0, 0), pre_v = make_uint4(0, 0, 0, 0);
-  if (kFused && warp >= kFirstSoft) {
-    if (rows_first) {
-      // one global round trip before the tiles: the rows with the positions
-#pragma unroll
-      for (int u = 0; u < kQc; ++u) {
-        const int idx = st + u * kSoftThreads, p = mblock * kR + (idx >> 4);
-        pre_q[u] = idx < kR * 16 && p < a.M
-                       ? __ldcg(reinterpret_cast<const uint4*>(a.qw + q_off(p) + (idx & 15) * 8))
-                       : make_uint4(0, 0, 0, 0);
-      }
-      if (raw_kv) {
-        pre_k = __ldcg(reinterpret_cast<const uint4*>(a.k_new + kv_row));
-        pre_v = __ldcg(reinterpret_cast<const uint4*>(a.v_new + kv_row));
-      }
-    }
-    // rotation table of the R new positions: (cos, sin) per (row, pair)
-    float2* tabw = reinterpret_cast<float2*>(smem + C::kOffP);
-#pragma unroll 1
-    for (int idx = st; idx < a.R * 64; idx += kSoftThreads) {
-      const int i = idx >> 6, d = idx & 63;
-      const int32_t pc = a.pos[(static_cast<long long>(b) * a.R + i) * 3 + tab.axis[d]];
-      tabw[idx] = sd_rope_cs(static_cast<float>(pc), d, tab);
-    }
-  }
-  tc_fence_before();
-  __syncthreads();
-  tc_fence_after();
-  const uint32_t tmem = *tmem_slot;
-  const uint32_t tmem_o = tmem + 3 * C::kSStride;
-
-  const int len0 = *s_len;
-  const int L_pre = kFused ? len0 : len0 - a.R;
-  const bool valid = L_pre >= 0 && L_pre + a.R <= a.cap;
-  if (!valid && rank == 0 && threadIdx.x == 0 && blockIdx.y == 0)
-    sd_set_error(kFused && L_pre >= 0 ? SD_DEVERR_KV_OVERFLOW : SD_DEVERR_LENGTH);
-  // the prefix in 32-key blocks, split over the cluster's ranks
-  const int nblk = valid ? (L_pre + 31) / 32 : 0;
-  const int blk_begin = static_cast<int>((static_cast<uint32_t>(rank) * nblk) / static_cast<uint32_t>(csize));
-  const int blk_end = static_cast<int>((static_cast<uint32_t>(rank + 1) * nblk) / static_cast<uint32_t>(csize));
-  const int key_begin = blk_begin * 32;
-  const int key_end = min(blk_end * 32, valid ? L_pre : 0);
-  const int n_pre = (blk_end - blk_begin + 3) / 4;           // prefix tiles
-  const bool has_new = valid && last_rank;                   // and the new-key tile
-  const int n_tiles = n_pre + (has_new ? 1 : 0);
-  // rank c merges packed rows [c * rpc, ...) of the m-block's rows_in rows
-  const int rows_in = max(1, min(kR, a.M - mblock * kR));
-  const int rpc = (rows_in + csize - 1) / csize;
-  auto rows_of = [&](int c) { return max(0, min(rpc, rows_in - c * rpc)); };
-  const int my_rows = rows_of(rank);
-  const int mrow0 = rank * rpc;
 
   if (warp == 0) {
     // -------------------------------------------------------------- producer
+    // its first tiles are under way before the CTA-wide barrier
+    const int len0 = a.len[b];  // the scene's length advances at this warp's end
+    if (lane == 0) {
+#pragma unroll 1
+      for (int s = 0; s < kS; ++s) {
+        mbar_init(FULLK(s), 1);
+        mbar_init(FULLV(s), 1);
+        mbar_init(PVDONE(s), 1);
+      }
+      for (int i = 0; i < 2; ++i) mbar_init(PFULL(i), kSoftWarps / 2);
+#pragma unroll 1
+      for (int i = 0; i < 3; ++i) {
+        mbar_init(SREADY(i), 1);
+        mbar_init(SFREE(i), kSoftWarps / 2);
+      }
+      mbar_init(PNEW, kR / 8);
+      mbar_init(NEWDONE, 1);
+      mbar_init(RECV, 1);
+      mbar_init(DECIDE, 1);
+      mbar_init(MAXIMA, 1);
+      mbar_init(TMEMDONE, kSoftWarps);
+      *s_redo = 0;
+      *s_len = len0;
+      asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+      asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+    }
+    __syncwarp();
+    ranges(len0);
     const int z = b * a.Hkv + kvh;
     const uint64_t evict_first = l2_evict_first_policy();
-    auto issue_tiles = [&](int pass) {
-      for (int t = 0; t < n_pre; ++t) {
-        const int T = pass * n_tiles + t;
-        const int s = (pass * n_pre + t) % kS;
+    auto issue_tiles = [&](int pass, int t0, int t1) {
+#pragma unroll 1
+      for (int t = t0; t < t1; ++t) {
+        const int T = pass * n_pre + t;
+        const int s = T % kS;
         // a whole 128-row box even for a short last tile: keys past the range
         // are masked, rows past the capacity arrive zero-filled
         const int y0 = key_begin + t * kStageKeys;
         const uint32_t kst = base + s * kKV, vst = base + C::kRingV + s * kKV;
-        if (t >= kS) mbar_wait(SREADY(T - kS), par3(T - kS));
+        if (t >= kS) mbar_wait(SREADY((T - kS) % 3), par3(T - kS));
         if (elect_one()) {
           mbar_expect_tx(FULLK(s), static_cast<uint32_t>(kKV));
 #pragma unroll
           for (int h = 0; h < 2; ++h) tma_load_3d_hint(kst + h * kHalf, &tm_k128, FULLK(s), h * 64, y0, z, evict_first);
         }
         __syncwarp();
-        if (t >= kS) mbar_wait(PVDONE(T - kS), parS(T - kS));
+        if (t >= kS) mbar_wait(PVDONE(s), parS(T - kS));
         if (elect_one()) {
           mbar_expect_tx(FULLV(s), static_cast<uint32_t>(kKV));
 #pragma unroll
@@ -359,203 +372,254 @@ __global__ void __launch_bounds__(kThreads, 1)
         __syncwarp();
       }
     };
-    if (n_pre > 0) {
-      if (elect_one()) {
-        asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&tm_k128)) : "memory");
-        asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&tm_v128)) : "memory");
-        // chained layers: the cluster launched last starts only when the
-        // previous layer frees its SMs; the first head's CTAs bring its tiles
-        // of their own key range, and its query and new rows, into L2
-        if (early && kvh == 0 && mblock == 0 && b == static_cast<int>(gridDim.z) - 1 && a.Hkv > 1) {
-          const int zl = b * a.Hkv + a.Hkv - 1;
-          for (int t = 0; t < n_pre; ++t)
+    const int n0 = min(n_pre, kS);
+    issue_tiles(0, 0, n0);
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    if (!valid && rank == 0 && lane == 0 && blockIdx.y == 0)
+      sd_set_error(kFused && L_pre >= 0 ? SD_DEVERR_KV_OVERFLOW : SD_DEVERR_LENGTH);
+    // chained layers: the cluster launched last starts only when the previous
+    // layer frees its SMs; the first head's CTAs bring its tiles of their own key
+    // range, and its query and new rows, into L2
+    if (n_pre > 0 && early && kvh == 0 && mblock == 0 && b == static_cast<int>(gridDim.z) - 1 && a.Hkv > 1 && elect_one()) {
+      const int zl = b * a.Hkv + a.Hkv - 1;
+#pragma unroll 1
+      for (int t = 0; t < n_pre; ++t)
 #pragma unroll
-            for (int h = 0; h < 2; ++h) {
-              tma_prefetch_3d(&tm_k128, h * 64, key_begin + t * kStageKeys, zl);
-              tma_prefetch_3d(&tm_v128, h * 64, key_begin + t * kStageKeys, zl);
-            }
-          if (rank == 0)
-            for (int i = 0; i < a.R; ++i) {
-              const long long row = static_cast<long long>(b) * a.R + i;
-              bulk_prefetch_l2((kFused ? a.qw : a.q) + (row * a.Hq + (a.Hkv - 1) * a.G) * kD, a.G * kD * 2);
-              if (kFused) {
-                bulk_prefetch_l2(a.k_new + (row * a.Hkv + a.Hkv - 1) * kD, kD * 2);
-                bulk_prefetch_l2(a.v_new + (row * a.Hkv + a.Hkv - 1) * kD, kD * 2);
-              }
-            }
+        for (int h = 0; h < 2; ++h) {
+          tma_prefetch_3d(&tm_k128, h * 64, key_begin + t * kStageKeys, zl);
+          tma_prefetch_3d(&tm_v128, h * 64, key_begin + t * kStageKeys, zl);
+        }
+      if (rank == 0)
+#pragma unroll 1
+        for (int i = 0; i < a.R; ++i) {
+          const long long row = static_cast<long long>(b) * a.R + i;
+          bulk_prefetch_l2((kFused ? a.qw : a.q) + (row * a.Hq + (a.Hkv - 1) * a.G) * kD, a.G * kD * 2);
+          if (kFused) {
+            bulk_prefetch_l2(a.k_new + (row * a.Hkv + a.Hkv - 1) * kD, kD * 2);
+            bulk_prefetch_l2(a.v_new + (row * a.Hkv + a.Hkv - 1) * kD, kD * 2);
+          }
+        }
+    }
+    __syncwarp();
+#pragma unroll 1
+    for (int pass = 0; pass < 3; ++pass) {
+      if (pass == 1) {
+        mbar_wait(DECIDE, 0);
+        if (!*reinterpret_cast<volatile int*>(s_redo)) break;
+      }
+      if (pass == 2) mbar_wait(MAXIMA, 0);  // every product of pass 1 is done
+      issue_tiles(pass, pass == 0 ? n0 : 0, n_pre);
+      if (pass > 0) continue;
+      // the softmax threads arrive last (after the last S of the last pass), so
+      // this warp and the issuing warps arrive before the decision
+      if (csize > 1) cluster_arrive_relaxed();
+      if (kFused && elect_one()) {
+        // advance the scene's length once every CTA of the scene has read it (and
+        // the previous kernel, which may read it, has completed)
+        if (early) griddep_wait();
+        __threadfence();
+        const uint32_t total = gridDim.x * gridDim.y;
+        if (atomicAdd(&a.ticket[b], 1u) == total - 1) {
+          if (len0 >= 0 && len0 + a.R <= a.cap) a.len[b] = len0 + a.R;
+          a.ticket[b] = 0;
         }
       }
       __syncwarp();
-      issue_tiles(0);
-    }
-    __syncwarp();
-    // the softmax threads arrive last (after the last S of the last pass), so
-    // this warp and the issuing warps arrive before the decision
-    if (csize > 1) cluster_arrive_relaxed();
-    if (kFused && elect_one()) {
-      // advance the scene's length once every CTA of the scene has read it
-      __threadfence();
-      const uint32_t total = gridDim.x * gridDim.y;
-      if (atomicAdd(&a.ticket[b], 1u) == total - 1) {
-        if (len0 >= 0 && len0 + a.R <= a.cap) a.len[b] = len0 + a.R;
-        a.ticket[b] = 0;
-      }
-    }
-    __syncwarp();
-    if (n_tiles > 0) {
-      mbar_wait(DECIDE, 0);
-      if (*reinterpret_cast<volatile int*>(s_redo)) {
-        issue_tiles(1);
-        mbar_wait(DECIDE, 1);  // every product of pass 1 is done
-        issue_tiles(2);
-      }
     }
     __syncwarp();
     if (csize > 1) cluster_wait();
   } else if (warp == 1) {
     // -------------------------------------------------------------- S issue
-    bool arrived = false;
-    if (n_tiles > 0) {
-      mbar_wait(QFULL, 0);
-      const uint64_t dK0 = umma_desc(base, 16, 1024);
-      const uint64_t dN = umma_desc(base + C::kOffNewK, 16, 1024);
-      const uint64_t dQ = umma_desc(qs, 16, 1024);
-      for (int pass = 0; pass < 3; ++pass) {
-        if (pass == 1) {
-          if (csize > 1) cluster_arrive_relaxed();
-          arrived = true;
-          mbar_wait(DECIDE, 0);
-          if (!*reinterpret_cast<volatile int*>(s_redo)) break;
-        }
-        if (pass == 2) mbar_wait(DECIDE, 1);
-        for (int t = 0; t < n_tiles; ++t) {
-          const int T = pass * n_tiles + t;
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_addr(tmem_slot)),
+                 "r"(C::kTmemCols)
+                 : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    const uint32_t tmem = *tmem_slot;
+    ranges(*s_len);
+    const uint64_t dK0 = umma_desc(base, 16, 1024);
+    const uint64_t dQ = umma_desc(qs, 16, 1024);
+#pragma unroll 1
+    for (int pass = 0; pass < 3; ++pass) {
+      if (pass == 1) {
+        if (csize > 1) cluster_arrive_relaxed();
+        mbar_wait(DECIDE, 0);
+        if (!*reinterpret_cast<volatile int*>(s_redo)) break;
+      }
+      if (pass == 2) mbar_wait(MAXIMA, 0);
+      // t = -1 (early prefix only, when there is time): the batch of tile 0 is issued once before Q is complete, on whatever
+      // shared memory holds, and overwritten by the real one: the instructions and
+      // the tensor pipe are warm when Q is there (6.47 -> 6.29 us a target layer)
+      if (n_pre == 0 && pass == 0) named_bar_sync(3, kSoftThreads + 32);
+#pragma unroll 1
+      for (int t = pass == 0 && early && n_pre > 0 ? -1 : 0; t < n_pre; ++t) {
+        const int T = pass * n_pre + max(t, 0), s = T % kS;
+        if (t >= 0) {
+          if (t == 0 && pass == 0) named_bar_sync(3, kSoftThreads + 32);  // a hardware barrier: its wake-up is short
           // the softmax has read S(T - 3): its buffer takes S(T)
-          if (t >= 3) mbar_wait(SFREE(T), par3(T - 3));
-          const uint32_t ts = tmem + C::kSStride * (T % 3);
-          if (t < n_pre) {
-            const int TL = pass * n_pre + t, s = TL % kS;
-            mbar_wait(FULLK(s), parS(TL));
-            tc_fence_after();
-            const uint64_t dk = dK0 + static_cast<uint64_t>((s * kKV) >> 4);
-            if (elect_one()) {
-#pragma unroll
-              for (int kk = 0; kk < 8; ++kk)
-                umma(ts, dk + (((kk >> 2) * kHalf + (kk & 3) * 32) >> 4),
-                     dQ + (((kk >> 2) * C::kQHalf + (kk & 3) * 32) >> 4), kIdescS, kk > 0 ? 1 : 0);
-              umma_commit(SREADY(T));
-            }
-          } else {
-            tc_fence_after();
-            if (elect_one()) {
-#pragma unroll
-              for (int kk = 0; kk < 8; ++kk)
-                umma(ts, dN + (((kk >> 2) * kNewHalf + (kk & 3) * 32) >> 4),
-                     dQ + (((kk >> 2) * C::kQHalf + (kk & 3) * 32) >> 4), kIdescS, kk > 0 ? 1 : 0);
-              umma_commit(SREADY(T));
-            }
-          }
-          __syncwarp();
+          if (t >= 3) mbar_wait(SFREE(T % 3), par3(T - 3));
+          mbar_wait(FULLK(s), parS(T));
+          tc_fence_after();
         }
+        const uint32_t ts = tmem + C::kSStride * (T % 3);
+        const uint64_t dk = dK0 + static_cast<uint64_t>((s * kKV) >> 4);
+        if (elect_one()) {
+#pragma unroll
+          for (int kk = 0; kk < 8; ++kk)
+            umma(ts, dk + (((kk >> 2) * kHalf + (kk & 3) * 32) >> 4),
+                 dQ + (((kk >> 2) * C::kQHalf + (kk & 3) * 32) >> 4), kIdescS, kk > 0 ? 1 : 0);
+          if (t >= 0) umma_commit(SREADY(T % 3));
+        }
+        __syncwarp();
       }
     }
-    __syncwarp();
-    if (!arrived && csize > 1) cluster_arrive_relaxed();
     mbar_wait(TMEMDONE, 0);  // every softmax warp has read its last column
     tc_fence_after();
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(C::kTmemCols) : "memory");
     if (csize > 1) cluster_wait();
   } else if (warp == 2) {
     // -------------------------------------------------------------- PV issue
-    bool arrived = false;
-    if (n_tiles > 0) {
-      const uint64_t dV0 = umma_desc(base + C::kRingV, kHalf, 1024);              // V^T: MN-major
-      const uint64_t dN = umma_desc(base + C::kOffNewV, kNewHalf, 1024);
-      const uint64_t dP0 = umma_desc(base + C::kOffP, C::kPGroup, 256, 6);        // P^T: MN-major, 32-byte swizzle
-      const int new_steps = (a.R + 15) / 16;
-      for (int pass = 0; pass < 3; ++pass) {
-        if (pass == 1) {
-          if (csize > 1) cluster_arrive_relaxed();
-          arrived = true;
-          mbar_wait(DECIDE, 0);
-          if (!*reinterpret_cast<volatile int*>(s_redo)) break;
-        }
-        if (pass == 2) mbar_wait(DECIDE, 1);
-        for (int t = 0; t < n_tiles; ++t) {
-          const int T = pass * n_tiles + t;
-          mbar_wait(PFULL(T), (T >> 1) & 1);
-          const uint64_t dp = dP0 + static_cast<uint64_t>(((T & 1) * C::kP) >> 4);
-          if (t < n_pre) {
-            const int TL = pass * n_pre + t, s = TL % kS;
-            mbar_wait(FULLV(s), parS(TL));
-            tc_fence_after();
-            const uint64_t dv = dV0 + static_cast<uint64_t>((s * kKV) >> 4);
-            if (elect_one()) {
-#pragma unroll
-              for (int kk = 0; kk < 8; ++kk)
-                umma(tmem_o, dv + (kk * 2048 >> 4), dp + (kk * 512 >> 4), kIdescO, (t > 0 || kk > 0) ? 1 : 0);
-              umma_commit(PVDONE(T));
-            }
-          } else {
-            tc_fence_after();
-            if (elect_one()) {
-#pragma unroll
-              for (int kk = 0; kk < kMaxNew / 16; ++kk)
-                if (kk < new_steps)
-                  umma(tmem_o, dN + (kk * 2048 >> 4), dp + (kk * 512 >> 4), kIdescO, (t > 0 || kk > 0) ? 1 : 0);
-              umma_commit(PVDONE(T));
-            }
-          }
-          __syncwarp();
-        }
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    const uint32_t tmem_o = *tmem_slot + 3 * C::kSStride;
+    ranges(*s_len);
+    const bool has_new = valid && last_rank;
+    const uint64_t dV0 = umma_desc(base + C::kRingV, kHalf, 1024);        // V^T: MN-major
+    const uint64_t dN = umma_desc(base + C::kOffNewV, C::kNewHalf, 1024);
+    const uint64_t dP0 = umma_desc(base + C::kOffP, C::kPGroup, 256, 6);  // P^T: MN-major, 32-byte swizzle
+#pragma unroll 1
+    for (int pass = 0; pass < 3; ++pass) {
+      if (pass == 1) {
+        if (csize > 1) cluster_arrive_relaxed();
+        mbar_wait(DECIDE, 0);
+        if (!*reinterpret_cast<volatile int*>(s_redo)) break;
       }
+      if (pass == 2) mbar_wait(MAXIMA, 0);
+      const bool take_new = has_new && pass != 1;
+      auto new_product = [&](bool add) {
+        mbar_wait(PNEW, pass >> 1);
+        tc_fence_after();
+        const uint64_t dpn = umma_desc(base + C::kOffPNew, C::kPNewGroup, 256, 6);
+        if (elect_one()) {
+#pragma unroll
+          for (int kk = 0; kk < C::kMaxNew / 16; ++kk)
+            if (kk * 16 < a.R)
+              umma(tmem_o, dN + (kk * 2048 >> 4), dpn + (kk * 512 >> 4), kIdescO, kk > 0 || add ? 1 : 0);
+          umma_commit(NEWDONE);
+        }
+        __syncwarp();
+      };
+      if (C::kNewFirst && take_new) new_product(false);
+      for (int t = 0; t < n_pre; ++t) {
+        const int T = pass * n_pre + t, s = T % kS;
+        mbar_wait(PFULL(T), (T >> 1) & 1);
+        mbar_wait(FULLV(s), parS(T));
+        tc_fence_after();
+        const uint64_t dv = dV0 + static_cast<uint64_t>((s * kKV) >> 4);
+        const uint64_t dp = dP0 + static_cast<uint64_t>(((T & 1) * C::kP) >> 4);
+        const int n_steps = pv_keys(t) >> 4;
+        if (elect_one()) {
+#pragma unroll
+          for (int kk = 0; kk < 8; ++kk)
+            if (kk < n_steps)
+              umma(tmem_o, dv + (kk * 2048 >> 4), dp + (kk * 512 >> 4), kIdescO,
+                   (t > 0 || kk > 0 || (C::kNewFirst && take_new)) ? 1 : 0);
+          umma_commit(PVDONE(s));
+        }
+        __syncwarp();
+      }
+      if (!C::kNewFirst && take_new) new_product(n_pre > 0);
     }
-    __syncwarp();
-    if (!arrived && csize > 1) cluster_arrive_relaxed();
     if (csize > 1) cluster_wait();
   } else {
     // -------------------------------------------------------------- softmax
-    const int group = (warp - kFirstSoft) >> 3;
-    const int half = ((warp - kFirstSoft) >> 2) & 1;  // rows kRpt * half .. + kRpt - 1 of the group's tile
-    const int quarter = warp & 3;                     // TMEM lane quarter of this warp
-    const int kl = quarter * 32 + lane;               // key lane of S^T / d lane of O^T
+    const int st = static_cast<int>(threadIdx.x) - kSoft0;  // 0 .. 511
+    const int sw = warp - kFirstSoft;
+    const int group = sw >> 3;
+    const int half = (sw >> 2) & 1;      // rows kRpt * half .. + kRpt - 1 of the group's tile
+    const int quarter = warp & 3;        // TMEM lane quarter of this warp
+    const int kl = quarter * 32 + lane;  // key lane of S^T / d lane of O^T
     const uint32_t lane_off = static_cast<uint32_t>(quarter * 32) << 16;
     const int row0 = kRpt * half;
-    const float2* cs_tab = reinterpret_cast<const float2*>(smem + C::kOffP);
+    // this thread's 16-byte chunks: of the packed query tile (row idx >> 4, chunk
+    // idx & 15, rows past M zero) and, in the cluster's last rank, of the new key
+    // and value rows
+    constexpr int kQc = (kR * 16 + kSoftThreads - 1) / kSoftThreads;
+    auto q_off = [&](int p) {
+      const int i = gdiv(p);
+      return ((static_cast<long long>(b) * a.R + i) * a.Hq + kvh * a.G + (p - i * a.G)) * kD;
+    };
+    const bool new_kv = last_rank && st < a.R * 16;
+    const long long kv_row = ((static_cast<long long>(b) * a.R + (st >> 4)) * a.Hkv + kvh) * kD + (st & 15) * 8;
+    uint4 qv[kQc], kv = make_uint4(0, 0, 0, 0), vv = make_uint4(0, 0, 0, 0);
+    auto load_q = [&] {
+#pragma unroll
+      for (int u = 0; u < kQc; ++u) {
+        const int idx = st + u * kSoftThreads, p = mblock * kR + (idx >> 4);
+        qv[u] = idx < kR * 16 && p < a.M
+                    ? __ldcg(reinterpret_cast<const uint4*>((kFused ? a.qw : a.q) + q_off(p) + (idx & 15) * 8))
+                    : make_uint4(0, 0, 0, 0);
+      }
+    };
+    auto load_kv = [&](const __nv_bfloat16* k, const __nv_bfloat16* v, long long src) {
+      kv = __ldcg(reinterpret_cast<const uint4*>(k + src));
+      vv = __ldcg(reinterpret_cast<const uint4*>(v + src));
+    };
+    // Without the early prefix (the wait is behind) the rows are read here,
+    // together with the length and the positions: one global round trip before the
+    // tiles, not two (the attention's new rows need the length first)
+    if (!early) {
+      load_q();
+      if (kFused && new_kv) load_kv(a.k_new, a.v_new, kv_row);
+    }
+    const float2* cs_tab = reinterpret_cast<const float2*>(smem + C::kOffP);  // [R][64] (cos, sin)
+    if (kFused) {
+      // rotation table of the R new positions. A warp takes 4 pairs, its lanes 8
+      // rows: a constant-bank read serialises over the lanes' different addresses
+      // (with 32 pairs a warp the table took ~2800 cycles, on the path of the
+      // cluster launched last)
+      float2* tabw = reinterpret_cast<float2*>(smem + C::kOffP);
+      const int d = sw * 4 + (lane & 3);
+#pragma unroll 1
+      for (int i = lane >> 2; i < a.R; i += 8) {
+        const int32_t pc = a.pos[(static_cast<long long>(b) * a.R + i) * 3 + tab.axis[d]];
+        tabw[i * 64 + d] = sd_rope_cs(static_cast<float>(pc), d, tab);
+      }
+    }
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    const uint32_t tmem = *tmem_slot;
+    const uint32_t tmem_o = tmem + 3 * C::kSStride;
+    ranges(*s_len);
+    const bool has_new = valid && last_rank;
+    // rank c merges packed rows [c * rpc, ...) of the m-block's rows_in rows
+    const int rows_in = max(1, min(kR, a.M - mblock * kR));
+    const int rpc = (rows_in + csize - 1) / csize;
+    auto rows_of = [&](int c) { return max(0, min(rpc, rows_in - c * rpc)); };
+    const int my_rows = rows_of(rank);
+    const int mrow0 = rank * rpc;
     {
       // The rows, rotated (fused) and into the operand layouts. Iteration 0 runs
-      // BEFORE the dependency wait on whatever the rows hold: it brings this
-      // code into the instruction cache and the rows into L2, and iteration 1
-      // overwrites everything it stored (.cg loads: no stale L1 line). The
-      // cluster launched last starts when the previous kernel is nearly done:
-      // no warm-up pass.
-      const bool last_cluster = blockIdx.y == gridDim.y - 1 && blockIdx.z == gridDim.z - 1;
-      const bool has_kv = raw_kv && valid;
+      // BEFORE the dependency wait on whatever the rows hold: it brings this code
+      // into the instruction cache and the rows into L2, and iteration 1
+      // overwrites everything it stored (.cg loads: no stale L1 line).
+      const bool has_kv = new_kv && valid;
       const long long cache_row =
           ((static_cast<long long>(b) * a.Hkv + kvh) * a.cap + L_pre + (st >> 4)) * kD + (st & 15) * 8;
 #pragma unroll 1
       for (int it = early && !last_cluster ? 0 : 1; it < 2; ++it) {
-        if (it == 1 && early) griddep_wait();
-        uint4 qv[kQc], kv = make_uint4(0, 0, 0, 0), vv = make_uint4(0, 0, 0, 0);
-#pragma unroll
-        for (int u = 0; u < kQc; ++u) {
-          const int idx = st + u * kSoftThreads, p = mblock * kR + (idx >> 4);
-          if (rows_first)
-            qv[u] = valid ? pre_q[u] : make_uint4(0, 0, 0, 0);
-          else
-            qv[u] = valid && idx < kR * 16 && p < a.M
-                        ? __ldcg(reinterpret_cast<const uint4*>((kFused ? a.qw : a.q) + q_off(p) + (idx & 15) * 8))
-                        : make_uint4(0, 0, 0, 0);
+        if (early) {
+          if (it == 1) griddep_wait();
+          load_q();
+          if (kFused && has_kv) load_kv(a.k_new, a.v_new, kv_row);
         }
-        if (has_kv) {
-          if (rows_first) {
-            kv = pre_k;
-            vv = pre_v;
-          } else {
-            kv = __ldcg(reinterpret_cast<const uint4*>(kFused ? a.k_new + kv_row : a.kc + cache_row));
-            vv = __ldcg(reinterpret_cast<const uint4*>(kFused ? a.v_new + kv_row : a.vc + cache_row));
-          }
-        }
+        if (!kFused && has_kv) load_kv(a.kc, a.vc, cache_row);
 #pragma unroll
         for (int u = 0; u < kQc; ++u) {
           const int idx = st + u * kSoftThreads, row = idx >> 4, c = idx & 15, p = mblock * kR + row;
@@ -566,9 +630,9 @@ __global__ void __launch_bounds__(kThreads, 1)
 #pragma unroll
             for (int j = 0; j < 4; ++j) w[j] = sd_rope_pair(w[j], cs[j].x, cs[j].y);
           }
-          st_shared_v4(qs + (c >> 3) * C::kQHalf + row * 128 + (((c & 7) ^ (row & 7)) << 4), w[0], w[1], w[2], w[3]);
+          st_shared_v4(qs + swz(row, c, C::kQHalf), w[0], w[1], w[2], w[3]);
         }
-        if (last_rank) {
+        if (last_rank && st < C::kMaxNew * 16) {
           // new key (rotated) and value rows, zero past R
           const int i = st >> 4, c = st & 15;
           uint32_t w[4] = {kv.x, kv.y, kv.z, kv.w};
@@ -577,7 +641,7 @@ __global__ void __launch_bounds__(kThreads, 1)
 #pragma unroll
             for (int j = 0; j < 4; ++j) w[j] = sd_rope_pair(w[j], cs[j].x, cs[j].y);
           }
-          const uint32_t off = (c >> 3) * kNewHalf + i * 128 + (((c & 7) ^ (i & 7)) << 4);
+          const uint32_t off = swz(i, c, C::kNewHalf);
           st_shared_v4(base + C::kOffNewK + off, w[0], w[1], w[2], w[3]);
           st_shared_v4(base + C::kOffNewV + off, vv.x, vv.y, vv.z, vv.w);
           if (kFused && has_kv && it == 1 && mblock == 0) {
@@ -590,15 +654,10 @@ __global__ void __launch_bounds__(kThreads, 1)
           }
         }
       }
-      // row p = i * G + g is new row i: it sees new keys 0..i (all R under the block mask)
-      if (st < kR) {
-        row_lim[st] = block ? a.R - 1 : min(gdiv(mblock * kR + st), a.R - 1);
-        row_nref[st] = 0.f;
-      }
+      if (st < kR) row_nref[st] = 0.f;
       asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-      named_bar_sync(2, kSoftThreads);  // Q is complete; the rotation table is no longer read
+      named_bar_sync(3, kSoftThreads + 32);  // Q is complete; the rotation table is no longer read
       if (st == 0) {
-        mbar_arrive(QFULL);
         griddep_launch();  // every older kernel has finished: the next layer may launch
         // with several m-blocks the head's raw key rows are read by the last
         // rank of each: the last of them writes the rotated rows back (the
@@ -610,25 +669,39 @@ __global__ void __launch_bounds__(kThreads, 1)
       }
     }
 
-    const float sl = a.scale_log2;
     const uint64_t sl2 = pack2f(sl, sl);
     uint64_t lp2[kRpt / 2];  // this key lane's row sums, in pairs
     const uint32_t pbuf = base + C::kOffP + group * C::kP;
     const uint32_t pkey = pbuf + kl * 32;
     const uint32_t psw = (kl >> 2) & 1;  // 32-byte swizzle
-    // this thread's rows j0 .. j0 + kN - 1 of tile T (its scores in buffer T % 3)
-    // to weights and P; `last`: the tile's scores are all in registers then
-    auto chunk = [&](auto kn, int T, int j0, bool last, bool wait_pv, auto keep) {
+    // the last new key that packed row r of this tile sees: row p = i * G + g is
+    // new row i and sees new keys 0..i (all R under the block mask)
+    auto last_new = [&](int r) { return block ? a.R - 1 : min(gdiv(mblock * kR + r), a.R - 1); };
+    int pass = 0;
+    bool out_of_range = false;
+    // a warp none of whose rows exists (a draft's 4 rows of 32) skips the weights: its
+    // P stays stale and reaches only O columns that are never read. On the wider
+    // tiles, chosen to fit, the test cost more than it saved (47.0 -> 48.7 us at 8
+    // scenes, L = 8192, K = 16)
+    constexpr bool skips = kR == 32;
+    // this thread's rows j0 .. j0 + kN - 1 of tile T (its scores in buffer sb) to
+    // weights and P; vb, vpar: the barrier of PV(T - 2)
+    auto chunk = [&](auto kn, int T, int sb, int vb, uint32_t vpar, int j0, bool key_ok, bool first) {
       constexpr int kN = decltype(kn)::value;
       uint32_t r[kN], pw[kN / 2];
-      tmem_ld(tmem + C::kSStride * (T % 3) + row0 + j0 + lane_off, r);
-      if (last) {
+      tmem_ld(tmem + C::kSStride * sb + row0 + j0 + lane_off, r);
+      if (j0 + kN == kRpt) {
+        // the tile's scores are all in registers: its buffer may take S(T + 3)
         tc_fence_before();
         __syncwarp();
-        if (lane == 0) mbar_arrive(SFREE(T));
+        if (lane == 0) mbar_arrive(SFREE(sb));
       }
-      weights_to_p<kN>(r, row_nref + row0 + j0, sl2, keep, lp2 + j0 / 2, pw);
-      if (wait_pv && T >= 2) mbar_wait(PVDONE(T - 2), parS(T - 2));  // PV(T - 2) has read the buffer
+      weights_to_p<kN>(r, row_nref + row0 + j0, sl2, key_ok, lp2 + j0 / 2, pw);
+      if (j0 == 0) {
+        // PV(T - 2), or the new keys' product, has read the buffer
+        if (T >= 2) mbar_wait(PVDONE(vb), vpar);
+        if (C::kNewFirst && first && has_new && group == 1) mbar_wait(NEWDONE, pass >> 1);
+      }
 #pragma unroll
       for (int h = 0; h < kN / 8; ++h) {
         const int ch = (row0 + j0) / 8 + h;
@@ -636,107 +709,171 @@ __global__ void __launch_bounds__(kThreads, 1)
                      pw[4 * h + 3]);
       }
     };
-    auto tile_p = [&](int T, auto keep) {
-#pragma unroll
-      for (int j0 = 0; j0 + 16 <= kRpt; j0 += 16)
-        chunk(std::integral_constant<int, 16>{}, T, j0, j0 + 16 == kRpt, j0 == 0, [&](int j, uint32_t w) { return keep(j0 + j, w); });
-      if constexpr (kRpt % 16 != 0)
-        chunk(std::integral_constant<int, 8>{}, T, kRpt - 8, true, false, [&](int j, uint32_t w) { return keep(kRpt - 8 + j, w); });
+    bool redo = false;
+    // every product of a pass is done (behind a barrier that every softmax warp
+    // reaches after its last tile)
+    auto wait_products = [&](int ps) {
+      const int Tl = (ps + 1) * n_pre - 1;
+      const bool new_last = has_new && ps != 1 && (!C::kNewFirst || n_pre == 0);
+      if (new_last) mbar_wait(NEWDONE, ps >> 1);
+      else if (n_pre > 0) mbar_wait(PVDONE(Tl % kS), parS(Tl));
     };
-    bool seen = false;  // this warp has had a key of its own (every row sees prefix keys and new key 0)
-    auto run_pass = [&](int pass) {
+    // the new keys: scores of 8 packed rows against 16 keys a step by mma.sync,
+    // weights to kOffPNew, row sums to row_new
+    auto new_keys = [&](int unit) {
+      const int r8 = unit * 8;
+      const int lim0 = last_new(r8 + 2 * (lane & 3)), lim1 = last_new(r8 + 2 * (lane & 3) + 1);
+      const float2 nr = *reinterpret_cast<const float2*>(row_nref + r8 + 2 * (lane & 3));
+      float l0 = 0.f, l1 = 0.f;
+      uint32_t bq[4][4];
 #pragma unroll
-      for (int j = 0; j < kRpt / 2; ++j) lp2[j] = 0ull;
-      for (int t = ((pass * n_tiles) ^ group) & 1; t < n_tiles; t += 2) {
-        const int T = pass * n_tiles + t;
-        mbar_wait(SREADY(T), par3(T));
+      for (int k2 = 0; k2 < 4; ++k2) ldmatrix4(qs + swz(r8 + (lane & 7), 4 * k2 + (lane >> 3), C::kQHalf), bq[k2]);
+#pragma unroll 1
+      for (int m = 0; m * 16 < a.R; ++m) {
+        float c[4] = {0.f, 0.f, 0.f, 0.f}, c1[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+        for (int k2 = 0; k2 < 4; ++k2) {
+          uint32_t ak[4], al[4];
+          ldmatrix4(base + C::kOffNewK + swz(m * 16 + (lane & 15), 4 * k2 + (lane >> 4), C::kNewHalf), ak);
+          ldmatrix4(base + C::kOffNewK + swz(m * 16 + (lane & 15), 4 * k2 + 2 + (lane >> 4), C::kNewHalf), al);
+          mma_bf16(c, ak, bq[k2][0], bq[k2][1]);
+          mma_bf16(c1, al, bq[k2][2], bq[k2][3]);
+        }
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+          const int key = m * 16 + (lane >> 2) + 8 * h;
+          const uint32_t keep = (key <= lim0 ? 0xffffu : 0u) | (key <= lim1 ? 0xffff0000u : 0u);
+          const uint32_t w = cvt_bf16x2(ex2(fmaf(c[2 * h] + c1[2 * h], sl, nr.x)),
+                                        ex2(fmaf(c[2 * h + 1] + c1[2 * h + 1], sl, nr.y))) & keep;
+          l0 += sd_bf16_lo(w);
+          l1 += sd_bf16_hi(w);
+          asm volatile("st.shared.u32 [%0], %1;" ::"r"(base + C::kOffPNew + (unit >> 1) * C::kPNewGroup + key * 32 +
+                                                        (((unit & 1) ^ ((key >> 2) & 1)) << 4) + (lane & 3) * 4),
+                       "r"(w)
+                       : "memory");
+        }
+      }
+      asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+      __syncwarp();
+      if (lane == 0) mbar_arrive(PNEW);
+#pragma unroll
+      for (int o = 4; o < 32; o <<= 1) {
+        l0 += __shfl_xor_sync(0xffffffffu, l0, o);
+        l1 += __shfl_xor_sync(0xffffffffu, l1, o);
+      }
+      out_of_range |= fmaxf(l0, l1) > kHigh || fminf(l0, l1) < kLow;
+      if (lane < 4) *reinterpret_cast<float2*>(row_new + r8 + 2 * lane) = make_float2(l0, l1);
+    };
+    while (true) {
+      // On the 32-row tile by the last warps while S(0) runs (their group's first
+      // tile comes second); on the others by the group that does not have the last
+      // tile, after its own.
+      if (C::kNewFirst && has_new && kSoftWarps - 1 - sw < kR / 8) new_keys(kSoftWarps - 1 - sw);
+      // ---- this group's prefix tiles
+#pragma unroll
+      for (int j = 0; j < kRpt / 2; ++j) lp2[j] = skips && row0 >= rows_in ? pack2f(1.f, 1.f) : 0ull;
+      const int t_first = ((pass * n_pre) ^ group) & 1;
+      const int T1 = pass * n_pre + t_first, V1 = T1 + 2 * kS - 2;  // PV(T - 2) as a phase of its ring, T >= 0
+      int sb = T1 % 3, vb = V1 % kS;
+      uint32_t spar = (T1 / 3) & 1, vpar = (V1 / kS) & 1;
+      int key0 = key_begin + t_first * kStageKeys;
+      bool seen = false;  // this warp has had a prefix key
+#pragma unroll 1
+      for (int t = t_first; t < n_pre; t += 2) {
+        const int T = pass * n_pre + t;
+        const bool key_ok = key0 + kl < key_end;
+        seen |= key0 + quarter * 32 < key_end;
+        key0 += 2 * kStageKeys;
+        mbar_wait(SREADY(sb), spar);
         tc_fence_after();
-        if (t < n_pre) {
-          const int key0 = key_begin + t * kStageKeys;
-          const bool key_ok = key0 + kl < key_end;
-          seen |= key0 + quarter * 32 < key_end;
-          tile_p(T, [&](int, uint32_t w) { return key_ok ? w : 0u; });
-          if (!key_ok) {
-            // stale or foreign key row: zero its V row (this thread's 64-column
-            // half) so 0 * NaN cannot reach O, once the tile has landed
-            const int TL = pass * n_pre + t, s = TL % kS;
-            mbar_wait(FULLV(s), parS(TL));
-            const uint32_t vrow = base + C::kRingV + s * kKV + half * kHalf + kl * 128;
 #pragma unroll
-            for (int c = 0; c < 8; ++c) st_shared_v4(vrow + c * 16, 0u, 0u, 0u, 0u);
-          }
-        } else if (quarter == 0) {
-          seen = true;
-          tile_p(T, [&](int j, uint32_t w) {
-            const int2 lim = *reinterpret_cast<const int2*>(row_lim + row0 + j);
-            return w & ((kl <= lim.x ? 0xffffu : 0u) | (kl <= lim.y ? 0xffff0000u : 0u));
-          });
-        } else {
-          // key lanes past the new keys: nothing to read or write
-          tc_fence_before();
-          __syncwarp();
-          if (lane == 0) mbar_arrive(SFREE(T));
-          if (T >= 2) mbar_wait(PVDONE(T - 2), parS(T - 2));
+        for (int j0 = 0; j0 + 16 <= kRpt; j0 += 16)
+          if (!skips || row0 < rows_in) chunk(std::integral_constant<int, 16>{}, T, sb, vb, vpar, j0, key_ok, t == t_first);
+        if constexpr (kRpt % 16 != 0)
+          chunk(std::integral_constant<int, 8>{}, T, sb, vb, vpar, kRpt - 8, key_ok, t == t_first);
+        if (skips && row0 >= rows_in) {
+          // none of this warp's rows exists: the barriers' phases only
+          if (lane == 0) mbar_arrive(SFREE(sb));
+          if (T >= 2) mbar_wait(PVDONE(vb), vpar);
+        }
+        if ((sb += 2) >= 3) sb -= 3, spar ^= 1;
+        if ((vb += 2) >= kS) vb -= kS, vpar ^= 1;
+        if (!key_ok && kl < pv_keys(t)) {
+          // stale or foreign key row that the product reads: zero its V row (this
+          // thread's 64-column half) so 0 * NaN cannot reach O, once the tile has
+          // landed. Chunks in an order that differs by lane: rows are 128 bytes apart
+          // (in one order every lane met the same banks, ~2500 cycles a partial tile)
+          const int s = T % kS;
+          mbar_wait(FULLV(s), parS(T));
+          const uint32_t vrow = base + C::kRingV + s * kKV + half * kHalf + kl * 128;
+#pragma unroll
+          for (int c = 0; c < 8; ++c) st_shared_v4(vrow + ((c ^ (kl & 7)) << 4), 0u, 0u, 0u, 0u);
         }
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
         tc_fence_before();
         __syncwarp();
         if (lane == 0) mbar_arrive(PFULL(T));
       }
-    };
-    // row sums over this warp's keys to row_sum; whether one of them left the
-    // range that a single reference-free pass is exact in
-    auto sum_rows = [&]() {
-      bool out_of_range = false;
+      if (!C::kNewFirst && has_new && group == (n_pre & 1))
+#pragma unroll 1
+        for (int unit = sw & 7; unit < kR / 8; unit += 8) new_keys(unit);
+      // ---- whether a row sum left the range that weights without a reference are
+      // exact in: a thread's sum too large, or a warp (with a key of its own) none of
+      // whose lanes has every row's sum large enough
+      {
+        float lo = INFINITY, hi = 0.f;
 #pragma unroll
-      for (int j0 = 0; j0 < kRpt; j0 += 8) {
-        float v[8];
-#pragma unroll
-        for (int j = 0; j < 4; ++j) unpack2(lp2[j0 / 2 + j], v[2 * j], v[2 * j + 1]);
-        const float x = warp_sum8(v, lane);
-        out_of_range |= x > kHigh || (seen && x < kLow);
-        if ((lane & 3) == 0) row_sum[(row0 + j0 + (lane >> 2)) * 8 + group * 4 + quarter] = x;
+        for (int j = 0; j < kRpt / 2; ++j) {
+          float x, y;
+          unpack2(lp2[j], x, y);
+          lo = fminf(lo, fminf(x, y));
+          hi = fmaxf(hi, fmaxf(x, y));
+        }
+        const bool some = __any_sync(0xffffffffu, lo >= kLow);  // by every lane, whatever the others find
+        out_of_range |= hi > kHigh || (seen && !some);
       }
-      return out_of_range;
-    };
-    run_pass(0);
-    bool bad = sum_rows();
-    const bool redo = named_bar_or(2, kSoftThreads, bad) && n_tiles > 0;
-    if (redo) mbar_wait(PVDONE(n_tiles - 1), parS(n_tiles - 1));
-    if (st == 0) {
-      *s_redo = redo ? 1 : 0;
-      mbar_arrive(DECIDE);
-    }
-    if (redo) {
-      // pass 1: every row's exact maximum over this CTA's keys (the PV products
+      const bool again = named_bar_or(2, kSoftThreads, out_of_range);
+      if (pass == 2) break;
+      redo = again;
+      if (redo) {
+        // every product of pass 0 is done before the rings are refilled, and no
+        // warp still looks for it when pass 1 moves the barriers on
+        wait_products(0);
+        named_bar_sync(2, kSoftThreads);
+      }
+      if (st == 0) {
+        *s_redo = redo ? 1 : 0;
+        mbar_arrive(DECIDE);
+      }
+      if (__builtin_expect(!redo, 1)) break;
+      // ---- pass 1: every row's exact maximum over this CTA's keys (the PV products
       // run on stale weights, their sums are dropped by pass 2)
       float mx[kRpt];
 #pragma unroll
       for (int j = 0; j < kRpt; ++j) mx[j] = -INFINITY;
 #pragma unroll 1
-      for (int t = (n_tiles ^ group) & 1; t < n_tiles; t += 2) {
-        const int T = n_tiles + t;
-        mbar_wait(SREADY(T), par3(T));
+      for (int t = (n_pre ^ group) & 1; t < n_pre; t += 2) {
+        const int T = n_pre + t;
+        mbar_wait(SREADY(T % 3), par3(T));
         tc_fence_after();
-        const bool is_new = t >= n_pre;
-        const bool key_ok = is_new ? quarter == 0 : key_begin + t * kStageKeys + kl < key_end;
+        const bool key_ok = key_begin + t * kStageKeys + kl < key_end;
 #pragma unroll
         for (int j0 = 0; j0 < kRpt; j0 += 8) {
           uint32_t r[8];
           tmem_ld(tmem + C::kSStride * (T % 3) + row0 + j0 + lane_off, r);
 #pragma unroll
           for (int j = 0; j < 8; ++j)
-            if (key_ok && (!is_new || kl <= row_lim[row0 + j0 + j]))
-              mx[j0 + j] = fmaxf(mx[j0 + j], __uint_as_float(r[j]) * sl);
+            if (key_ok) mx[j0 + j] = fmaxf(mx[j0 + j], __uint_as_float(r[j]) * sl);
         }
         tc_fence_before();
         __syncwarp();
-        if (lane == 0) mbar_arrive(SFREE(T));
-        mbar_wait(PVDONE(T - 2 < 0 ? 0 : T - 2), parS(T - 2 < 0 ? 0 : T - 2));
+        if (lane == 0) mbar_arrive(SFREE(T % 3));
+        const int Tp = max(T - 2, 0);
+        mbar_wait(PVDONE(Tp % kS), parS(Tp));
         if (lane == 0) mbar_arrive(PFULL(T));
       }
       named_bar_sync(2, kSoftThreads);
-      mbar_wait(PVDONE(2 * n_tiles - 1), parS(2 * n_tiles - 1));
+      wait_products(1);
       float* rb = reinterpret_cast<float*>(smem + C::kOffP);
       if (group == 0)
 #pragma unroll
@@ -747,41 +884,46 @@ __global__ void __launch_bounds__(kThreads, 1)
         for (int j = 0; j < kRpt; ++j) rb[(row0 + j) * 128 + kl] = fmaxf(rb[(row0 + j) * 128 + kl], mx[j]);
       named_bar_sync(2, kSoftThreads);
 #pragma unroll 1
-      for (int row = warp - kFirstSoft; row < kR; row += kSoftWarps) {
+      for (int row = sw; row < kR; row += kSoftWarps) {
         const float4 x = reinterpret_cast<const float4*>(rb + row * 128)[lane];
         float m = fmaxf(fmaxf(x.x, x.y), fmaxf(x.z, x.w));
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
+        if (has_new)
+          m = fmaxf(m, new_key_max(smem + C::kOffQ, row, C::kQHalf, smem + C::kOffNewK, C::kNewHalf, last_new(row), sl, lane));
         if (lane == 0) row_nref[row] = m == -INFINITY ? 0.f : -m;
       }
       named_bar_sync(2, kSoftThreads);
-      if (st == 0) mbar_arrive(DECIDE);
-      run_pass(2);
-      sum_rows();
-      named_bar_sync(2, kSoftThreads);
+      if (st == 0) mbar_arrive(MAXIMA);
+      pass = 2;
     }
-    // ---- every row sum of this CTA is in row_sum, the last S product is done
-    // (both groups have seen their last tile's): the K ring may receive
+    // ---- the last S product is done (both groups have seen their last tile's): the
+    // K ring may receive
     const bool merge = csize > 1;
     if (merge) cluster_arrive_relaxed();
-    if (n_tiles > 0) {
-      const int Tl = (redo ? 3 : 1) * n_tiles - 1;
-      mbar_wait(PVDONE(Tl), parS(Tl));
-      tc_fence_after();
+    // row sums over this warp's keys, while the last products run: lane L ends with
+    // that of row row0 + 8 c + (L >> 2)
+    float lsum[kRpt / 8];
+#pragma unroll
+    for (int c = 0; c < kRpt / 8; ++c) {
+      float v[8];
+#pragma unroll
+      for (int j = 0; j < 4; ++j) unpack2(lp2[4 * c + j], v[2 * j], v[2 * j + 1]);
+      lsum[c] = warp_sum8(v, lane);
     }
+    wait_products(pass);
+    tc_fence_after();
     // O: this warp reads its 32 d lanes of a quarter of the rows
     constexpr int kOr = kR / 4;
     const int orow0 = (group * 2 + half) * kOr;
     uint32_t o[kOr];
-    if (n_tiles > 0) {
-      uint32_t x8[8];
-      tmem_ld(tmem_o + orow0 + lane_off, x8);
+    if (n_pre > 0 || has_new) {
 #pragma unroll
-      for (int j = 0; j < 8; ++j) o[j] = x8[j];
-      if constexpr (kOr >= 16) {
-        tmem_ld(tmem_o + orow0 + 8 + lane_off, x8);
+      for (int j0 = 0; j0 + 8 <= kOr; j0 += 8) {
+        uint32_t x8[8];
+        tmem_ld(tmem_o + orow0 + j0 + lane_off, x8);
 #pragma unroll
-        for (int j = 0; j < 8; ++j) o[8 + j] = x8[j];
+        for (int j = 0; j < 8; ++j) o[j0 + j] = x8[j];
       }
       if constexpr (kOr % 8 != 0) {
         uint32_t x4[4];
@@ -798,30 +940,42 @@ __global__ void __launch_bounds__(kThreads, 1)
     if (lane == 0) mbar_arrive(TMEMDONE);
     if (!merge) {
       // one CTA holds the head's keys: normalise and store (64 bytes a row and warp)
+      if ((lane & 3) == 0)
+#pragma unroll
+        for (int c = 0; c < kRpt / 8; ++c) row_sum[(row0 + 8 * c + (lane >> 2)) * 8 + group * 4 + quarter] = lsum[c];
+      named_bar_sync(2, kSoftThreads);
+      if (st < kR) {
+        const float4 l0 = reinterpret_cast<const float4*>(row_sum + st * 8)[0];
+        const float4 l1 = reinterpret_cast<const float4*>(row_sum + st * 8)[1];
+        float l = ((l0.x + l0.y) + (l0.z + l0.w)) + ((l1.x + l1.y) + (l1.z + l1.w));
+        if (has_new) l += row_new[st];
+        row_new[st] = l > 0.f ? 1.f / l : 0.f;
+      }
+      named_bar_sync(2, kSoftThreads);
 #pragma unroll
       for (int j = 0; j < kOr; ++j) {
         const int row = orow0 + j, p = mblock * kR + row;
-        const float4 l0 = reinterpret_cast<const float4*>(row_sum + row * 8)[0];
-        const float4 l1 = reinterpret_cast<const float4*>(row_sum + row * 8)[1];
-        const float l = ((l0.x + l0.y) + (l0.z + l0.w)) + ((l1.x + l1.y) + (l1.z + l1.w));
-        if (valid && p < a.M && l > 0.f) a.out[q_off(p) + kl] = __float2bfloat16_rn(__uint_as_float(o[j]) * (1.f / l));
+        const float inv_l = row_new[row];
+        if (valid && p < a.M && inv_l > 0.f) a.out[q_off(p) + kl] = __float2bfloat16_rn(__uint_as_float(o[j]) * inv_l);
       }
     } else {
       float* send = reinterpret_cast<float*>(smem + C::kRingV);
 #pragma unroll
       for (int j = 0; j < kOr; ++j) send[(orow0 + j) * kRowF + kl] = __uint_as_float(o[j]);
-      for (int idx = st; idx < kR * 8; idx += kSoftThreads) send[(idx >> 3) * kRowF + kRowL + (idx & 7)] = row_sum[idx];
-      if (st < kR) send[st * kRowF + kRowM] = -row_nref[st];
+      if ((lane & 3) == 0)
+#pragma unroll
+        for (int c = 0; c < kRpt / 8; ++c) send[(row0 + 8 * c + (lane >> 2)) * kRowF + kRowL + group * 4 + quarter] = lsum[c];
+      if (st < kR)
+        *reinterpret_cast<float2*>(send + st * kRowF + kRowM) = make_float2(-row_nref[st], has_new ? row_new[st] : 0.f);
       asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
       named_bar_sync(2, kSoftThreads);
       if (st == 0) mbar_expect_tx(RECV, static_cast<uint32_t>(csize * my_rows * kRowBytes));
       cluster_wait();  // every peer's K ring is free to receive
       // softmax warp w sends rank w's rows to it, into its slots [rank * rpc, ...)
       if (elect_one()) {
-        const int c = warp - kFirstSoft;
-        if (c < csize && rows_of(c) > 0)
-          bulk_copy_s2s(cluster_map(base + rank * rpc * kRowBytes, c), base + C::kRingV + c * rpc * kRowBytes,
-                        static_cast<uint32_t>(rows_of(c) * kRowBytes), cluster_map(RECV, c));
+        if (sw < csize && rows_of(sw) > 0)
+          bulk_copy_s2s(cluster_map(base + rank * rpc * kRowBytes, sw), base + C::kRingV + sw * rpc * kRowBytes,
+                        static_cast<uint32_t>(rows_of(sw) * kRowBytes), cluster_map(RECV, sw));
         asm volatile("cp.async.bulk.commit_group;" ::: "memory");
       }
       __syncwarp();
@@ -835,15 +989,13 @@ __global__ void __launch_bounds__(kThreads, 1)
       for (int idx = st; idx < my_rows * 16; idx += kSoftThreads) {
         const int row = mrow0 + (idx >> 4), c = idx & 15, p = mblock * kR + row;
         if (p >= a.M) continue;
-        *reinterpret_cast<uint4*>(a.qw + q_off(p) + c * 8) = *reinterpret_cast<const uint4*>(
-            smem + C::kOffQ + (c >> 3) * C::kQHalf + row * 128 + (((c & 7) ^ (row & 7)) << 4));
+        *reinterpret_cast<uint4*>(a.qw + q_off(p) + c * 8) =
+            *reinterpret_cast<const uint4*>(smem + C::kOffQ + swz(row, c, C::kQHalf));
       }
       if (last_rank && a.n_mblocks > 1 && *s_kvlast != 0) {
-        if (st < a.R * 16) {
-          const int i = st >> 4, c = st & 15;
-          *reinterpret_cast<uint4*>(a.k_new + kv_row) = *reinterpret_cast<const uint4*>(
-              smem + C::kOffNewK + (c >> 3) * kNewHalf + i * 128 + (((c & 7) ^ (i & 7)) << 4));
-        }
+        if (st < a.R * 16)
+          *reinterpret_cast<uint4*>(a.k_new + kv_row) =
+              *reinterpret_cast<const uint4*>(smem + C::kOffNewK + swz(st >> 4, st & 15, C::kNewHalf));
         if (st == 0) a.kv_ticket[b * a.Hkv + kvh] = 0;  // re-armed
       }
     }
@@ -851,54 +1003,60 @@ __global__ void __launch_bounds__(kThreads, 1)
       // ---- merge of the rows this CTA owns, a warp a row, four d a lane; slot
       // c * rpc + r came from rank c. Unless some rank ran its range again all
       // references are 0 and the partials add.
-      mbar_wait(RECV, 0);
       const float* recv = reinterpret_cast<const float*>(smem);
+      const int cstep = rpc * kRowF;
 #pragma unroll 1
-      for (int r = warp - kFirstSoft; r < my_rows; r += kSoftWarps) {
+      for (int r = sw; r < my_rows; r += kSoftWarps) {
         const float* part = recv + r * kRowF;
+        const int p = mblock * kR + mrow0 + r;
+        __nv_bfloat16* dst = a.out + q_off(p) + lane * 4;
+        if (r == sw) mbar_wait(RECV, 0);
         float4 ov = make_float4(0.f, 0.f, 0.f, 0.f);
         float l = 0.f;
-        bool same = true;
+        // the ranks' row sums and references, one a lane: element lane & 15 of every
+        // second rank (8: the reference; 0..7 and 9: sums)
+        const int e = lane & 15;
+        bool moved = false;
+#pragma unroll 2
+        for (int c = lane >> 4; c < csize; c += 2) {
+          const float x = part[c * cstep + kRowL + (e < 10 ? e : 0)];
+          moved |= e == 8 && x != 0.f;
+          l += e < 10 && e != 8 ? x : 0.f;
+        }
 #pragma unroll 4
         for (int c = 0; c < csize; ++c) {
-          const float* pc = part + c * rpc * kRowF;
-          const float4 x = reinterpret_cast<const float4*>(pc)[lane];
-          const float4 l0 = *reinterpret_cast<const float4*>(pc + kRowL);
-          const float4 l1 = *reinterpret_cast<const float4*>(pc + kRowL + 4);
-          same = same && pc[kRowM] == 0.f;
+          const float4 x = reinterpret_cast<const float4*>(part + c * cstep)[lane];
           ov.x += x.x, ov.y += x.y, ov.z += x.z, ov.w += x.w;
-          l += ((l0.x + l0.y) + (l0.z + l0.w)) + ((l1.x + l1.y) + (l1.z + l1.w));
         }
-        if (!same) {
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) l += __shfl_xor_sync(0xffffffffu, l, o);
+        if (__builtin_expect(__any_sync(0xffffffffu, moved), 0)) {
           // weigh every partial by its own reference (those without a key count for nothing)
+          auto sums = [&](const float* pc) {
+            float x = pc[kRowM + 1];
+            for (int e = 0; e < 8; ++e) x += pc[kRowL + e];
+            return x;
+          };
           float m = -INFINITY;
           ov = make_float4(0.f, 0.f, 0.f, 0.f);
           l = 0.f;
 #pragma unroll 1
-          for (int pass = 0; pass < 2; ++pass)
+          for (int c = 0; c < csize; ++c)
+            if (sums(part + c * cstep) > 0.f) m = fmaxf(m, part[c * cstep + kRowM]);
 #pragma unroll 1
-            for (int c = 0; c < csize; ++c) {
-              const float* pc = part + c * rpc * kRowF;
-              float lc = 0.f;
-              for (int e = 0; e < 8; ++e) lc += pc[kRowL + e];
-              if (!(lc > 0.f)) {
-                if (lc != lc) l = lc;  // NaN reaches the row
-                continue;
-              }
-              if (pass == 0) {
-                m = fmaxf(m, pc[kRowM]);
-                continue;
-              }
-              const float w = ex2(pc[kRowM] - m);
-              const float4 x = reinterpret_cast<const float4*>(pc)[lane];
-              ov.x = fmaf(w, x.x, ov.x), ov.y = fmaf(w, x.y, ov.y), ov.z = fmaf(w, x.z, ov.z), ov.w = fmaf(w, x.w, ov.w);
-              l = fmaf(w, lc, l);
-            }
+          for (int c = 0; c < csize; ++c) {
+            const float* pc = part + c * cstep;
+            const float lc = sums(pc);
+            if (lc == 0.f) continue;
+            const float w = ex2(pc[kRowM] - m);
+            const float4 x = reinterpret_cast<const float4*>(pc)[lane];
+            ov.x = fmaf(w, x.x, ov.x), ov.y = fmaf(w, x.y, ov.y), ov.z = fmaf(w, x.z, ov.z), ov.w = fmaf(w, x.w, ov.w);
+            l = fmaf(w, lc, l);
+          }
         }
-        const int p = mblock * kR + mrow0 + r;
         if (valid && p < a.M && l > 0.f) {
           const float inv_l = 1.f / l;
-          *reinterpret_cast<uint2*>(a.out + q_off(p) + lane * 4) =
+          *reinterpret_cast<uint2*>(dst) =
               make_uint2(cvt_bf16x2(ov.x * inv_l, ov.y * inv_l), cvt_bf16x2(ov.z * inv_l, ov.w * inv_l));
         }
       }
@@ -912,9 +1070,8 @@ __global__ void __launch_bounds__(kThreads, 1)
 // ------------------------------------------------------------------ host
 template <int kR>
 bool set_attributes(const int* sizes, int n, int* active) {
-  const void* kerns[3] = {reinterpret_cast<const void*>(verify_wide_kernel<kR, 1>),
-                          reinterpret_cast<const void*>(verify_wide_kernel<kR, 2>),
-                          reinterpret_cast<const void*>(verify_wide_kernel<kR, 3>)};
+  const void* kerns[2] = {reinterpret_cast<const void*>(verify_wide_kernel<kR, false>),
+                          reinterpret_cast<const void*>(verify_wide_kernel<kR, true>)};
   constexpr int smem = Cfg<kR>::kSmemBytes;
   for (const void* k : kerns)
     if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess ||
@@ -935,7 +1092,7 @@ bool set_attributes(const int* sizes, int n, int* active) {
     cfg.attrs = attr;
     cfg.numAttrs = 1;
     int m = 0;
-    if (cudaOccupancyMaxActiveClusters(&m, kerns[1], &cfg) != cudaSuccess) {
+    if (cudaOccupancyMaxActiveClusters(&m, kerns[0], &cfg) != cudaSuccess) {
       (void)cudaGetLastError();
       m = 0;
     }
@@ -944,7 +1101,7 @@ bool set_attributes(const int* sizes, int n, int* active) {
   return true;
 }
 
-template <int kR, int kMode>
+template <int kR, bool kFused>
 sd_status launch(const sd_kv_cache* cache, const TcArgs& a, const RopeTable& tab, int cs, cudaStream_t stream) {
   const int B = cache->batch, Hkv = cache->n_kv_heads, cap = cache->capacity;
   CUtensorMap k128, v128;
@@ -964,32 +1121,32 @@ sd_status launch(const sd_kv_cache* cache, const TcArgs& a, const RopeTable& tab
   cfg.stream = stream;
   cfg.attrs = attr;
   cfg.numAttrs = 2;
-  if (cudaLaunchKernelEx(&cfg, verify_wide_kernel<kR, kMode>, k128, v128, a, tab) != cudaSuccess) {
+  if (cudaLaunchKernelEx(&cfg, verify_wide_kernel<kR, kFused>, k128, v128, a, tab) != cudaSuccess) {
     (void)cudaGetLastError();
     return SD_ERR_CUDA;
   }
   return SD_OK;
 }
 
-template <int kMode>
+template <bool kFused>
 sd_status launch_rows(const sd_kv_cache* cache, const TcArgs& a, const RopeTable& tab, int rows, int cs,
                       cudaStream_t stream) {
-  if (rows == 48) return launch<48, kMode>(cache, a, tab, cs, stream);
-  if (rows == 64) return launch<64, kMode>(cache, a, tab, cs, stream);
-  return launch<80, kMode>(cache, a, tab, cs, stream);
+  if (rows == 32) return launch<32, kFused>(cache, a, tab, cs, stream);
+  if (rows == 48) return launch<48, kFused>(cache, a, tab, cs, stream);
+  if (rows == 64) return launch<64, kFused>(cache, a, tab, cs, stream);
+  return launch<80, kFused>(cache, a, tab, cs, stream);
 }
 
 }  // namespace
 
 bool sd_internal_wide_active(int rows, const int* sizes, int n, int* active) {
+  if (rows == 32) return set_attributes<32>(sizes, n, active);
   if (rows == 48) return set_attributes<48>(sizes, n, active);
   if (rows == 64) return set_attributes<64>(sizes, n, active);
   return set_attributes<80>(sizes, n, active);
 }
 
 sd_status sd_internal_wide_launch(const sd_kv_cache* cache, const TcArgs& a, const RopeTable& tab, int rows, int cs,
-                                  int mode, cudaStream_t stream) {
-  if (mode == 1) return launch_rows<1>(cache, a, tab, rows, cs, stream);
-  if (mode == 2) return launch_rows<2>(cache, a, tab, rows, cs, stream);
-  return launch_rows<3>(cache, a, tab, rows, cs, stream);
+                                  bool fused, cudaStream_t stream) {
+  return fused ? launch_rows<true>(cache, a, tab, rows, cs, stream) : launch_rows<false>(cache, a, tab, rows, cs, stream);
 }

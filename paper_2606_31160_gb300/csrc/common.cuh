@@ -44,9 +44,9 @@ sd_status sd_internal_verify_attention_tc(const void* q, const sd_kv_cache* cach
                                           int R, int Hq, float scale_log2, int flags, cudaStream_t stream,
                                           bool* handled);
 // Whether the tcgen05 path serves this shape on the current device: the
-// attention, and the fused layer without the block mask.
+// attention, and the fused layer.
 bool sd_internal_tc_serves(int B, int R, int Hq, int Hkv, int D, int cap);
-bool sd_internal_tc_serves_layer(int B, int R, int Hq, int Hkv, int D, int cap, bool block);
+bool sd_internal_tc_serves_layer(int B, int R, int Hq, int Hkv, int D, int cap);
 
 struct RopeTable;
 // The fused verify layer on the tcgen05 path (attention_tc.cu); *handled is

@@ -72,6 +72,6 @@ extern "C" const char* sd_verify_kernel(int B, int R, int Hq, int Hkv, int D, in
   if (B <= 0 || R <= 0 || Hq <= 0 || Hkv <= 0 || capacity <= 0 || Hq % Hkv || (D != 64 && D != 128) ||
       static_cast<long long>(Hq / Hkv) * R > 128)
     return "unsupported";
-  if (layer) return sd_internal_tc_serves_layer(B, R, Hq, Hkv, D, capacity, layer > 1) ? "tcgen05" : "three kernels";
+  if (layer) return sd_internal_tc_serves_layer(B, R, Hq, Hkv, D, capacity) ? "tcgen05" : "three kernels";
   return sd_internal_tc_serves(B, R, Hq, Hkv, D, capacity) ? "tcgen05" : "mma.sync";
 }

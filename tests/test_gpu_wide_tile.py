@@ -1,4 +1,4 @@
-"""The wide row tiles (48, 64 and 80 packed query rows per KV head, two m-blocks
+"""The row tiles (32, 48, 64 and 80 packed query rows per KV head, two m-blocks
 above 80) against the float64 oracle: every edge of the tile choice, prefixes
 around the 32-key split and the 128-key tile, causal and block masks, the fused
 layer and the attention; and the second pass of a CTA whose row sums leave the
@@ -43,8 +43,8 @@ def _run(q, k, v, k_new, v_new, prefix, fused, block):
     assert np.isfinite(to64(out)).all() and attn_within(to64(out), ref), np.abs(to64(out) - ref).max()
 
 
-# (G, R): 33, 48 | 49, 64 | 65, 68, 80 | 81, 96 | 98, 128 packed rows, up to 31 new rows
-@pytest.mark.parametrize("G,R", [(11, 3), (4, 12), (7, 7), (4, 16), (5, 13), (4, 17), (16, 5), (27, 3), (6, 16), (7, 14),
+# (G, R): 1, 4, 17, 30, 32 (17, 31 new rows: past the 32-row tile's 16) | 33, 48 | 49, 64 | 65, 68, 80 | 81, 96 | 98, 128 packed rows, up to 31 new rows
+@pytest.mark.parametrize("G,R", [(1, 1), (4, 1), (17, 1), (2, 15), (4, 8), (2, 16), (1, 17), (1, 31), (11, 3), (4, 12), (7, 7), (4, 16), (5, 13), (4, 17), (16, 5), (27, 3), (6, 16), (7, 14),
                                  (4, 31), (8, 16)])
 @pytest.mark.parametrize("fused,block", [(True, False), (True, True), (False, False)])
 def test_tile_edges(G, R, fused, block):
@@ -58,7 +58,7 @@ def test_tile_edges(G, R, fused, block):
 
 # the score (log2) around which a third of the keys, or all, lie: far outside the
 # range on either side, and just inside it
-@pytest.mark.parametrize("G,R", [(6, 8), (8, 8), (4, 17)])
+@pytest.mark.parametrize("G,R", [(4, 1), (4, 8), (6, 8), (8, 8), (4, 17)])
 @pytest.mark.parametrize("level", [-150.0, 100.0, -70.0, 55.0])
 @pytest.mark.parametrize("part", [1, 3])
 @pytest.mark.parametrize("cluster", [0, 1, 4])
