@@ -166,8 +166,10 @@ size_t sd_verify_attention_workspace(int B, int R, int Hq, int Hkv, int D, int c
  * SD_DEVERR_LENGTH and its output is left unwritten. The first call per
  * device and shape should come before any stream capture (it sets kernel
  * attributes and queries the occupancy).
- * Kernel choice is by shape: head_dim 128 with G*R <= 128 takes the tcgen05
- * kernel, every other shape the mma.sync kernel (sd_verify_kernel names it). A test-only override exists:
+ * Kernel choice is by shape: head_dim 128, and head_dim 64 with up to 31 new
+ * rows, take the tcgen05 kernels, every other shape the mma.sync kernel
+ * (sd_verify_kernel names it; the workspace size does not depend on it for
+ * head_dim 64). A test-only override exists:
  * the environment variable SD_ATTENTION_KERNEL=mma, read once per process,
  * sends every shape to the mma.sync kernel so that tests can compare the two
  * kernels on the same inputs; production callers leave it unset.

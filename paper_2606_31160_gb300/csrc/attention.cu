@@ -1,5 +1,6 @@
 // K3: verify attention of the K + 1 new rows against the cached prefix
-// (Eq. verify, Sec. 3.2), GQA, causal, bf16 in / bf16 out, fp32 softmax.
+// (Eq. verify, Sec. 3.2), GQA, causal, bf16 in / bf16 out, fp32 softmax, for the
+// shapes that the tcgen05 kernels do not take (head dim 64 with more than 31 new rows).
 //
 // Work decomposition (one launch):
 //   * A "unit" is (scene b, KV head g, block of packed query rows). The G
@@ -782,7 +783,9 @@ static sd_status check_shape(int B, int R, int Hq, int Hkv, int D, int cap) {
 
 extern "C" size_t sd_verify_attention_workspace(int B, int R, int Hq, int Hkv, int D, int capacity) {
   if (check_shape(B, R, Hq, Hkv, D, capacity) != SD_OK || B == 0) return 0;
-  if (sd_internal_tc_serves(B, R, Hq, Hkv, D, capacity)) return 0;
+  // (the size is the mma.sync kernel's for every head_dim-64 shape, whichever kernel
+  // then serves it: callers size and keep their workspaces by it)
+  if (D == 128 && sd_internal_tc_serves(B, R, Hq, Hkv, D, capacity)) return 0;
   Plan p;
   if (!make_plan(B, R, Hq, Hkv, D, capacity, &p)) return 0;
   return p.ws_bytes;
@@ -811,15 +814,22 @@ extern "C" sd_status sd_verify_attention_ex(const void* q, const sd_kv_cache* ca
   const float sc = scale > 0.f ? scale : static_cast<float>(1.0 / sqrt(static_cast<double>(D)));
   const float scale_log2 = static_cast<float>(static_cast<double>(sc) * 1.4426950408889634);
   cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
-  {
-    bool handled = false;
-    const sd_status s = sd_internal_verify_attention_tc(q, cache, out, R, Hq, scale_log2, flags, st, &handled);
+  const auto tc = [&](bool* handled) {
+    return sd_internal_verify_attention_tc(q, cache, out, R, Hq, scale_log2, flags, st, handled);
+  };
+  bool handled = false;
+  if (D == 128) {
+    const sd_status s = tc(&handled);
     if (handled) return s;
   }
   Plan p;
   if (!make_plan(B, R, Hq, Hkv, D, cap, &p)) return SD_ERR_CUDA;
   if (p.ws_bytes > 0 && (!workspace || ws_bytes < p.ws_bytes || !sd_aligned16(workspace)))
     return SD_ERR_WORKSPACE;
+  if (D == 64) {
+    const sd_status s = tc(&handled);
+    if (handled) return s;
+  }
   CUtensorMap tk, tv;
   if (!make_kv_map(&tk, cache->k, D, cap, B * Hkv) || !make_kv_map(&tv, cache->v, D, cap, B * Hkv))
     return SD_ERR_CUDA;

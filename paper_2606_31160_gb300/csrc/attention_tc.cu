@@ -1,5 +1,5 @@
 // K3 on the 5th-generation tensor cores (tcgen05 + TMEM), and the choice of
-// kernel for head_dim 128: verify attention of the K + 1 new rows against the
+// tcgen05 kernel: verify attention of the K + 1 new rows against the
 // cached prefix (Eq. verify, Sec. 3.2) and the fused verify layer (M-RoPE of
 // Sec. 3.3 / Sec. 4.2 + the KV append of Eq. commit + the attention).
 //
@@ -726,9 +726,10 @@ constexpr int kNumClusterSizes = 6;
 constexpr int kClusterSizes[kNumClusterSizes] = {1, 2, 4, 6, 8, 16};
 
 // The row tiles: 32, 48, 64 and 80 packed rows of attention_wide.cu (the new rows
-// beside the prefix loop), 64 of this file's kernel (every key in the loop).
-enum Tile { kWide32 = 0, kWide48, kWide64, kWide80, kAll64, kNumTiles };
-constexpr int kTileRows[kNumTiles] = {32, 48, 64, 80, 64};
+// beside the prefix loop) for head dims 128 and 64, 64 of this file's kernel (every
+// key in the loop).
+enum Tile { kWide32 = 0, kWide48, kWide64, kWide80, kWideTiles, kAll64 = 2 * kWideTiles, kNumTiles };
+constexpr int kTileRows[kWideTiles] = {32, 48, 64, 80};
 
 // per device: how many clusters of each size fit at once, for each row tile
 struct DevState {
@@ -778,8 +779,9 @@ DevState* state() {
     s.ready = true;
     const void* all64[1] = {reinterpret_cast<const void*>(verify_attn_tc_kernel<64>)};
     s.ok = set_attributes(all64, 1, Cfg<64>::kSmemBytes, s.active[kAll64]);
-    for (int i = kWide32; i <= kWide80; ++i)
-      s.ok = s.ok && sd_internal_wide_active(kTileRows[i], kClusterSizes, kNumClusterSizes, s.active[i]);
+    for (int i = 0; i < 2 * kWideTiles; ++i)
+      s.ok = s.ok && sd_internal_wide_active(kTileRows[i % kWideTiles], i < kWideTiles ? 128 : 64, kClusterSizes,
+                                             kNumClusterSizes, s.active[i]);
   }
   return &s;
 }
@@ -818,8 +820,7 @@ static bool tc_enabled() {
 // How the tcgen05 path runs a shape: row tile, its packed rows, m-blocks (row
 // tiles per KV head) and cluster size; cs == 0: not served.
 struct TcPlan {
-  Tile tile = kWide32;
-  int rows = 0, mblocks = 0, cs = 0;
+  int tile = kWide32, rows = 0, mblocks = 0, cs = 0;
 };
 
 // Cluster size forced by sd_set_cluster_size (0: chosen per call).
@@ -844,7 +845,7 @@ extern "C" sd_status sd_set_cluster_size(int cluster_size) {
 // (all_keys). The 32-row tile holds 16 new rows.
 static TcPlan tc_plan(int B, int R, int Hq, int Hkv, int D, int cap, bool all_keys) {
   TcPlan p;
-  if (!tc_enabled() || D != kD || Hkv <= 0 || Hq % Hkv || R <= 0) return p;
+  if (!tc_enabled() || (D != kD && (D != 64 || all_keys)) || Hkv <= 0 || Hq % Hkv || R <= 0) return p;
   const int M = (Hq / Hkv) * R;
   if (M > 2 * 64) return p;
   if (all_keys) {
@@ -853,7 +854,8 @@ static TcPlan tc_plan(int B, int R, int Hq, int Hkv, int D, int cap, bool all_ke
     if (R > 31) return p;
     p.tile = M <= 32 && R <= 16 ? kWide32 : (M <= 48 ? kWide48 : (M <= 64 ? kWide64 : (M <= 80 ? kWide80 : (M <= 96 ? kWide48 : kWide64))));
   }
-  p.rows = kTileRows[p.tile];
+  p.rows = all_keys ? 64 : kTileRows[p.tile];
+  if (!all_keys && D == 64) p.tile += kWideTiles;
   DevState* s = state();
   if (!s || !s->ok) return p;
   p.mblocks = (M + p.rows - 1) / p.rows;
@@ -866,11 +868,11 @@ static TcPlan tc_plan(int B, int R, int Hq, int Hkv, int D, int cap, bool all_ke
 }
 
 bool sd_internal_tc_serves(int B, int R, int Hq, int Hkv, int D, int cap) {
-  return tc_plan(B, R, Hq, Hkv, D, cap, true).cs > 0;
+  return tc_plan(B, R, Hq, Hkv, D, cap, D == kD).cs > 0;
 }
 
 bool sd_internal_tc_serves_layer(int B, int R, int Hq, int Hkv, int D, int cap) {
-  return tc_plan(B, R, Hq, Hkv, D, cap, false).cs > 0;
+  return D == kD && tc_plan(B, R, Hq, Hkv, D, cap, false).cs > 0;
 }
 
 template <int kR>
@@ -898,8 +900,7 @@ static sd_status launch_tc(const sd_kv_cache* cache, const TcArgs& a, const TcPl
   return SD_OK;
 }
 
-// Routed here by sd_verify_attention for head_dim 128 and G * R <= 128. Up to
-// 31 new rows take the wide tiles, whose loop covers the prefix only, with the
+// Routed here by sd_verify_attention for G * R <= 128. Up to 31 new rows take the wide tiles, whose loop covers the prefix only, with the
 // prefix optionally streamed before the dependency wait (SD_ATTN_PREFIX_EARLY);
 // more take the kernel whose loop covers every key (the flag is then a promise it
 // does not need).
@@ -931,7 +932,7 @@ sd_status sd_internal_verify_attention_tc(const void* q, const sd_kv_cache* cach
   *handled = true;
   if (!all_keys) {
     RopeTable tab = {};
-    a.early = (early ? 1 : 0) | (block ? 2 : 0);
+    a.early = (early && cache->head_dim == kD ? 1 : 0) | (block ? 2 : 0);  // (the flag is for head dim 128)
     // a programmatic dependent launch either way: without the flag the kernel
     // waits before its first global access, so only its launch and set-up
     // (barriers, tensor memory) overlap the kernel before it
@@ -948,6 +949,7 @@ sd_status sd_internal_verify_layer_tc(void* q, void* k_new, const void* v_new, c
                                       int block, cudaStream_t stream, bool* handled) {
   *handled = false;
   const int B = cache->batch, Hkv = cache->n_kv_heads;
+  if (cache->head_dim != kD) return SD_OK;
   const TcPlan plan = tc_plan(B, R, Hq, Hkv, cache->head_dim, cache->capacity, false);
   if (plan.cs <= 0) return SD_OK;
   TcArgs a = {};

@@ -1,6 +1,6 @@
 // The verify attention and the fused verify layer (Eq. verify, Sec. 3.2; the
-// rotations of Sec. 3.3 / 4.2, the append of Eq. commit) for head dim 128 and up to
-// 31 new rows, on the 5th-generation tensor cores (tcgen05 + TMEM).
+// rotations of Sec. 3.3 / 4.2, the append of Eq. commit) for up to 31 new rows, head
+// dim 128 and (the attention) 64, on the 5th-generation tensor cores (tcgen05 + TMEM).
 //
 // The packed query rows of a KV head (G * R) are few, so both products run
 // transposed, the 128-wide dimension on the MMA's M side:
@@ -17,6 +17,11 @@
 // ~0.4 us of products each, the exchange (~0.7 us), the merge (target layer
 // 6.77 -> 6.27 us, K = 8 10.0 -> 7.8, K = 16 block 15.9 -> 11.4, draft step 6.8 -> 6.1
 // on one cache).
+//
+// Head dim 64 (the attention; its layers run as the rotation, append and attention
+// kernels) is the same kernel with half rows and 16-bit weights: 5 scenes, 28 query
+// heads on 4, L = 4099, K = 5: 15.3 -> 9.6 us against the mma.sync kernel, the tiny
+// layer's 256 keys 7.3 -> 4.3.
 //
 // The new rows stay out of the loop: the cluster's last rank holds the R (rotated)
 // new keys and values in shared memory, scores them by mma.sync, 8 rows by 16 keys a
@@ -51,7 +56,6 @@ namespace {
 
 constexpr int kStageKeys = 128;
 constexpr int kHalf = kStageKeys * 128;  // one 64-column half of a 128-key tile (16 KB)
-constexpr int kKV = 2 * kHalf;           // one K (or V) tile (32 KB)
 constexpr int kSoftWarps = 16;
 constexpr int kSoftThreads = 32 * kSoftWarps;
 constexpr int kFirstSoft = 3;            // the first softmax warp
@@ -59,18 +63,17 @@ constexpr int kSoft0 = 32 * kFirstSoft;  // the first softmax thread
 constexpr int kThreads = kSoft0 + kSoftThreads;
 constexpr float kHigh = 18446744073709551616.f;          // 2^64: a larger row sum runs the range again
 constexpr float kLow = 8.271806125530277e-25f;           // 2^-80: a smaller one too
-// a partial row sent to its owner: [O(128) | prefix row sums by softmax group and
-// lane quarter (8) | reference | new keys' row sum | 2 pad] fp32 (560 bytes)
-constexpr int kRowL = kD;
-constexpr int kRowM = kD + 8;
-constexpr int kRowF = kD + 12;
-constexpr int kRowBytes = kRowF * 4;
-
-template <int kR>
+template <int kR, int kDim>
 struct Cfg {
   static_assert(kR == 32 || kR == 48 || kR == 64 || kR == 80, "row tile");
+  static_assert(kDim == 64 || kDim == 128, "head dim");
   static constexpr int kRpt = kR / 2;                   // rows of a softmax thread in its tile
-  static constexpr int kStages = kR == 32 ? 3 : 2;      // K slots, and V slots
+  static constexpr int kHalves = kDim / 64;             // 64-column halves of a row
+  static constexpr int kChunks = kDim / 8;              // 16-byte chunks of a row
+  static constexpr int kKV = kHalves * kHalf;           // one K (or V) tile of 128 keys
+  // K slots, and V slots: at most 3, as the producer's wait for S(T - kStages) must see
+  // its phase before S(T - kStages + 3) completes the next one of that S buffer
+  static constexpr int kStages = kDim == 64 || kR == 32 ? 3 : 2;
   static constexpr int kMaxNew = kR == 32 ? 16 : 32;    // new rows held in shared memory
   static constexpr int kNewHalf = kMaxNew * 128;        // one 64-column half of the new key (value) rows
   static constexpr int kRingV = kStages * kKV;
@@ -80,19 +83,25 @@ struct Cfg {
   // 16-row groups kPGroup apart
   static constexpr int kPGroup = kStageKeys * 32;
   static constexpr int kP = (kR / 16) * kPGroup;
+  // head dim 64 keeps the weights to 16 bits as two bf16 terms (two PV products): the
+  // mma.sync kernel that served it rounds weights below a running maximum, which is
+  // 14% closer to 64 bits than one term without a reference (2.1e-3 against 2.4e-3)
+  static constexpr bool kSplit = kDim == 64;
+  static constexpr int kPBuf = kSplit ? 2 * kP : kP;  // a group's P buffer: the high terms, then the low ones
   static constexpr int kSStride = kR == 32 ? 32 : (kR <= 64 ? 64 : 128);  // columns between S0 | S1 | S2 | O
   static constexpr int kTmemCols = 4 * kSStride;
   // shared memory (offsets from the 1024-aligned base)
   static constexpr int kOffNewK = kRing;
-  static constexpr int kOffNewV = kOffNewK + 2 * kNewHalf;
-  static constexpr int kOffQ = kOffNewV + 2 * kNewHalf;
-  static constexpr int kOffP = kOffQ + 2 * kQHalf;
+  static constexpr int kOffNewV = kOffNewK + kHalves * kNewHalf;
+  static constexpr int kOffQ = kOffNewV + kHalves * kNewHalf;
+  static constexpr int kOffP = kOffQ + kHalves * kQHalf;
   // the new keys' weights: on the 32-row tile, which has no room for more, in P
   // buffer 1 ahead of its first tile; on the others beside it, in the same layout
   static constexpr bool kNewFirst = kR == 32;
-  static constexpr int kOffPNew = kNewFirst ? kOffP + kP : kOffP + 2 * kP;
+  static constexpr int kOffPNew = kOffP + (kNewFirst ? kPBuf : 2 * kPBuf);
   static constexpr int kPNewGroup = kNewFirst ? kPGroup : kMaxNew * 32;
-  static constexpr int kOffBar = kNewFirst ? kOffP + 2 * kP : kOffPNew + (kR / 16) * kPNewGroup;
+  static constexpr int kPNewLow = kNewFirst ? kP : (kR / 16) * kPNewGroup;  // from the high to the low terms
+  static constexpr int kOffBar = kNewFirst ? kOffP + 2 * kPBuf : kOffPNew + (kSplit ? 2 : 1) * kPNewLow;
   // full_k[S] full_v[S] p_full[2] s_ready[3] s_free[3] pv_done[S] p_new new_done recv decide maxima tmem_done
   static constexpr int kNumBars = 3 * kStages + 14;
   static constexpr int kOffMisc = round_up(kOffBar + kNumBars * 8, 16);
@@ -102,8 +111,14 @@ struct Cfg {
   static constexpr int kSmemBytes = kOffSum + kR * 32 + 1024;
   static_assert(kSmemBytes <= 227 * 1024, "shared memory budget");
   static_assert(kOffNewV % 1024 == 0 && kOffQ % 1024 == 0 && kOffP % 1024 == 0 && kQHalf % 1024 == 0, "swizzle atoms");
-  static_assert(kMaxNew * 64 * 8 <= 2 * kP, "rotation table fits the P buffers");
+  static_assert(kMaxNew * (kDim / 2) * 8 <= 2 * kP, "rotation table fits the P buffers");
   static_assert(kR * 128 * 4 <= 2 * kP, "row maxima fit the P buffers");
+  // a partial row sent to its owner: [O(kDim) | prefix row sums by softmax group and
+  // lane quarter (8) | reference | new keys' row sum | 2 pad] fp32 (560 or 304 bytes)
+  static constexpr int kRowL = kDim;
+  static constexpr int kRowM = kDim + 8;
+  static constexpr int kRowF = kDim + 12;
+  static constexpr int kRowBytes = kRowF * 4;
   // cluster merge: incoming rows in the K ring (free after the last S), this
   // CTA's in the V ring (free after the last PV). ceil(n / c) * c < n + 16
   static_assert((kR + 15) * kRowBytes <= kRingV && kR * kRowBytes <= kRing - kRingV, "merge buffers");
@@ -148,12 +163,25 @@ __device__ __forceinline__ uint64_t add2(uint64_t a, uint64_t b) {
   return d;
 }
 
-// Weights of kN rows of one key: P = 2^(S * scale - ref) in bf16 (0 for a key out
-// of the range, whatever its score, NaN included), the row sums advanced by the
-// same rounded weights.
-template <int kN>
+// Two weights as bf16 terms: the high ones, and with kSplit what rounding left.
+// l: the weights that the terms stand for.
+template <bool kSplit>
+__device__ __forceinline__ void weight_terms(float e0, float e1, uint32_t& hi, uint32_t& lo, uint64_t& l) {
+  hi = cvt_bf16x2(e0, e1);
+  if (kSplit) {
+    lo = cvt_bf16x2(e0 - sd_bf16_lo(hi), e1 - sd_bf16_hi(hi));
+    l = pack2f(e0, e1);
+  } else {
+    l = pack2(hi << 16, hi & 0xffff0000u);
+  }
+}
+
+// Weights of kN rows of one key: P = 2^(S * scale - ref) in bf16 terms (0 for a key
+// out of the range, whatever its score, NaN included), the row sums advanced by the
+// same weights.
+template <int kN, bool kSplit>
 __device__ __forceinline__ void weights_to_p(const uint32_t (&r)[kN], const float* nref, uint64_t sl2, bool key_ok,
-                                             uint64_t* lp2, uint32_t (&pw)[kN / 2]) {
+                                             uint64_t* lp2, uint32_t (&pw)[kN / 2], uint32_t (&pl)[kN / 2]) {
 #pragma unroll
   for (int j = 0; j < kN; j += 4) {
     const float4 nr = *reinterpret_cast<const float4*>(nref + j);
@@ -161,9 +189,17 @@ __device__ __forceinline__ void weights_to_p(const uint32_t (&r)[kN], const floa
     for (int e = 0; e < 2; ++e) {
       float y0, y1;
       unpack2(fma2(pack2(r[j + 2 * e], r[j + 2 * e + 1]), sl2, e == 0 ? pack2f(nr.x, nr.y) : pack2f(nr.z, nr.w)), y0, y1);
-      const uint32_t w = key_ok ? cvt_bf16x2(ex2(y0), ex2(y1)) : 0u;
-      pw[j / 2 + e] = w;
-      lp2[j / 2 + e] = add2(lp2[j / 2 + e], pack2(w << 16, w & 0xffff0000u));
+      uint32_t hi, lo = 0;
+      uint64_t l;
+      if (kSplit) {
+        weight_terms<true>(key_ok ? ex2(y0) : 0.f, key_ok ? ex2(y1) : 0.f, hi, lo, l);
+      } else {
+        hi = key_ok ? cvt_bf16x2(ex2(y0), ex2(y1)) : 0u;
+        l = pack2(hi << 16, hi & 0xffff0000u);
+      }
+      pw[j / 2 + e] = hi;
+      pl[j / 2 + e] = lo;
+      lp2[j / 2 + e] = add2(lp2[j / 2 + e], l);
     }
   }
 }
@@ -210,17 +246,21 @@ __device__ __forceinline__ uint32_t swz(int r, int c, int half) {
 
 // A row's largest score against the new keys it sees (the range is run again:
 // out of line). One warp; qrow / krow0: the packed query row and new key row 0.
+template <int kDim>
 __device__ __noinline__ float new_key_max(const uint8_t* q, int row, int q_half, const uint8_t* k, int k_half, int last,
                                           float sl, int lane) {
-  const int c = lane >> 1, e = (lane & 1) * 8;  // 4 d a lane
-  const uint2 qw = *reinterpret_cast<const uint2*>(q + swz(row, c, q_half) + e);
+  constexpr int kPer = kDim / 32;  // d a lane: 4 or 2
+  const int c = lane * kPer / 8, e = lane * kPer % 8 * 2;
+  const uint32_t* qw = reinterpret_cast<const uint32_t*>(q + swz(row, c, q_half) + e);
   float m = -INFINITY;
   for (int n = 0; n <= last; ++n) {
-    const uint2 kw = *reinterpret_cast<const uint2*>(k + swz(n, c, k_half) + e);
-    float x = sd_bf16_lo(qw.x) * sd_bf16_lo(kw.x);
-    x = fmaf(sd_bf16_hi(qw.x), sd_bf16_hi(kw.x), x);
-    x = fmaf(sd_bf16_lo(qw.y), sd_bf16_lo(kw.y), x);
-    x = fmaf(sd_bf16_hi(qw.y), sd_bf16_hi(kw.y), x);
+    const uint32_t* kw = reinterpret_cast<const uint32_t*>(k + swz(n, c, k_half) + e);
+    float x = 0.f;
+#pragma unroll
+    for (int j = 0; j < kPer / 2; ++j) {
+      x = fmaf(sd_bf16_lo(qw[j]), sd_bf16_lo(kw[j]), x);
+      x = fmaf(sd_bf16_hi(qw[j]), sd_bf16_hi(kw[j]), x);
+    }
     for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
     m = fmaxf(m, x * sl);
   }
@@ -233,11 +273,13 @@ __device__ __noinline__ float new_key_max(const uint8_t* q, int row, int q_half,
 // and pos may be read before the dependency wait; bit 1: the block mask. Grid:
 // (cluster size, Hkv * n_mblocks, B); m-block mb takes packed rows mb * kR ..
 // mb * kR + kR - 1.
-template <int kR, bool kFused>
+template <int kR, int kDim, bool kFused>
 __global__ void __launch_bounds__(kThreads, 1)
     verify_wide_kernel(const __grid_constant__ CUtensorMap tm_k128, const __grid_constant__ CUtensorMap tm_v128,
                        const TcArgs a, const RopeTable tab) {
-  using C = Cfg<kR>;
+  using C = Cfg<kR, kDim>;
+  constexpr int kHalves = C::kHalves, kChunks = C::kChunks, kKV = C::kKV;
+  constexpr int kRowL = C::kRowL, kRowM = C::kRowM, kRowF = C::kRowF, kRowBytes = C::kRowBytes;
   constexpr int kS = C::kStages;
   constexpr int kRpt = C::kRpt;
   constexpr uint32_t kIdescS = umma_idesc(128, kR, 0, 0);
@@ -360,14 +402,14 @@ __global__ void __launch_bounds__(kThreads, 1)
         if (elect_one()) {
           mbar_expect_tx(FULLK(s), static_cast<uint32_t>(kKV));
 #pragma unroll
-          for (int h = 0; h < 2; ++h) tma_load_3d_hint(kst + h * kHalf, &tm_k128, FULLK(s), h * 64, y0, z, evict_first);
+          for (int h = 0; h < kHalves; ++h) tma_load_3d_hint(kst + h * kHalf, &tm_k128, FULLK(s), h * 64, y0, z, evict_first);
         }
         __syncwarp();
         if (t >= kS) mbar_wait(PVDONE(s), parS(T - kS));
         if (elect_one()) {
           mbar_expect_tx(FULLV(s), static_cast<uint32_t>(kKV));
 #pragma unroll
-          for (int h = 0; h < 2; ++h) tma_load_3d_hint(vst + h * kHalf, &tm_v128, FULLV(s), h * 64, y0, z, evict_first);
+          for (int h = 0; h < kHalves; ++h) tma_load_3d_hint(vst + h * kHalf, &tm_v128, FULLV(s), h * 64, y0, z, evict_first);
         }
         __syncwarp();
       }
@@ -387,7 +429,7 @@ __global__ void __launch_bounds__(kThreads, 1)
 #pragma unroll 1
       for (int t = 0; t < n_pre; ++t)
 #pragma unroll
-        for (int h = 0; h < 2; ++h) {
+        for (int h = 0; h < kHalves; ++h) {
           tma_prefetch_3d(&tm_k128, h * 64, key_begin + t * kStageKeys, zl);
           tma_prefetch_3d(&tm_v128, h * 64, key_begin + t * kStageKeys, zl);
         }
@@ -395,10 +437,10 @@ __global__ void __launch_bounds__(kThreads, 1)
 #pragma unroll 1
         for (int i = 0; i < a.R; ++i) {
           const long long row = static_cast<long long>(b) * a.R + i;
-          bulk_prefetch_l2((kFused ? a.qw : a.q) + (row * a.Hq + (a.Hkv - 1) * a.G) * kD, a.G * kD * 2);
+          bulk_prefetch_l2((kFused ? a.qw : a.q) + (row * a.Hq + (a.Hkv - 1) * a.G) * kDim, a.G * kDim * 2);
           if (kFused) {
-            bulk_prefetch_l2(a.k_new + (row * a.Hkv + a.Hkv - 1) * kD, kD * 2);
-            bulk_prefetch_l2(a.v_new + (row * a.Hkv + a.Hkv - 1) * kD, kD * 2);
+            bulk_prefetch_l2(a.k_new + (row * a.Hkv + a.Hkv - 1) * kDim, kDim * 2);
+            bulk_prefetch_l2(a.v_new + (row * a.Hkv + a.Hkv - 1) * kDim, kDim * 2);
           }
         }
     }
@@ -469,7 +511,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         const uint64_t dk = dK0 + static_cast<uint64_t>((s * kKV) >> 4);
         if (elect_one()) {
 #pragma unroll
-          for (int kk = 0; kk < 8; ++kk)
+          for (int kk = 0; kk < kDim / 16; ++kk)
             umma(ts, dk + (((kk >> 2) * kHalf + (kk & 3) * 32) >> 4),
                  dQ + (((kk >> 2) * C::kQHalf + (kk & 3) * 32) >> 4), kIdescS, kk > 0 ? 1 : 0);
           if (t >= 0) umma_commit(SREADY(T % 3));
@@ -489,8 +531,10 @@ __global__ void __launch_bounds__(kThreads, 1)
     const uint32_t tmem_o = *tmem_slot + 3 * C::kSStride;
     ranges(*s_len);
     const bool has_new = valid && last_rank;
-    const uint64_t dV0 = umma_desc(base + C::kRingV, kHalf, 1024);        // V^T: MN-major
-    const uint64_t dN = umma_desc(base + C::kOffNewV, C::kNewHalf, 1024);
+    // V^T: MN-major. Head dim 64 keeps M = 128 with both 64-row halves of the operand
+    // on the same rows (stride 0): O's lanes 64..127 repeat 0..63 and are not read
+    const uint64_t dV0 = umma_desc(base + C::kRingV, kHalves == 2 ? kHalf : 0, 1024);
+    const uint64_t dN = umma_desc(base + C::kOffNewV, kHalves == 2 ? C::kNewHalf : 0, 1024);
     const uint64_t dP0 = umma_desc(base + C::kOffP, C::kPGroup, 256, 6);  // P^T: MN-major, 32-byte swizzle
 #pragma unroll 1
     for (int pass = 0; pass < 3; ++pass) {
@@ -508,8 +552,10 @@ __global__ void __launch_bounds__(kThreads, 1)
         if (elect_one()) {
 #pragma unroll
           for (int kk = 0; kk < C::kMaxNew / 16; ++kk)
-            if (kk * 16 < a.R)
+            if (kk * 16 < a.R) {
               umma(tmem_o, dN + (kk * 2048 >> 4), dpn + (kk * 512 >> 4), kIdescO, kk > 0 || add ? 1 : 0);
+              if (C::kSplit) umma(tmem_o, dN + (kk * 2048 >> 4), dpn + ((C::kPNewLow + kk * 512) >> 4), kIdescO, 1);
+            }
           umma_commit(NEWDONE);
         }
         __syncwarp();
@@ -521,14 +567,16 @@ __global__ void __launch_bounds__(kThreads, 1)
         mbar_wait(FULLV(s), parS(T));
         tc_fence_after();
         const uint64_t dv = dV0 + static_cast<uint64_t>((s * kKV) >> 4);
-        const uint64_t dp = dP0 + static_cast<uint64_t>(((T & 1) * C::kP) >> 4);
+        const uint64_t dp = dP0 + static_cast<uint64_t>(((T & 1) * C::kPBuf) >> 4);
         const int n_steps = pv_keys(t) >> 4;
         if (elect_one()) {
 #pragma unroll
           for (int kk = 0; kk < 8; ++kk)
-            if (kk < n_steps)
+            if (kk < n_steps) {
               umma(tmem_o, dv + (kk * 2048 >> 4), dp + (kk * 512 >> 4), kIdescO,
                    (t > 0 || kk > 0 || (C::kNewFirst && take_new)) ? 1 : 0);
+              if (C::kSplit) umma(tmem_o, dv + (kk * 2048 >> 4), dp + ((C::kP + kk * 512) >> 4), kIdescO, 1);
+            }
           umma_commit(PVDONE(s));
         }
         __syncwarp();
@@ -546,23 +594,23 @@ __global__ void __launch_bounds__(kThreads, 1)
     const int kl = quarter * 32 + lane;  // key lane of S^T / d lane of O^T
     const uint32_t lane_off = static_cast<uint32_t>(quarter * 32) << 16;
     const int row0 = kRpt * half;
-    // this thread's 16-byte chunks: of the packed query tile (row idx >> 4, chunk
-    // idx & 15, rows past M zero) and, in the cluster's last rank, of the new key
+    // this thread's 16-byte chunks: of the packed query tile (row idx / kChunks, chunk
+    // idx % kChunks, rows past M zero) and, in the cluster's last rank, of the new key
     // and value rows
-    constexpr int kQc = (kR * 16 + kSoftThreads - 1) / kSoftThreads;
+    constexpr int kQc = (kR * kChunks + kSoftThreads - 1) / kSoftThreads;
     auto q_off = [&](int p) {
       const int i = gdiv(p);
-      return ((static_cast<long long>(b) * a.R + i) * a.Hq + kvh * a.G + (p - i * a.G)) * kD;
+      return ((static_cast<long long>(b) * a.R + i) * a.Hq + kvh * a.G + (p - i * a.G)) * kDim;
     };
-    const bool new_kv = last_rank && st < a.R * 16;
-    const long long kv_row = ((static_cast<long long>(b) * a.R + (st >> 4)) * a.Hkv + kvh) * kD + (st & 15) * 8;
+    const bool new_kv = last_rank && st < a.R * kChunks;
+    const long long kv_row = ((static_cast<long long>(b) * a.R + (st / kChunks)) * a.Hkv + kvh) * kDim + (st % kChunks) * 8;
     uint4 qv[kQc], kv = make_uint4(0, 0, 0, 0), vv = make_uint4(0, 0, 0, 0);
     auto load_q = [&] {
 #pragma unroll
       for (int u = 0; u < kQc; ++u) {
-        const int idx = st + u * kSoftThreads, p = mblock * kR + (idx >> 4);
-        qv[u] = idx < kR * 16 && p < a.M
-                    ? __ldcg(reinterpret_cast<const uint4*>((kFused ? a.qw : a.q) + q_off(p) + (idx & 15) * 8))
+        const int idx = st + u * kSoftThreads, p = mblock * kR + (idx / kChunks);
+        qv[u] = idx < kR * kChunks && p < a.M
+                    ? __ldcg(reinterpret_cast<const uint4*>((kFused ? a.qw : a.q) + q_off(p) + (idx % kChunks) * 8))
                     : make_uint4(0, 0, 0, 0);
       }
     };
@@ -611,7 +659,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       // overwrites everything it stored (.cg loads: no stale L1 line).
       const bool has_kv = new_kv && valid;
       const long long cache_row =
-          ((static_cast<long long>(b) * a.Hkv + kvh) * a.cap + L_pre + (st >> 4)) * kD + (st & 15) * 8;
+          ((static_cast<long long>(b) * a.Hkv + kvh) * a.cap + L_pre + (st / kChunks)) * kDim + (st % kChunks) * 8;
 #pragma unroll 1
       for (int it = early && !last_cluster ? 0 : 1; it < 2; ++it) {
         if (early) {
@@ -622,8 +670,8 @@ __global__ void __launch_bounds__(kThreads, 1)
         if (!kFused && has_kv) load_kv(a.kc, a.vc, cache_row);
 #pragma unroll
         for (int u = 0; u < kQc; ++u) {
-          const int idx = st + u * kSoftThreads, row = idx >> 4, c = idx & 15, p = mblock * kR + row;
-          if (idx >= kR * 16) break;
+          const int idx = st + u * kSoftThreads, row = idx / kChunks, c = idx % kChunks, p = mblock * kR + row;
+          if (idx >= kR * kChunks) break;
           uint32_t w[4] = {qv[u].x, qv[u].y, qv[u].z, qv[u].w};
           if (kFused && p < a.M) {
             const float2* cs = cs_tab + gdiv(p) * 64 + c * 4;
@@ -632,9 +680,9 @@ __global__ void __launch_bounds__(kThreads, 1)
           }
           st_shared_v4(qs + swz(row, c, C::kQHalf), w[0], w[1], w[2], w[3]);
         }
-        if (last_rank && st < C::kMaxNew * 16) {
+        if (last_rank && st < C::kMaxNew * kChunks) {
           // new key (rotated) and value rows, zero past R
-          const int i = st >> 4, c = st & 15;
+          const int i = st / kChunks, c = st % kChunks;
           uint32_t w[4] = {kv.x, kv.y, kv.z, kv.w};
           if (kFused && has_kv) {
             const float2* cs = cs_tab + i * 64 + c * 4;
@@ -671,7 +719,7 @@ __global__ void __launch_bounds__(kThreads, 1)
 
     const uint64_t sl2 = pack2f(sl, sl);
     uint64_t lp2[kRpt / 2];  // this key lane's row sums, in pairs
-    const uint32_t pbuf = base + C::kOffP + group * C::kP;
+    const uint32_t pbuf = base + C::kOffP + group * C::kPBuf;
     const uint32_t pkey = pbuf + kl * 32;
     const uint32_t psw = (kl >> 2) & 1;  // 32-byte swizzle
     // the last new key that packed row r of this tile sees: row p = i * G + g is
@@ -688,7 +736,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     // weights and P; vb, vpar: the barrier of PV(T - 2)
     auto chunk = [&](auto kn, int T, int sb, int vb, uint32_t vpar, int j0, bool key_ok, bool first) {
       constexpr int kN = decltype(kn)::value;
-      uint32_t r[kN], pw[kN / 2];
+      uint32_t r[kN], pw[kN / 2], pl[kN / 2];
       tmem_ld(tmem + C::kSStride * sb + row0 + j0 + lane_off, r);
       if (j0 + kN == kRpt) {
         // the tile's scores are all in registers: its buffer may take S(T + 3)
@@ -696,7 +744,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         __syncwarp();
         if (lane == 0) mbar_arrive(SFREE(sb));
       }
-      weights_to_p<kN>(r, row_nref + row0 + j0, sl2, key_ok, lp2 + j0 / 2, pw);
+      weights_to_p<kN, C::kSplit>(r, row_nref + row0 + j0, sl2, key_ok, lp2 + j0 / 2, pw, pl);
       if (j0 == 0) {
         // PV(T - 2), or the new keys' product, has read the buffer
         if (T >= 2) mbar_wait(PVDONE(vb), vpar);
@@ -705,8 +753,9 @@ __global__ void __launch_bounds__(kThreads, 1)
 #pragma unroll
       for (int h = 0; h < kN / 8; ++h) {
         const int ch = (row0 + j0) / 8 + h;
-        st_shared_v4(pkey + (ch >> 1) * C::kPGroup + (((ch & 1) ^ psw) << 4), pw[4 * h], pw[4 * h + 1], pw[4 * h + 2],
-                     pw[4 * h + 3]);
+        const uint32_t dst = pkey + (ch >> 1) * C::kPGroup + (((ch & 1) ^ psw) << 4);
+        st_shared_v4(dst, pw[4 * h], pw[4 * h + 1], pw[4 * h + 2], pw[4 * h + 3]);
+        if (C::kSplit) st_shared_v4(dst + C::kP, pl[4 * h], pl[4 * h + 1], pl[4 * h + 2], pl[4 * h + 3]);
       }
     };
     bool redo = false;
@@ -725,14 +774,14 @@ __global__ void __launch_bounds__(kThreads, 1)
       const int lim0 = last_new(r8 + 2 * (lane & 3)), lim1 = last_new(r8 + 2 * (lane & 3) + 1);
       const float2 nr = *reinterpret_cast<const float2*>(row_nref + r8 + 2 * (lane & 3));
       float l0 = 0.f, l1 = 0.f;
-      uint32_t bq[4][4];
+      uint32_t bq[kDim / 32][4];
 #pragma unroll
-      for (int k2 = 0; k2 < 4; ++k2) ldmatrix4(qs + swz(r8 + (lane & 7), 4 * k2 + (lane >> 3), C::kQHalf), bq[k2]);
+      for (int k2 = 0; k2 < kDim / 32; ++k2) ldmatrix4(qs + swz(r8 + (lane & 7), 4 * k2 + (lane >> 3), C::kQHalf), bq[k2]);
 #pragma unroll 1
       for (int m = 0; m * 16 < a.R; ++m) {
         float c[4] = {0.f, 0.f, 0.f, 0.f}, c1[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
-        for (int k2 = 0; k2 < 4; ++k2) {
+        for (int k2 = 0; k2 < kDim / 32; ++k2) {
           uint32_t ak[4], al[4];
           ldmatrix4(base + C::kOffNewK + swz(m * 16 + (lane & 15), 4 * k2 + (lane >> 4), C::kNewHalf), ak);
           ldmatrix4(base + C::kOffNewK + swz(m * 16 + (lane & 15), 4 * k2 + 2 + (lane >> 4), C::kNewHalf), al);
@@ -742,15 +791,20 @@ __global__ void __launch_bounds__(kThreads, 1)
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
           const int key = m * 16 + (lane >> 2) + 8 * h;
-          const uint32_t keep = (key <= lim0 ? 0xffffu : 0u) | (key <= lim1 ? 0xffff0000u : 0u);
-          const uint32_t w = cvt_bf16x2(ex2(fmaf(c[2 * h] + c1[2 * h], sl, nr.x)),
-                                        ex2(fmaf(c[2 * h + 1] + c1[2 * h + 1], sl, nr.y))) & keep;
-          l0 += sd_bf16_lo(w);
-          l1 += sd_bf16_hi(w);
-          asm volatile("st.shared.u32 [%0], %1;" ::"r"(base + C::kOffPNew + (unit >> 1) * C::kPNewGroup + key * 32 +
-                                                        (((unit & 1) ^ ((key >> 2) & 1)) << 4) + (lane & 3) * 4),
-                       "r"(w)
-                       : "memory");
+          // (a masked score may be anything: selected away before it is a weight)
+          const float e0 = key <= lim0 ? ex2(fmaf(c[2 * h] + c1[2 * h], sl, nr.x)) : 0.f;
+          const float e1 = key <= lim1 ? ex2(fmaf(c[2 * h + 1] + c1[2 * h + 1], sl, nr.y)) : 0.f;
+          uint32_t hi, lo = 0;
+          uint64_t l;
+          weight_terms<C::kSplit>(e0, e1, hi, lo, l);
+          float x0, x1;
+          unpack2(l, x0, x1);
+          l0 += x0;
+          l1 += x1;
+          const uint32_t dst = base + C::kOffPNew + (unit >> 1) * C::kPNewGroup + key * 32 +
+                               (((unit & 1) ^ ((key >> 2) & 1)) << 4) + (lane & 3) * 4;
+          asm volatile("st.shared.u32 [%0], %1;" ::"r"(dst), "r"(hi) : "memory");
+          if (C::kSplit) asm volatile("st.shared.u32 [%0], %1;" ::"r"(dst + C::kPNewLow), "r"(lo) : "memory");
         }
       }
       asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
@@ -798,7 +852,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         }
         if ((sb += 2) >= 3) sb -= 3, spar ^= 1;
         if ((vb += 2) >= kS) vb -= kS, vpar ^= 1;
-        if (!key_ok && kl < pv_keys(t)) {
+        if (!key_ok && kl < pv_keys(t) && half < kHalves) {
           // stale or foreign key row that the product reads: zero its V row (this
           // thread's 64-column half) so 0 * NaN cannot reach O, once the tile has
           // landed. Chunks in an order that differs by lane: rows are 128 bytes apart
@@ -890,7 +944,7 @@ __global__ void __launch_bounds__(kThreads, 1)
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
         if (has_new)
-          m = fmaxf(m, new_key_max(smem + C::kOffQ, row, C::kQHalf, smem + C::kOffNewK, C::kNewHalf, last_new(row), sl, lane));
+          m = fmaxf(m, new_key_max<kDim>(smem + C::kOffQ, row, C::kQHalf, smem + C::kOffNewK, C::kNewHalf, last_new(row), sl, lane));
         if (lane == 0) row_nref[row] = m == -INFINITY ? 0.f : -m;
       }
       named_bar_sync(2, kSoftThreads);
@@ -956,12 +1010,13 @@ __global__ void __launch_bounds__(kThreads, 1)
       for (int j = 0; j < kOr; ++j) {
         const int row = orow0 + j, p = mblock * kR + row;
         const float inv_l = row_new[row];
-        if (valid && p < a.M && inv_l > 0.f) a.out[q_off(p) + kl] = __float2bfloat16_rn(__uint_as_float(o[j]) * inv_l);
+        if (valid && p < a.M && inv_l > 0.f && kl < kDim) a.out[q_off(p) + kl] = __float2bfloat16_rn(__uint_as_float(o[j]) * inv_l);
       }
     } else {
       float* send = reinterpret_cast<float*>(smem + C::kRingV);
+      if (kl < kDim)
 #pragma unroll
-      for (int j = 0; j < kOr; ++j) send[(orow0 + j) * kRowF + kl] = __uint_as_float(o[j]);
+        for (int j = 0; j < kOr; ++j) send[(orow0 + j) * kRowF + kl] = __uint_as_float(o[j]);
       if ((lane & 3) == 0)
 #pragma unroll
         for (int c = 0; c < kRpt / 8; ++c) send[(row0 + 8 * c + (lane >> 2)) * kRowF + kRowL + group * 4 + quarter] = lsum[c];
@@ -986,32 +1041,36 @@ __global__ void __launch_bounds__(kThreads, 1)
       // go back to q, and with several m-blocks the head's last reader of the
       // raw key rows writes the rotated ones back to k_new
 #pragma unroll 1
-      for (int idx = st; idx < my_rows * 16; idx += kSoftThreads) {
-        const int row = mrow0 + (idx >> 4), c = idx & 15, p = mblock * kR + row;
+      for (int idx = st; idx < my_rows * kChunks; idx += kSoftThreads) {
+        const int row = mrow0 + (idx / kChunks), c = idx % kChunks, p = mblock * kR + row;
         if (p >= a.M) continue;
         *reinterpret_cast<uint4*>(a.qw + q_off(p) + c * 8) =
             *reinterpret_cast<const uint4*>(smem + C::kOffQ + swz(row, c, C::kQHalf));
       }
       if (last_rank && a.n_mblocks > 1 && *s_kvlast != 0) {
-        if (st < a.R * 16)
+        if (st < a.R * kChunks)
           *reinterpret_cast<uint4*>(a.k_new + kv_row) =
-              *reinterpret_cast<const uint4*>(smem + C::kOffNewK + swz(st >> 4, st & 15, C::kNewHalf));
+              *reinterpret_cast<const uint4*>(smem + C::kOffNewK + swz(st / kChunks, st % kChunks, C::kNewHalf));
         if (st == 0) a.kv_ticket[b * a.Hkv + kvh] = 0;  // re-armed
       }
     }
     if (merge) {
-      // ---- merge of the rows this CTA owns, a warp a row, four d a lane; slot
+      // ---- merge of the rows this CTA owns, a warp a row, kDim / 32 d a lane; slot
       // c * rpc + r came from rank c. Unless some rank ran its range again all
       // references are 0 and the partials add.
       const float* recv = reinterpret_cast<const float*>(smem);
       const int cstep = rpc * kRowF;
+      constexpr int kPer = kDim / 32;
+      struct alignas(kPer * 4) Row {
+        float v[kPer];
+      };
 #pragma unroll 1
       for (int r = sw; r < my_rows; r += kSoftWarps) {
         const float* part = recv + r * kRowF;
         const int p = mblock * kR + mrow0 + r;
-        __nv_bfloat16* dst = a.out + q_off(p) + lane * 4;
+        __nv_bfloat16* dst = a.out + q_off(p) + lane * kPer;
         if (r == sw) mbar_wait(RECV, 0);
-        float4 ov = make_float4(0.f, 0.f, 0.f, 0.f);
+        Row ov = {};
         float l = 0.f;
         // the ranks' row sums and references, one a lane: element lane & 15 of every
         // second rank (8: the reference; 0..7 and 9: sums)
@@ -1025,8 +1084,9 @@ __global__ void __launch_bounds__(kThreads, 1)
         }
 #pragma unroll 4
         for (int c = 0; c < csize; ++c) {
-          const float4 x = reinterpret_cast<const float4*>(part + c * cstep)[lane];
-          ov.x += x.x, ov.y += x.y, ov.z += x.z, ov.w += x.w;
+          const Row x = reinterpret_cast<const Row*>(part + c * cstep)[lane];
+#pragma unroll
+          for (int j = 0; j < kPer; ++j) ov.v[j] += x.v[j];
         }
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) l += __shfl_xor_sync(0xffffffffu, l, o);
@@ -1038,7 +1098,7 @@ __global__ void __launch_bounds__(kThreads, 1)
             return x;
           };
           float m = -INFINITY;
-          ov = make_float4(0.f, 0.f, 0.f, 0.f);
+          ov = Row{};
           l = 0.f;
 #pragma unroll 1
           for (int c = 0; c < csize; ++c)
@@ -1049,15 +1109,17 @@ __global__ void __launch_bounds__(kThreads, 1)
             const float lc = sums(pc);
             if (lc == 0.f) continue;
             const float w = ex2(pc[kRowM] - m);
-            const float4 x = reinterpret_cast<const float4*>(pc)[lane];
-            ov.x = fmaf(w, x.x, ov.x), ov.y = fmaf(w, x.y, ov.y), ov.z = fmaf(w, x.z, ov.z), ov.w = fmaf(w, x.w, ov.w);
+            const Row x = reinterpret_cast<const Row*>(pc)[lane];
+#pragma unroll
+            for (int j = 0; j < kPer; ++j) ov.v[j] = fmaf(w, x.v[j], ov.v[j]);
             l = fmaf(w, lc, l);
           }
         }
         if (valid && p < a.M && l > 0.f) {
           const float inv_l = 1.f / l;
-          *reinterpret_cast<uint2*>(dst) =
-              make_uint2(cvt_bf16x2(ov.x * inv_l, ov.y * inv_l), cvt_bf16x2(ov.z * inv_l, ov.w * inv_l));
+#pragma unroll
+          for (int j = 0; j < kPer; j += 2)
+            *reinterpret_cast<uint32_t*>(dst + j) = cvt_bf16x2(ov.v[j] * inv_l, ov.v[j + 1] * inv_l);
         }
       }
       if (elect_one()) asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
@@ -1068,11 +1130,12 @@ __global__ void __launch_bounds__(kThreads, 1)
 }
 
 // ------------------------------------------------------------------ host
-template <int kR>
+template <int kR, int kDim>
 bool set_attributes(const int* sizes, int n, int* active) {
-  const void* kerns[2] = {reinterpret_cast<const void*>(verify_wide_kernel<kR, false>),
-                          reinterpret_cast<const void*>(verify_wide_kernel<kR, true>)};
-  constexpr int smem = Cfg<kR>::kSmemBytes;
+  // (head dim 64 layers run as the rotation, append and attention kernels)
+  const void* kerns[2] = {reinterpret_cast<const void*>(verify_wide_kernel<kR, kDim, false>),
+                          reinterpret_cast<const void*>(verify_wide_kernel<kR, kDim, kDim == 128>)};
+  constexpr int smem = Cfg<kR, kDim>::kSmemBytes;
   for (const void* k : kerns)
     if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess ||
         cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) {
@@ -1101,11 +1164,11 @@ bool set_attributes(const int* sizes, int n, int* active) {
   return true;
 }
 
-template <int kR, bool kFused>
+template <int kR, int kDim, bool kFused>
 sd_status launch(const sd_kv_cache* cache, const TcArgs& a, const RopeTable& tab, int cs, cudaStream_t stream) {
   const int B = cache->batch, Hkv = cache->n_kv_heads, cap = cache->capacity;
   CUtensorMap k128, v128;
-  if (!make_map(&k128, cache->k, cap, B * Hkv, 128) || !make_map(&v128, cache->v, cap, B * Hkv, 128))
+  if (!make_map(&k128, cache->k, cap, B * Hkv, 128, kDim) || !make_map(&v128, cache->v, cap, B * Hkv, 128, kDim))
     return SD_ERR_CUDA;
   cudaLaunchConfig_t cfg = {};
   cudaLaunchAttribute attr[2];
@@ -1117,36 +1180,43 @@ sd_status launch(const sd_kv_cache* cache, const TcArgs& a, const RopeTable& tab
   attr[1].val.programmaticStreamSerializationAllowed = 1;
   cfg.gridDim = dim3(cs, Hkv * a.n_mblocks, B);
   cfg.blockDim = dim3(kThreads, 1, 1);
-  cfg.dynamicSmemBytes = Cfg<kR>::kSmemBytes;
+  cfg.dynamicSmemBytes = Cfg<kR, kDim>::kSmemBytes;
   cfg.stream = stream;
   cfg.attrs = attr;
   cfg.numAttrs = 2;
-  if (cudaLaunchKernelEx(&cfg, verify_wide_kernel<kR, kFused>, k128, v128, a, tab) != cudaSuccess) {
+  if (cudaLaunchKernelEx(&cfg, verify_wide_kernel<kR, kDim, kFused>, k128, v128, a, tab) != cudaSuccess) {
     (void)cudaGetLastError();
     return SD_ERR_CUDA;
   }
   return SD_OK;
 }
 
-template <bool kFused>
+template <int kDim, bool kFused>
 sd_status launch_rows(const sd_kv_cache* cache, const TcArgs& a, const RopeTable& tab, int rows, int cs,
                       cudaStream_t stream) {
-  if (rows == 32) return launch<32, kFused>(cache, a, tab, cs, stream);
-  if (rows == 48) return launch<48, kFused>(cache, a, tab, cs, stream);
-  if (rows == 64) return launch<64, kFused>(cache, a, tab, cs, stream);
-  return launch<80, kFused>(cache, a, tab, cs, stream);
+  if (rows == 32) return launch<32, kDim, kFused>(cache, a, tab, cs, stream);
+  if (rows == 48) return launch<48, kDim, kFused>(cache, a, tab, cs, stream);
+  if (rows == 64) return launch<64, kDim, kFused>(cache, a, tab, cs, stream);
+  return launch<80, kDim, kFused>(cache, a, tab, cs, stream);
+}
+
+template <int kDim>
+bool active_of(int rows, const int* sizes, int n, int* active) {
+  if (rows == 32) return set_attributes<32, kDim>(sizes, n, active);
+  if (rows == 48) return set_attributes<48, kDim>(sizes, n, active);
+  if (rows == 64) return set_attributes<64, kDim>(sizes, n, active);
+  return set_attributes<80, kDim>(sizes, n, active);
 }
 
 }  // namespace
 
-bool sd_internal_wide_active(int rows, const int* sizes, int n, int* active) {
-  if (rows == 32) return set_attributes<32>(sizes, n, active);
-  if (rows == 48) return set_attributes<48>(sizes, n, active);
-  if (rows == 64) return set_attributes<64>(sizes, n, active);
-  return set_attributes<80>(sizes, n, active);
+bool sd_internal_wide_active(int rows, int D, const int* sizes, int n, int* active) {
+  return D == 64 ? active_of<64>(rows, sizes, n, active) : active_of<128>(rows, sizes, n, active);
 }
 
 sd_status sd_internal_wide_launch(const sd_kv_cache* cache, const TcArgs& a, const RopeTable& tab, int rows, int cs,
                                   bool fused, cudaStream_t stream) {
-  return fused ? launch_rows<true>(cache, a, tab, rows, cs, stream) : launch_rows<false>(cache, a, tab, rows, cs, stream);
+  if (cache->head_dim == 64) return launch_rows<64, false>(cache, a, tab, rows, cs, stream);
+  return fused ? launch_rows<128, true>(cache, a, tab, rows, cs, stream)
+               : launch_rows<128, false>(cache, a, tab, rows, cs, stream);
 }

@@ -35,7 +35,7 @@ struct TcArgs {
 
 // attention_wide.cu: clusters of each size that fit at once (false: not
 // available here), and the launch on row tiles of `rows` (32, 48, 64, 80).
-bool sd_internal_wide_active(int rows, const int* sizes, int n, int* active);
+bool sd_internal_wide_active(int rows, int D, const int* sizes, int n, int* active);
 sd_status sd_internal_wide_launch(const sd_kv_cache* cache, const TcArgs& a, const RopeTable& tab, int rows, int cs,
                                   bool fused, cudaStream_t stream);
 
@@ -251,13 +251,14 @@ EncodeTiledFn encode_fn() {
   return fn;
 }
 
-bool make_map(CUtensorMap* map, void* base, int cap, int planes, int box_rows) {
+// [planes][cap][D] bf16 rows in boxes of 64 columns x box_rows, 128-byte swizzle
+bool make_map(CUtensorMap* map, void* base, int cap, int planes, int box_rows, int D = kD) {
   EncodeTiledFn fn = encode_fn();
   if (!fn) return false;
-  cuuint64_t dims[3] = {static_cast<cuuint64_t>(kD), static_cast<cuuint64_t>(cap),
+  cuuint64_t dims[3] = {static_cast<cuuint64_t>(D), static_cast<cuuint64_t>(cap),
                         static_cast<cuuint64_t>(planes)};
-  cuuint64_t strides[2] = {static_cast<cuuint64_t>(kD) * 2,
-                           static_cast<cuuint64_t>(cap) * static_cast<cuuint64_t>(kD) * 2};
+  cuuint64_t strides[2] = {static_cast<cuuint64_t>(D) * 2,
+                           static_cast<cuuint64_t>(cap) * static_cast<cuuint64_t>(D) * 2};
   cuuint32_t box[3] = {64, static_cast<cuuint32_t>(box_rows), 1};
   cuuint32_t estr[3] = {1, 1, 1};
   return fn(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, base, dims, strides, box, estr,

@@ -21,6 +21,7 @@ def _lib():
 
 def _run(q, k, v, k_new, v_new, prefix, fused, block):
     """Position-0 new rows (an identity rotation) through the layer or the attention."""
+    sections = (16, 24, 24) if q.shape[-1] == 128 else (8, 12, 12)
     B, R, Hq, D = q.shape
     bf = workloads.to_bf16
     kc, vc = np.full_like(k, np.nan), np.full_like(v, np.nan)  # stale rows hold NaN
@@ -34,7 +35,7 @@ def _run(q, k, v, k_new, v_new, prefix, fused, block):
     qd = bf(q).cuda()
     if fused:
         pos = torch.zeros((B, R, 3), dtype=torch.int32).cuda()
-        out = sd.verify_layer(qd, bf(k_new).cuda(), bf(v_new).cuda(), pos, (16, 24, 24), cache, 0, 1e6, block=block)
+        out = sd.verify_layer(qd, bf(k_new).cuda(), bf(v_new).cuda(), pos, sections, cache, 0, 1e6, block=block)
     else:
         out = sd.verify_attention(qd, cache, block=block)
     torch.cuda.synchronize()
@@ -46,10 +47,11 @@ def _run(q, k, v, k_new, v_new, prefix, fused, block):
 # (G, R): 1, 4, 17, 30, 32 (17, 31 new rows: past the 32-row tile's 16) | 33, 48 | 49, 64 | 65, 68, 80 | 81, 96 | 98, 128 packed rows, up to 31 new rows
 @pytest.mark.parametrize("G,R", [(1, 1), (4, 1), (17, 1), (2, 15), (4, 8), (2, 16), (1, 17), (1, 31), (11, 3), (4, 12), (7, 7), (4, 16), (5, 13), (4, 17), (16, 5), (27, 3), (6, 16), (7, 14),
                                  (4, 31), (8, 16)])
-@pytest.mark.parametrize("fused,block", [(True, False), (True, True), (False, False)])
-def test_tile_edges(G, R, fused, block):
+@pytest.mark.parametrize("fused,block,D", [(True, False, 128), (True, True, 128), (False, False, 128), (False, False, 64),
+                                           (False, True, 64)])
+def test_tile_edges(G, R, fused, block, D):
     prefix = [0, 1, 31, 127, 128, 129, 700]
-    B, Hkv, D, cap = len(prefix), 2, 128, 760
+    B, Hkv, cap = len(prefix), 2, 760
     rng = np.random.default_rng(100 * G + R)
     draw = lambda *s: rng.standard_normal(s).astype(np.float32)  # noqa: E731
     _run(draw(B, R, Hkv * G, D), draw(B, Hkv, cap, D), draw(B, Hkv, cap, D), draw(B, R, Hkv, D), draw(B, R, Hkv, D),
@@ -61,10 +63,10 @@ def test_tile_edges(G, R, fused, block):
 @pytest.mark.parametrize("G,R", [(4, 1), (4, 8), (6, 8), (8, 8), (4, 17)])
 @pytest.mark.parametrize("level", [-150.0, 100.0, -70.0, 55.0])
 @pytest.mark.parametrize("part", [1, 3])
-@pytest.mark.parametrize("cluster", [0, 1, 4])
-def test_row_sums_out_of_range(G, R, level, part, cluster):
+@pytest.mark.parametrize("cluster,D", [(0, 128), (1, 128), (4, 128), (0, 64), (1, 64)])
+def test_row_sums_out_of_range(G, R, level, part, cluster, D):
     prefix = [1500, 40]
-    B, Hkv, D, cap = len(prefix), 1, 128, 1540
+    B, Hkv, cap = len(prefix), 1, 1540
     rng = np.random.default_rng(int(1000 + level + 10 * G + R))
     draw = lambda *s: rng.standard_normal(s).astype(np.float32)  # noqa: E731
     u = np.zeros(D, dtype=np.float32)
@@ -78,7 +80,8 @@ def test_row_sums_out_of_range(G, R, level, part, cluster):
     k_new[..., 5] = beta if part == 1 else 0.0
     sd.set_cluster_size(cluster)
     try:
-        _run(q, k, draw(B, Hkv, cap, D), k_new, draw(B, R, Hkv, D), prefix, True, False)
+        if D == 128:
+            _run(q, k, draw(B, Hkv, cap, D), k_new, draw(B, R, Hkv, D), prefix, True, False)
         _run(q, k, draw(B, Hkv, cap, D), k_new, draw(B, R, Hkv, D), prefix, False, False)
     finally:
         sd.set_cluster_size(0)
