@@ -8,6 +8,7 @@ no CPU fallback, and loading fails loudly when the library is missing.
 """
 
 import ctypes
+import functools
 import os
 import re
 
@@ -104,10 +105,14 @@ def _check(status, what):
 
 
 def _stream():
-    return ctypes.c_void_p(torch.cuda.current_stream().cuda_stream)
+    """Handle of torch's current stream on the current device (without the Stream
+    object that torch.cuda.current_stream() builds, ~1 us a call)."""
+    return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
 
 
 def _dev(t, name, dtype=None, ndim=None):
+    """The checked tensor's device address (an int: the declared argument types
+    convert it; a c_void_p object an argument cost as much as its checks)."""
     if not isinstance(t, torch.Tensor):
         raise TypeError("%s must be a torch.Tensor" % name)
     if not t.is_cuda:
@@ -118,7 +123,12 @@ def _dev(t, name, dtype=None, ndim=None):
         raise ValueError("%s must be %s, got %s" % (name, dtype, t.dtype))
     if ndim is not None and t.dim() != ndim:
         raise ValueError("%s must have %d dims, got %s" % (name, ndim, tuple(t.shape)))
-    return ctypes.c_void_p(t.data_ptr())
+    return t.data_ptr()
+
+
+@functools.lru_cache(maxsize=64)
+def _sections(sections):
+    return (ctypes.c_int32 * 3)(*sections)
 
 
 def workspace(nbytes, device=None):
@@ -135,7 +145,7 @@ def rope_apply(q, k, pos, sections, interleaved=0, base=1e6):
     Hkv = k.shape[2]
     if tuple(k.shape) != (B, R, Hkv, D) or tuple(pos.shape) != (B, R, 3):
         raise ValueError("shape mismatch")
-    sec = (ctypes.c_int32 * 3)(*[int(s) for s in sections])
+    sec = _sections(tuple(int(s) for s in sections))
     _check(lib().sd_rope_apply(_dev(q, "q", torch.bfloat16), _dev(k, "k", torch.bfloat16), B, R, Hq,
                                Hkv, D, _dev(pos, "pos", torch.int32), sec, int(interleaved),
                                float(base), _stream()), "sd_rope_apply")
@@ -166,6 +176,8 @@ class KVCache:
         self.k, self.v, self.len = k, v, lens
         B, H, cap, D = k.shape
         self._struct = KVCacheStruct(k.data_ptr(), v.data_ptr(), lens.data_ptr(), B, H, cap, D)
+        # what a call reads, fixed with the struct
+        self._ref, self._shape = ctypes.byref(self._struct), (B, H, cap, D)
 
     @classmethod
     def empty(cls, B, Hkv, cap, D, device="cuda"):
@@ -174,11 +186,11 @@ class KVCache:
 
     @property
     def struct(self):
-        return ctypes.byref(self._struct)
+        return self._ref
 
     @property
     def shape(self):
-        return tuple(self.k.shape)
+        return self._shape
 
 
 def kv_append(cache, k_new, v_new):
@@ -286,7 +298,7 @@ def verify_layer(q, k_new, v_new, pos, sections, cache, interleaved=0, base=1e6,
         if ws is None or ws.numel() < need:
             ws = workspace(need, q.device)
             cache._layer_ws = ws
-    sec = (ctypes.c_int32 * 3)(*[int(x) for x in sections])
+    sec = _sections(tuple(int(x) for x in sections))
     _check(lib().sd_verify_layer(_dev(q, "q", torch.bfloat16), _dev(k_new, "k_new", torch.bfloat16),
                                  _dev(v_new, "v_new", torch.bfloat16), _dev(pos, "pos", torch.int32), sec,
                                  int(interleaved), float(base), cache.struct, _dev(out, "out", torch.bfloat16),
@@ -382,7 +394,7 @@ def verify_kernel(B, R, Hq, Hkv, D, capacity, layer=False):
 def get_device_error():
     """Synchronise the current stream; return and clear the device error bits."""
     bits = ctypes.c_uint32(0)
-    st = lib().sd_get_device_error(_stream(), ctypes.byref(bits))
+    st = lib().sd_get_device_error(torch.cuda.current_stream().cuda_stream, ctypes.byref(bits))
     if st not in (0, 5, 6):
         raise SDError("sd_get_device_error", st)
     return int(bits.value)
