@@ -105,8 +105,7 @@ struct Cfg {
   // cluster merge buffers (in the rings, free once this CTA's last MMA is done)
   static constexpr int kSend = 0;                           // this CTA's kR rows
   static constexpr int kRecv = round_up(kR * kRowBytes, 1024);
-  // slots for ceil(kR / c) rows from each of c ranks, c in {1, 2, 4, 6, 8, 16}
-  static constexpr int kRecvSlots = 66;
+  static constexpr int kRecvSlots = kR + 15;                // ceil(kR / c) rows from each of c <= 16 ranks
   static_assert(kRecv + kRecvSlots * kRowBytes <= kRing, "merge buffers");
 };
 
@@ -722,8 +721,9 @@ __global__ void __launch_bounds__(kThreads, 1)
 }
 
 // ------------------------------------------------------------------ host
-constexpr int kNumClusterSizes = 6;
-constexpr int kClusterSizes[kNumClusterSizes] = {1, 2, 4, 6, 8, 16};
+// cluster sizes that a call may choose (sd_set_cluster_size forces 1, 2, 4, 6, 8 or 16)
+constexpr int kNumClusterSizes = 8;
+constexpr int kClusterSizes[kNumClusterSizes] = {1, 2, 4, 5, 6, 8, 12, 16};
 
 // The row tiles: 32, 48, 64 and 80 packed rows of attention_wide.cu (the new rows
 // beside the prefix loop) for head dims 128 and 64, 64 of this file's kernel (every
@@ -786,17 +786,35 @@ DevState* state() {
   return &s;
 }
 
-// Cluster size: minimise waves x (32-key blocks per CTA + a fixed per-CTA cost)
-int pick_cluster(const int* active, long long units, int cap) {
-  const long long nblk = (cap + 31) / 32;
-  long long best_cost = -1;
+// Cluster size: the least waves x (128-key tiles a CTA + a fixed cost a wave), in
+// tiles; those past the first three, which are in shared memory before the rows are,
+// count a quarter more. Sizes above 8 cost more a wave (their set-up and exchange),
+// and one that leaves no room for the next layer's clusters loses the overlap of its
+// stream when layers are chained (the choice is the same with and without the early
+// prefix, so that both give the same bits); both weigh less on the wider row tiles,
+// whose 128 keys take longer. The weights are fitted to 60 measured shapes (1 to 256
+// (scene, head) pairs, L = 512 to 16384): the choice is within 2% of the best size on
+// 51 of them and 15% on the rest. Measured, one scene, 8 KV heads, us a launch at sizes 8 / 12:
+//   chained, 32 rows: L = 4096 6.3 / 8.1, 8192 10.0 / 10.2, 12288 13.3 / 12.0, 16384 15.7 / 14.2
+//   chained, 80 rows: L = 4096 10.8 / 11.5, 8192 15.5 / 14.8, 16384 23.2 / 20.1
+//   plain, 32 rows:   L = 2048 6.2 / 6.4, 4096 7.5 / 7.5, 8192 10.5 / 10.0, 16384 16.0 / 14.7
+// 4 KV heads at 8 / 12 / 16: draft step L = 4096 7.1 / 6.2 / 6.2, chained 5.5 / 5.1 / 5.6, L = 16384
+// 13.3 / 11.0 / 10.0. 24 (scene, head) pairs, L = 8192, at 4 / 5: 18.0 / 17.7.
+int pick_cluster(const int* active, long long units, int cap, int rows) {
+  const double nblk = (cap + 31) / 32, wide = rows <= 32 ? 1.0 : (rows <= 48 ? 0.8 : 0.5);
+  double best_cost = -1;
   int best = 0;
   for (int i = 0; i < kNumClusterSizes; ++i) {
     const int cs = kClusterSizes[i];
     if (active[i] <= 0) continue;
-    if (cs > 1 && nblk < 2LL * cs) continue;
+    if (cs > 1 && nblk < 2.0 * cs) continue;
     const long long waves = (units + active[i] - 1) / active[i];
-    const long long cost = waves * ((nblk + cs - 1) / cs + 6);
+    // the share of the next layer's clusters that fit beside this layer's
+    const double room = waves > 1 ? 0.0 : static_cast<double>(active[i] - units) / static_cast<double>(units);
+    const double fixed = (waves > 1 ? 3.0 : 1.0) + wide * ((cs == 12 ? 1.2 : (cs == 16 ? 1.6 : 0.0)) +
+                                                           2.3 * (room < 1.0 ? 1.0 - room : 0.0));
+    const double tiles = nblk / (4.0 * cs);
+    const double cost = static_cast<double>(waves) * (tiles + 0.25 * (tiles > 3.0 ? tiles - 3.0 : 0.0) + fixed);
     if (best_cost < 0 || cost < best_cost) {
       best_cost = cost;
       best = cs;
@@ -831,8 +849,8 @@ extern "C" sd_status sd_set_cluster_size(int cluster_size) {
     g_forced_cluster.store(0);
     return SD_OK;
   }
-  for (int i = 0; i < kNumClusterSizes; ++i)
-    if (kClusterSizes[i] == cluster_size) {
+  for (int cs : {1, 2, 4, 6, 8, 16})
+    if (cs == cluster_size) {
       g_forced_cluster.store(cluster_size);
       return SD_OK;
     }
@@ -863,7 +881,7 @@ static TcPlan tc_plan(int B, int R, int Hq, int Hkv, int D, int cap, bool all_ke
   const int forced = g_forced_cluster.load();
   for (int i = 0; i < kNumClusterSizes && forced > 0; ++i)
     if (kClusterSizes[i] == forced && active[i] > 0) p.cs = forced;
-  if (p.cs == 0) p.cs = pick_cluster(active, static_cast<long long>(B) * Hkv * p.mblocks, cap);
+  if (p.cs == 0) p.cs = pick_cluster(active, static_cast<long long>(B) * Hkv * p.mblocks, cap, p.rows);
   return p;
 }
 

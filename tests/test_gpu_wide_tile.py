@@ -85,3 +85,17 @@ def test_row_sums_out_of_range(G, R, level, part, cluster, D):
         _run(q, k, draw(B, Hkv, cap, D), k_new, draw(B, R, Hkv, D), prefix, False, False)
     finally:
         sd.set_cluster_size(0)
+
+
+# (scenes, KV heads, capacity) whose clusters are of 5, 12, 12 and 16 CTAs: a scene that
+# leaves most of them without a key, and one whose last 32-key split is partial
+@pytest.mark.parametrize("prefix,Hkv,cap", [([0, 37, 4099], 8, 4112), ([70, 4099], 2, 4112), ([4088], 4, 4112), ([16390], 4, 16400)])
+@pytest.mark.parametrize("G,R", [(4, 1), (4, 8), (8, 8), (5, 12)])
+@pytest.mark.parametrize("fused,D", [(True, 128), (False, 64)])
+def test_cluster_sizes(prefix, Hkv, cap, G, R, fused, D):
+    B = len(prefix)
+    rng = np.random.default_rng(cap + 10 * G + R)
+    draw = lambda *s: rng.standard_normal(s).astype(np.float32)  # noqa: E731
+    prefix = [min(n, cap - R) for n in prefix]
+    _run(draw(B, R, Hkv * G, D), draw(B, Hkv, cap, D), draw(B, Hkv, cap, D), draw(B, R, Hkv, D), draw(B, R, Hkv, D),
+         prefix, fused, False)
