@@ -56,6 +56,11 @@ sd_status sd_internal_verify_layer_tc(void* q, void* k_new, const void* v_new, c
                                       int R, int Hq, float scale_log2, uint32_t* ticket, int early,
                                       int block, cudaStream_t stream, bool* handled);
 
+// The rotation of a layer's new rows and the KV append as one launch (kv.cu);
+// D 64 or 128, at most 65535 scenes, arguments checked by the layer.
+sd_status sd_internal_rope_append(void* q, void* k_new, const void* v_new, const int32_t* pos, const RopeTable& tab,
+                                  const sd_kv_cache* cache, int R, int Hq, cudaStream_t stream);
+
 // ---------------------------------------------------------------------------
 // Host helpers
 // ---------------------------------------------------------------------------
@@ -166,14 +171,33 @@ __device__ __forceinline__ uint32_t sd_rope_pair(uint32_t w, float c, float s) {
   return sd_pack_bf16x2(fmaf(x, c, -y * s), fmaf(x, s, y * c));
 }
 
-// Rotate 4 adjacent pairs (8 bf16 packed in w[4]) of head-vector chunk `vec`
-// (pairs 4*vec .. 4*vec+3) at coordinates p3 (t, h, w).
-__device__ __forceinline__ void sd_rope_rotate8(uint32_t (&w)[4], int vec, const int (&p3)[3],
-                                                const RopeTable& tab) {
+// The table entries of head-vector chunk `vec` (pairs 4*vec .. 4*vec+3). A
+// warp's lanes index the constant bank at D / 8 places, one access each: read
+// before the wait for the previous kernel, off the dependent path.
+struct RopeChunk {
+  float hi[4], lo[4];
+  int axis[4];
+};
+__device__ __forceinline__ RopeChunk sd_rope_chunk(int vec, const RopeTable& tab) {
+  RopeChunk c;
 #pragma unroll
   for (int j = 0; j < 4; ++j) {
-    const int d = vec * 4 + j;
-    const float2 cs = sd_rope_cs(static_cast<float>(p3[tab.axis[d]]), d, tab);
-    w[j] = sd_rope_pair(w[j], cs.x, cs.y);
+    c.hi[j] = tab.tau_hi[vec * 4 + j];
+    c.lo[j] = tab.tau_lo[vec * 4 + j];
+    c.axis[j] = tab.axis[vec * 4 + j];
   }
+  return c;
+}
+
+// Rotate the chunk's 4 adjacent pairs (8 bf16) at coordinates (t, h, w).
+__device__ __forceinline__ uint4 sd_rope_rotate8(const uint4& v, int pt, int ph, int pw, const RopeChunk& c) {
+  uint32_t w[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+  for (int j = 0; j < 4; ++j) {
+    const float p = static_cast<float>(c.axis[j] == 0 ? pt : (c.axis[j] == 1 ? ph : pw));
+    float s, co;
+    sincospif(2.0f * sd_frac_turns(p, c.hi[j], c.lo[j]), &s, &co);
+    w[j] = sd_rope_pair(w[j], co, s);
+  }
+  return make_uint4(w[0], w[1], w[2], w[3]);
 }

@@ -47,6 +47,52 @@ __global__ void __launch_bounds__(512) kv_append_kernel(uint4* __restrict__ kc, 
   if (threadIdx.x == 0) len[b] = l0 + R;
 }
 
+// The rotation of a layer's new query and key rows and the append in one
+// launch: block 0 of a scene rotates its key rows in place and copies them and
+// the value rows into the cache, then advances len[b] (read by all of its
+// threads before); the other blocks rotate the query rows, a 16-byte chunk a
+// thread. Bound by the latency of one launch: rows, positions and length travel
+// together, the rotation's table is read before the wait.
+template <int D>
+__global__ void __launch_bounds__(512) rope_append_kernel(uint4* __restrict__ q, uint4* __restrict__ kn,
+                                                          const uint4* __restrict__ vn, const int32_t* __restrict__ pos,
+                                                          uint4* __restrict__ kc, uint4* __restrict__ vc,
+                                                          int32_t* __restrict__ len, int R, int hq, int hkv, int cap,
+                                                          const __grid_constant__ RopeTable tab) {
+  constexpr int kVec = D / 8;
+  const int b = blockIdx.y, vec = threadIdx.x % kVec;
+  const RopeChunk chunk = sd_rope_chunk(vec, tab);
+  sd_pdl_enter();
+  pos += static_cast<long long>(b) * R * 3;
+  if (blockIdx.x > 0) {
+    const long long i = (blockIdx.x - 1) * 512ll + threadIdx.x, n = static_cast<long long>(R) * hq * kVec;
+    if (i >= n) return;
+    const int32_t* p3 = pos + i / (kVec * hq) * 3;
+    uint4* x = q + b * n + i;
+    *x = sd_rope_rotate8(*x, p3[0], p3[1], p3[2], chunk);
+    return;
+  }
+  const int l0 = len[b], n = R * hkv * kVec;
+  const bool ok = l0 >= 0 && static_cast<long long>(l0) + R <= cap;
+  for (int i = threadIdx.x; i < n; i += 512) {
+    const int t = i / kVec, g = t % hkv, r = t / hkv;
+    const long long src = static_cast<long long>(b) * n + i;  // [b][r][g][vec]
+    const uint4 k = kn[src], v = vn[src];
+    const uint4 kr = sd_rope_rotate8(k, pos[r * 3], pos[r * 3 + 1], pos[r * 3 + 2], chunk);
+    kn[src] = kr;
+    if (ok) {
+      const long long dst = ((static_cast<long long>(b) * hkv + g) * cap + (l0 + r)) * kVec + vec;
+      kc[dst] = kr;
+      vc[dst] = v;
+    }
+  }
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    if (ok) len[b] = l0 + R;
+    else sd_set_error(SD_DEVERR_KV_OVERFLOW);
+  }
+}
+
 __global__ void kv_rollback_kernel(int32_t* __restrict__ len, int count, int B,
                                    const int32_t* __restrict__ committed, int n_appended) {
   sd_pdl_enter();
@@ -79,6 +125,20 @@ extern "C" sd_status sd_kv_append(const sd_kv_cache* cache, const void* k_new, c
                     static_cast<uint4*>(cache->k), static_cast<uint4*>(cache->v), cache->len,
                     static_cast<const uint4*>(k_new), static_cast<const uint4*>(v_new), R, hkv, cap,
                     D / 8) != cudaSuccess) {
+    (void)cudaGetLastError();
+    return SD_ERR_CUDA;
+  }
+  return SD_OK;
+}
+
+sd_status sd_internal_rope_append(void* q, void* k_new, const void* v_new, const int32_t* pos, const RopeTable& tab,
+                                  const sd_kv_cache* cache, int R, int Hq, cudaStream_t stream) {
+  const int B = cache->batch, hkv = cache->n_kv_heads, D = cache->head_dim;
+  const long long nq = (static_cast<long long>(R) * Hq * (D / 8) + 511) / 512;
+  if (sd_launch_pdl(D == 64 ? rope_append_kernel<64> : rope_append_kernel<128>, dim3(static_cast<unsigned>(1 + nq), B),
+                    dim3(512), 0, stream, static_cast<uint4*>(q), static_cast<uint4*>(k_new),
+                    static_cast<const uint4*>(v_new), pos, static_cast<uint4*>(cache->k), static_cast<uint4*>(cache->v),
+                    cache->len, R, Hq, hkv, cache->capacity, tab) != cudaSuccess) {
     (void)cudaGetLastError();
     return SD_ERR_CUDA;
   }

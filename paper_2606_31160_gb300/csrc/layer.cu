@@ -18,6 +18,12 @@ namespace {
 constexpr size_t kTicketBytes(int B, int Hkv) {
   return (static_cast<size_t>(B) * (1 + static_cast<size_t>(Hkv)) * 4 + 255) / 256 * 256;
 }
+// 16-byte chunks of a scene's new key rows up to which the rotation and the
+// append run as one launch: one a thread of the block that keeps a scene's append
+// together. Measured as a layer, us with two launches / one: 40 chunks (one scene)
+// 7.3 / 6.6, 192 (five) 12.6 / 11.8, 256 (eight) 14.6 / 13.4; 1024 (one) 9.6 / 9.8,
+// 1984 9.7 / 11.9.
+constexpr long long kAppendChunks = 512;
 }  // namespace
 
 extern "C" size_t sd_verify_layer_workspace(int B, int R, int Hq, int Hkv, int D, int capacity) {
@@ -58,11 +64,17 @@ extern "C" sd_status sd_verify_layer(void* q, void* k_new, const void* v_new, co
                                                   scale_log2, ticket, flags & SD_LAYER_PREFIX_EARLY,
                                                   block, st, &handled);
   if (handled) return s;
-  // other shapes: the same three steps as separate kernels
-  sd_status r = sd_rope_apply(q, k_new, B, R, Hq, Hkv, D, pos, sections, interleaved, base, stream);
-  if (r != SD_OK) return r;
-  r = sd_kv_append(cache, k_new, v_new, R, stream);
-  if (r != SD_OK) return r;
+  // other shapes: the same three steps, the first two in one launch while a
+  // scene's new key rows are few enough for one block
+  if (static_cast<long long>(R) * Hkv * (D / 8) <= kAppendChunks && B <= 65535) {
+    const sd_status r = sd_internal_rope_append(q, k_new, v_new, pos, tab, cache, R, Hq, st);
+    if (r != SD_OK) return r;
+  } else {
+    sd_status r = sd_rope_apply(q, k_new, B, R, Hq, Hkv, D, pos, sections, interleaved, base, stream);
+    if (r != SD_OK) return r;
+    r = sd_kv_append(cache, k_new, v_new, R, stream);
+    if (r != SD_OK) return r;
+  }
   return sd_verify_attention_ex(q, cache, out, R, Hq, scale, block ? SD_ATTN_BLOCK_MASK : 0,
                                 static_cast<char*>(workspace) + kTicketBytes(B, Hkv),
                                 ws_bytes - kTicketBytes(B, Hkv), stream);

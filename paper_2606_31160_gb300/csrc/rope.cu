@@ -28,13 +28,15 @@ __global__ void __launch_bounds__(256) rope_kernel(__nv_bfloat16* __restrict__ q
                                                    int rows, int hq, int hkv,
                                                    const int32_t* __restrict__ pos,
                                                    RopeTable tab) {
-  sd_pdl_enter();
   constexpr int kVecPerHead = D / 8;
+  // every chunk of a thread is the same one of its head: the stride is a multiple of D / 8
+  const int vec = threadIdx.x % kVecPerHead;
+  const RopeChunk chunk = sd_rope_chunk(vec, tab);
+  sd_pdl_enter();
   const int heads = hq + hkv;
   const long long total = (long long)rows * heads * kVecPerHead;
   for (long long idx = blockIdx.x * (long long)blockDim.x + threadIdx.x; idx < total;
        idx += (long long)gridDim.x * blockDim.x) {
-    const int vec = (int)(idx % kVecPerHead);
     const long long t = idx / kVecPerHead;
     const int head = (int)(t % heads);
     const long long row = t / heads;  // flattened (b, r)
@@ -42,17 +44,8 @@ __global__ void __launch_bounds__(256) rope_kernel(__nv_bfloat16* __restrict__ q
                                     : k + ((row * hkv + (head - hq)) * D);
     uint4* ptr = reinterpret_cast<uint4*>(base) + vec;
     const uint4 v = *ptr;
-    uint32_t words[4] = {v.x, v.y, v.z, v.w};
-    int p3[3];
-    if (kFlat) {
-      p3[0] = p3[1] = p3[2] = pos[row];
-    } else {
-      p3[0] = pos[row * 3 + 0];
-      p3[1] = pos[row * 3 + 1];
-      p3[2] = pos[row * 3 + 2];
-    }
-    sd_rope_rotate8(words, vec, p3, tab);
-    *ptr = make_uint4(words[0], words[1], words[2], words[3]);
+    const int32_t* pr = pos + (kFlat ? row : row * 3);
+    *ptr = sd_rope_rotate8(v, pr[0], pr[kFlat ? 0 : 1], pr[kFlat ? 0 : 2], chunk);
   }
 }
 

@@ -188,3 +188,33 @@ def test_fused_layer_interleaved_mrope(K):
     ref_blocked = oracle.mrope_apply(to64(case.q), pos, case.sections, 0, case.base)
     assert np.abs(to64(qb) - ref_blocked).max() > 0.1
     assert sd.get_device_error() == 0
+
+
+# layers outside the tcgen05 path: a single row, 504 and 512 16-byte chunks of new key rows a scene
+# (rotation and append in one launch), 520 (two launches), and head_dim 128 past 31 new rows at 512 and
+# 528; the last scene has no room and keeps its cache and length
+@pytest.mark.parametrize("R,Hq,Hkv,D,interleaved", [(1, 1, 1, 64, 0), (7, 18, 9, 64, 1), (16, 16, 4, 64, 0), (5, 13, 13, 64, 0),
+                                                    (32, 4, 1, 128, 1), (33, 1, 1, 128, 0)])
+def test_rotation_and_append_of_a_layer(R, Hq, Hkv, D, interleaved):
+    sections = (16, 24, 24) if D == 128 else (8, 12, 12)
+    prefix = [0, 5, 90]
+    B, cap = len(prefix), 90 + R - 1
+    rng = np.random.default_rng(R + Hkv)
+    bf = lambda *s: workloads.to_bf16(rng.standard_normal(s)).cuda()  # noqa: E731
+    q, k, v = bf(B, R, Hq, D), bf(B, R, Hkv, D), bf(B, R, Hkv, D)
+    pos = torch.from_numpy(rng.integers(0, 16000, (B, R, 3)).astype(np.int32)).cuda()
+    kc, vc = bf(B, Hkv, cap, D), bf(B, Hkv, cap, D)
+    got = []
+    for fused in (False, True):
+        qi, ki = q.clone(), k.clone()
+        cache = sd.KVCache(kc.clone(), vc.clone(), torch.tensor(prefix, dtype=torch.int32).cuda())
+        if fused:
+            sd.verify_layer(qi, ki, v, pos, sections, cache, interleaved, 1e6)
+        else:
+            sd.rope_apply(qi, ki, pos, sections, interleaved, 1e6)
+            sd.kv_append(cache, ki, v)
+        torch.cuda.synchronize()
+        assert sd.get_device_error() & sd.SD_DEVERR_KV_OVERFLOW
+        got.append((qi, ki, cache.k, cache.v, cache.len))
+    assert all(torch.equal(a, b) for a, b in zip(*got))
+    assert got[1][4].tolist() == [prefix[0] + R, prefix[1] + R, prefix[2]]
