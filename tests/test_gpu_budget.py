@@ -61,3 +61,29 @@ def test_visual_count_out_of_range_sets_error():
     sd.get_device_error()
     sd.attention_budget(q, cache, torch.tensor([29], dtype=torch.int32, device="cuda"))
     assert sd.get_device_error() & sd.SD_DEVERR_LENGTH
+
+
+# clusters of 1, 2, 8 and 16 CTAs; 31, 32, 33, 64, 65 and 96 packed rows (one to three passes); scenes that
+# leave CTAs of a cluster without a key; key counts around 8, 64 and the 320 staged at once (5120 a cluster
+# of 16); query rows that start on 4 bytes only; scores around 0 and spread over tens of bits
+@pytest.mark.parametrize("R,Hq,Hkv,D,prefix,nvis,cap", [
+    (31, 1, 1, 64, [0, 1, 33], [0, 0, 2], 64),
+    (8, 4, 1, 128, [56, 57, 312, 313], [56, 1, 300, 0], 500),
+    (11, 3, 1, 128, [1, 505, 2030], [1, 500, 2030], 2047),
+    (16, 8, 2, 64, [0, 31, 5104, 5105], [0, 30, 4000, 5105], 5140),
+    (13, 10, 2, 128, [20, 5107, 5108], [7, 5000, 5108], 5121),
+    (12, 8, 1, 64, [3, 10235], [1, 9000], 10300),
+])
+@pytest.mark.parametrize("offset,spread", [(0, 1.0), (2, 1.0), (0, 6.0)])
+def test_cluster_and_chunk_edges(R, Hq, Hkv, D, prefix, nvis, cap, offset, spread):
+    B = len(prefix)
+    rng = np.random.default_rng(R * Hq + cap)
+    k = workloads.to_bf16(rng.standard_normal((B, Hkv, cap, D)))
+    for b, n in enumerate(prefix):
+        k[b, :, n + R:] = float("nan")  # stale rows
+    n = B * R * Hq * D
+    q = torch.zeros(n + offset, dtype=torch.bfloat16, device="cuda")[offset:].view(B, R, Hq, D)
+    q.copy_(workloads.to_bf16(spread * rng.standard_normal((B, R, Hq, D))))
+    kd = k.cuda()
+    cache = sd.KVCache(kd, kd, torch.tensor([p + R for p in prefix], dtype=torch.int32).cuda())
+    _check(q, cache, torch.tensor(nvis, dtype=torch.int32, device="cuda"))
