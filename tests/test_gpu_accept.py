@@ -229,3 +229,34 @@ def test_greedy_scan_edges(dtype, B, R, V, shift):
         assert np.array_equal(tokens.cpu().numpy(), want)
         assert int(ws.count_nonzero()) == 0
     assert sd.get_device_error() == 0
+
+
+# one value a row, chunk edges, more drafts than a warp's lanes, 486 rows (more CTAs than three an SM: the
+# shorter ring), unaligned rows and an unaligned base, two chunk sizes of the statistics; peaked rows, so
+# that the oracle's margins decide nearly every scene
+@pytest.mark.parametrize("B,K,V,shift", [(2, 0, 1, 0), (3, 1, 4095, 0), (3, 2, 4097, 0), (2, 33, 4100, 0), (1, 128, 8192, 0),
+                                         (2, 128, 3001, 0), (6, 40, 16388, 0), (3, 3, 8192, 1), (2, 5, 50257, 1)])
+def test_sample_edges(B, K, V, shift):
+    rng = np.random.default_rng(B + K + V)
+    z_t = (4.0 * rng.standard_normal((B, K + 1, V))).astype(np.float32)
+    z_d = (z_t[:, :K] + (0.3 if K < 16 else 0.02) * rng.standard_normal((B, K, V))).astype(np.float32)
+    z_t[0, 0, V // 2 + 1:] = -np.inf
+    T = 0.6
+    g = rng.gumbel(size=z_d.shape)
+    draft = (z_d / T + g).argmax(-1).astype(np.int32)
+    u = workloads.uniforms24(rng, (B, K + 1))
+
+    def put(a):
+        buf = torch.zeros(a.size + shift, dtype=torch.float32, device="cuda")
+        out = buf[shift:].view(a.shape)
+        out.copy_(torch.from_numpy(a))
+        return out
+
+    n, t = sd.accept_sample(put(z_t), put(z_d), torch.from_numpy(draft).cuda(), torch.from_numpy(u).cuda(), T)
+    rn, rt, margins = oracle.accept_sample(z_t, z_d, draft, u, T)
+    n, t = n.cpu().numpy(), t.cpu().numpy()
+    clear = [b for b in range(B) if min(margins[b][:-1], default=1.0) >= ACCEPT_MARGIN and margins[b][-1] >= DRAW_MARGIN]
+    assert 2 * len(clear) >= B
+    for b in clear:
+        assert n[b] == rn[b] and t[b].tolist() == rt[b].tolist(), (b, n[b], rn[b], t[b], rt[b])
+    assert sd.get_device_error() == 0
