@@ -12,10 +12,10 @@
 // shared memory.
 //
 // What bounds it. With many scenes the stream of K and V (32 scenes, L = 8192: K = 7
-// 153 -> 142 us, K = 8 165 -> 146, 1.0 of the measured copy). With one scene the
+// 153 -> 142 us, K = 8 165 -> 143, 1.0 of the measured copy). With one scene the
 // dependent path behind the previous kernel: rows, rotation, S(0), the tiles at
 // ~0.4 us of products each, the exchange (~0.7 us), the merge (target layer
-// 6.77 -> 6.27 us, K = 8 10.0 -> 7.8, K = 16 block 15.9 -> 11.4, draft step 6.8 -> 6.1
+// 6.77 -> 6.27 us, K = 8 10.0 -> 7.2, K = 16 block 15.9 -> 10.6, draft step 6.8 -> 6.1
 // on one cache).
 //
 // Head dim 64 (the attention; its layers run as the rotation, append and attention
@@ -389,33 +389,55 @@ __global__ void __launch_bounds__(kThreads, 1)
     ranges(len0);
     const int z = b * a.Hkv + kvh;
     const uint64_t evict_first = l2_evict_first_policy();
-    auto issue_tiles = [&](int pass, int t0, int t1) {
+    auto issue_k = [&](int pass, int t) {
+      const int T = pass * n_pre + t, s = T % kS;
+      // a whole 128-row box even for a short last tile: keys past the range
+      // are masked, rows past the capacity arrive zero-filled
+      if (t >= kS) mbar_wait(SREADY((T - kS) % 3), par3(T - kS));
+      if (elect_one()) {
+        mbar_expect_tx(FULLK(s), static_cast<uint32_t>(kKV));
+#pragma unroll
+        for (int h = 0; h < kHalves; ++h)
+          tma_load_3d_hint(base + s * kKV + h * kHalf, &tm_k128, FULLK(s), h * 64, key_begin + t * kStageKeys, z, evict_first);
+      }
+      __syncwarp();
+    };
+    auto issue_v = [&](int pass, int t) {
+      const int T = pass * n_pre + t, s = T % kS;
+      if (t >= kS) mbar_wait(PVDONE(s), parS(T - kS));
+      if (elect_one()) {
+        mbar_expect_tx(FULLV(s), static_cast<uint32_t>(kKV));
+#pragma unroll
+        for (int h = 0; h < kHalves; ++h)
+          tma_load_3d_hint(base + C::kRingV + s * kKV + h * kHalf, &tm_v128, FULLV(s), h * 64, key_begin + t * kStageKeys, z,
+                           evict_first);
+      }
+      __syncwarp();
+    };
+    // a ring of tiles waits for nothing
+    auto issue_first = [&](int pass, int n) {
 #pragma unroll 1
-      for (int t = t0; t < t1; ++t) {
-        const int T = pass * n_pre + t;
-        const int s = T % kS;
-        // a whole 128-row box even for a short last tile: keys past the range
-        // are masked, rows past the capacity arrive zero-filled
-        const int y0 = key_begin + t * kStageKeys;
-        const uint32_t kst = base + s * kKV, vst = base + C::kRingV + s * kKV;
-        if (t >= kS) mbar_wait(SREADY((T - kS) % 3), par3(T - kS));
-        if (elect_one()) {
-          mbar_expect_tx(FULLK(s), static_cast<uint32_t>(kKV));
-#pragma unroll
-          for (int h = 0; h < kHalves; ++h) tma_load_3d_hint(kst + h * kHalf, &tm_k128, FULLK(s), h * 64, y0, z, evict_first);
-        }
-        __syncwarp();
-        if (t >= kS) mbar_wait(PVDONE(s), parS(T - kS));
-        if (elect_one()) {
-          mbar_expect_tx(FULLV(s), static_cast<uint32_t>(kKV));
-#pragma unroll
-          for (int h = 0; h < kHalves; ++h) tma_load_3d_hint(vst + h * kHalf, &tm_v128, FULLV(s), h * 64, y0, z, evict_first);
-        }
-        __syncwarp();
+      for (int t = 0; t < n; ++t) {
+        issue_k(pass, t);
+        issue_v(pass, t);
+      }
+    };
+    // past it the keys go one tile ahead of the values: a key slot is free once its S
+    // is done, a value slot only after the softmax and the PV product, and waiting for
+    // that before the next keys left S idle for a memory round trip. Measured: a layer
+    // of 16384 keys 14.2 -> 13.7 us at K = 4, 19.9 -> 18.4 at 16; of 4096 keys at K = 8
+    // 7.75 -> 7.2; the attention of 8 scenes, 8192 keys, K = 16: 45.9 -> 43.9. (Every wait
+    // stays ahead of the phase after the one it waits for: K(T) and V(T) are still issued
+    // after S(T - kS) and PV(T - kS), and neither of those needs a later tile.)
+    auto issue_rest = [&](int pass, int n0) {
+#pragma unroll 1
+      for (int t = n0; t <= n_pre; ++t) {
+        if (t < n_pre) issue_k(pass, t);
+        if (t > n0) issue_v(pass, t - 1);
       }
     };
     const int n0 = min(n_pre, kS);
-    issue_tiles(0, 0, n0);
+    issue_first(0, n0);
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
@@ -452,7 +474,8 @@ __global__ void __launch_bounds__(kThreads, 1)
         if (!*reinterpret_cast<volatile int*>(s_redo)) break;
       }
       if (pass == 2) mbar_wait(MAXIMA, 0);  // every product of pass 1 is done
-      issue_tiles(pass, pass == 0 ? n0 : 0, n_pre);
+      if (pass > 0) issue_first(pass, n0);
+      issue_rest(pass, n0);
       if (pass > 0) continue;
       // the softmax threads arrive last (after the last S of the last pass), so
       // this warp and the issuing warps arrive before the decision
