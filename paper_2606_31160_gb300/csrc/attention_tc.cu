@@ -722,8 +722,8 @@ __global__ void __launch_bounds__(kThreads, 1)
 
 // ------------------------------------------------------------------ host
 // cluster sizes that a call may choose (sd_set_cluster_size forces 1, 2, 4, 6, 8 or 16)
-constexpr int kNumClusterSizes = 8;
-constexpr int kClusterSizes[kNumClusterSizes] = {1, 2, 4, 5, 6, 8, 12, 16};
+constexpr int kNumClusterSizes = 9;
+constexpr int kClusterSizes[kNumClusterSizes] = {1, 2, 4, 5, 6, 8, 10, 12, 16};
 
 // The row tiles: 32, 48, 64 and 80 packed rows of attention_wide.cu (the new rows
 // beside the prefix loop) for head dims 128 and 64, 64 of this file's kernel (every
@@ -794,12 +794,13 @@ DevState* state() {
 // prefix, so that both give the same bits); both weigh less on the wider row tiles,
 // whose 128 keys take longer. The weights are fitted to 60 measured shapes (1 to 256
 // (scene, head) pairs, L = 512 to 16384): the choice is within 2% of the best size on
-// 51 of them and 15% on the rest. Measured, one scene, 8 KV heads, us a launch at sizes 8 / 12:
-//   chained, 32 rows: L = 4096 6.3 / 8.1, 8192 10.0 / 10.2, 12288 13.3 / 12.0, 16384 15.7 / 14.2
-//   chained, 80 rows: L = 4096 10.8 / 11.5, 8192 15.5 / 14.8, 16384 23.2 / 20.1
-//   plain, 32 rows:   L = 2048 6.2 / 6.4, 4096 7.5 / 7.5, 8192 10.5 / 10.0, 16384 16.0 / 14.7
-// 4 KV heads at 8 / 12 / 16: draft step L = 4096 7.1 / 6.2 / 6.2, chained 5.5 / 5.1 / 5.6, L = 16384
-// 13.3 / 11.0 / 10.0. 24 (scene, head) pairs, L = 8192, at 4 / 5: 18.0 / 17.7.
+// 51 of them and 15% on the rest. Measured, one scene, 8 KV heads, us a launch at sizes
+// 8 / 10 / 12 (sizes 7, 9, 11 lie between or above; 13 and more do not fit in one wave):
+//   chained, 32 rows: L = 4096 6.3 / 6.6 / 7.8, 8192 9.4 / 8.9 / 9.8, 16384 14.8 / 14.6 / 13.7
+//   chained, 80 rows: L = 4096 10.7 / 11.1 / 11.5, 8192 14.6 / 14.2 / 14.2, 16384 20.9 / 19.9 / 18.6
+// 4 KV heads at 8 / 10 / 12 / 16: draft step L = 4096 6.9 / 6.6 / 6.1 / 6.2, chained 5.5 /
+// 5.6 / 5.2 / 5.6. 20 pairs, L = 4099, 48 rows, at 5 / 6 / 8: 11.2 / 11.0 / 16.9. 24 pairs,
+// L = 8192, 32 rows, at 4 / 5: 18.0 / 17.7.
 int pick_cluster(const int* active, long long units, int cap, int rows) {
   const double nblk = (cap + 31) / 32, wide = rows <= 32 ? 1.0 : (rows <= 48 ? 0.8 : 0.5);
   double best_cost = -1;
@@ -811,8 +812,8 @@ int pick_cluster(const int* active, long long units, int cap, int rows) {
     const long long waves = (units + active[i] - 1) / active[i];
     // the share of the next layer's clusters that fit beside this layer's
     const double room = waves > 1 ? 0.0 : static_cast<double>(active[i] - units) / static_cast<double>(units);
-    const double fixed = (waves > 1 ? 3.0 : 1.0) + wide * ((cs == 12 ? 1.2 : (cs == 16 ? 1.6 : 0.0)) +
-                                                           2.3 * (room < 1.0 ? 1.0 - room : 0.0));
+    const double fixed = (waves > 1 ? 3.0 : 1.0) + (cs == 10 ? 0.8 : wide * (cs == 12 ? 1.2 : (cs == 16 ? 1.6 : 0.0))) +
+                         wide * 2.3 * (room < 1.0 ? 1.0 - room : 0.0);
     const double tiles = nblk / (4.0 * cs);
     const double cost = static_cast<double>(waves) * (tiles + 0.25 * (tiles > 3.0 ? tiles - 3.0 : 0.0) + fixed);
     if (best_cost < 0 || cost < best_cost) {

@@ -87,9 +87,9 @@ def test_row_sums_out_of_range(G, R, level, part, cluster, D):
         sd.set_cluster_size(0)
 
 
-# (scenes, KV heads, capacity) whose clusters are of 5, 12, 12 and 16 CTAs: a scene that
+# (scenes, KV heads, capacity) whose clusters are of 5, 12, 12, 16 and 10 CTAs: a scene that
 # leaves most of them without a key, and one whose last 32-key split is partial
-@pytest.mark.parametrize("prefix,Hkv,cap", [([0, 37, 4099], 8, 4112), ([70, 4099], 2, 4112), ([4088], 4, 4112), ([16390], 4, 16400)])
+@pytest.mark.parametrize("prefix,Hkv,cap", [([0, 37, 4099], 8, 4112), ([70, 4099], 2, 4112), ([4088], 4, 4112), ([16390], 4, 16400), ([8189], 8, 8206)])
 @pytest.mark.parametrize("G,R", [(4, 1), (4, 8), (8, 8), (5, 12)])
 @pytest.mark.parametrize("fused,D", [(True, 128), (False, 64)])
 def test_cluster_sizes(prefix, Hkv, cap, G, R, fused, D):
