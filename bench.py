@@ -83,7 +83,7 @@ def measured_peaks():
 
 
 def kernel_source_hash():
-    path = os.path.join(ROOT, "paper_2606_31160_gb300", "csrc", "attention_tc.cu")
+    path = os.path.join(ROOT, "paper_2606_31160_gb300", "csrc", "attention_wide.cu")
     with open(path, "rb") as f:
         return hashlib.sha256(f.read()).hexdigest()
 
@@ -809,7 +809,7 @@ def main():
         "block_draft_step_gbs": round(long_bytes / (long_us * 1e-6) / 1e9, 1),
         "bytes_per_step": step_bytes(1),
         "roofline": {
-            "kernel": "sd_verify_layer -> verify_attn_tc_kernel<fused> (M-RoPE + append + attention, tcgen05)",
+            "kernel": "sd_verify_layer -> verify_wide_kernel<32, 128, fused> (M-RoPE + append + attention, tcgen05)",
             "bound": "hbm",
             "achieved": round(achieved, 1),
             "peak": peak,
@@ -901,9 +901,9 @@ def sweep(args):
                 torch.cuda.empty_cache()
 
 
-# The 32-row fused layer kernel's launch shape: 8 heads x a cluster of 8 CTAs
-# of 352 threads, 230,976 bytes of dynamic shared memory, 256 tensor-memory
-# columns.
+# A launch shape like the 32-row fused layer kernel's (8 heads x a cluster of 8
+# CTAs; that kernel has 608 threads and 231,888 bytes of dynamic shared memory):
+# 352 threads, 230,976 bytes, 256 tensor-memory columns.
 FLOOR_SHAPE = {"ctas": 64, "cluster": 8, "threads": 352, "smem": 230976, "tmem_cols": 256}
 
 
@@ -979,8 +979,8 @@ def profile_only(args):
                           "device_error": sd.get_device_error()}))
         return
     if args.only == "tiny":
-        # the tiny verify step (4 q / 1 KV x 64, L = 256, K = 4): M-RoPE, append
-        # and the mma.sync attention kernel (head_dim 64), accept, rollback
+        # the tiny verify step (4 q / 1 KV x 64, L = 256, K = 4): M-RoPE and
+        # append as one kernel, attention (head_dim 64), accept, rollback
         dev = torch.device("cuda", 0)
         case = workloads.tiny()
         q, k, v, pos = (x.to(dev) for x in (case.q, case.k_new, case.v_new, case.pos))

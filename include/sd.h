@@ -158,7 +158,8 @@ size_t sd_verify_attention_workspace(int B, int R, int Hq, int Hkv, int D, int c
  * The G*R query rows that share a KV head are packed into one tile, so each
  * K/V row is read from HBM once; when B*Hkv alone cannot fill the GPU each
  * head's keys are split over several CTAs whose partial softmax states merge
- * through `workspace` (sd_verify_attention_workspace bytes, zero-filled
+ * in the cluster (tcgen05 kernels) or through `workspace` (mma.sync kernel;
+ * required either way: sd_verify_attention_workspace bytes, zero-filled
  * before its first use and left zeroed by every completed call; calls that
  * share a workspace must not overlap on the device; after SD_ERR_TIMEOUT it
  * must be zero-filled again). Requires D in {64, 128}, Hq % Hkv == 0 and
@@ -206,12 +207,13 @@ sd_status sd_verify_attention_ex(const void* q, const sd_kv_cache* cache, void* 
 
 /*
  * Cluster size of the tcgen05 verify-attention kernels (sd_verify_attention
- * and sd_verify_layer, head_dim 128): one
+ * and sd_verify_layer; sd_verify_kernel says which shapes take them): one
  * thread-block cluster of `cluster_size` CTAs per (scene, KV head) splits that
  * head's keys evenly and merges the partial softmax states in distributed
  * shared memory (the split-L form of Eq. verify). 0 (the default) lets every
- * call choose from the occupancy of each size and the capacity; 1, 2, 4, 6, 8
- * or 16 forces that size for later calls on every device (a size of which no
+ * call choose among 1, 2, 4, 5, 6, 8, 10, 12 and 16 from the occupancy of each
+ * size and the capacity; 1, 2, 4, 6, 8 or 16 forces that size for later calls on
+ * every device (a size of which no
  * cluster fits on the device falls back to the automatic choice). Process-wide, host-only, no
  * device work; results are the same for every size up to fp32 rounding order.
  * Returns SD_ERR_INVALID_ARG for any other value.
@@ -295,7 +297,7 @@ size_t sd_verify_layer_workspace(int B, int R, int Hq, int Hkv, int D, int capac
  * For head_dim 128 this is one kernel: the tcgen05 kernel for G * R <= 128
  * and R <= 31;
  * other shapes run the three kernels in sequence (sd_verify_kernel names the
- * choice). A scene whose append would pass the
+ * choice), the first two as one launch where the new rows are few. A scene whose append would pass the
  * capacity sets SD_DEVERR_KV_OVERFLOW and is left untouched.
  */
 sd_status sd_verify_layer(void* q, void* k_new, const void* v_new, const int32_t* pos,
