@@ -15,7 +15,7 @@
 // 153 -> 142 us, K = 8 165 -> 143, 1.0 of the measured copy). With one scene the
 // dependent path behind the previous kernel: rows, rotation, S(0), the tiles at
 // ~0.4 us of products each, the exchange (~0.7 us), the merge (target layer
-// 6.77 -> 6.27 us, K = 8 10.0 -> 7.2, K = 16 block 15.9 -> 10.6, draft step 6.8 -> 6.1
+// 6.77 -> 6.24 us, K = 8 10.0 -> 7.2, K = 16 block 15.9 -> 10.4, draft step 6.8 -> 5.9
 // on one cache).
 //
 // Head dim 64 (the attention; its layers run as the rotation, append and attention
@@ -354,8 +354,9 @@ __global__ void __launch_bounds__(kThreads, 1)
   // keys of tile t that its PV product reads: whole 16-key steps up to the last key
   auto pv_keys = [&](int t) { return min(kStageKeys, (key_end - key_begin - t * kStageKeys + 15) & ~15); };
 
-  // a launch without the early prefix waits here, before any global access
-  if (!early) griddep_wait();
+  // a launch without the early prefix waits before any global access: here, and the
+  // softmax warps after a dry run of their set-up
+  if (!early && warp < kFirstSoft) griddep_wait();
 
   if (warp == 0) {
     // -------------------------------------------------------------- producer
@@ -627,7 +628,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     };
     const bool new_kv = last_rank && st < a.R * kChunks;
     const long long kv_row = ((static_cast<long long>(b) * a.R + (st / kChunks)) * a.Hkv + kvh) * kDim + (st % kChunks) * 8;
-    uint4 qv[kQc], kv = make_uint4(0, 0, 0, 0), vv = make_uint4(0, 0, 0, 0);
+    uint4 qv[kQc] = {}, kv = make_uint4(0, 0, 0, 0), vv = make_uint4(0, 0, 0, 0);
     auto load_q = [&] {
 #pragma unroll
       for (int u = 0; u < kQc; ++u) {
@@ -641,97 +642,120 @@ __global__ void __launch_bounds__(kThreads, 1)
       kv = __ldcg(reinterpret_cast<const uint4*>(k + src));
       vv = __ldcg(reinterpret_cast<const uint4*>(v + src));
     };
-    // Without the early prefix (the wait is behind) the rows are read here,
-    // together with the length and the positions: one global round trip before the
-    // tiles, not two. The attention's new rows need the length: the last rank's threads
-    // read it themselves rather than wait for the producer's at the CTA barrier (one
-    // scene, L = 4096, K = 7: 7.8 -> 7.4 us; head dim 64, L = 4099: 9.5 -> 8.9)
     auto cache_row = [&] {
       return ((static_cast<long long>(b) * a.Hkv + kvh) * a.cap + L_pre + (st / kChunks)) * kDim + (st % kChunks) * 8;
     };
-    if (!early) {
-      load_q();
-      if (kFused && new_kv) load_kv(a.k_new, a.v_new, kv_row);
-      if (!kFused && new_kv) {
-        ranges(__ldcg(a.len + b));
-        if (valid) load_kv(a.kc, a.vc, cache_row());
-      }
-    }
     const float2* cs_tab = reinterpret_cast<const float2*>(smem + C::kOffP);  // [R][64] (cos, sin)
-    if (kFused) {
-      // rotation table of the R new positions. A warp takes 4 pairs, its lanes 8
-      // rows: a constant-bank read serialises over the lanes' different addresses
-      // (with 32 pairs a warp the table took ~2800 cycles, on the path of the
-      // cluster launched last)
+    // rotation table of the R new positions. A warp takes 4 pairs, its lanes 8
+    // rows: a constant-bank read serialises over the lanes' different addresses
+    // (with 32 pairs a warp the table took ~2800 cycles, on the path of the
+    // cluster launched last)
+    auto make_table = [&](bool known) {
       float2* tabw = reinterpret_cast<float2*>(smem + C::kOffP);
       const int d = sw * 4 + (lane & 3);
 #pragma unroll 1
       for (int i = lane >> 2; i < a.R; i += 8) {
-        const int32_t pc = a.pos[(static_cast<long long>(b) * a.R + i) * 3 + tab.axis[d]];
+        const int32_t pc = known ? a.pos[(static_cast<long long>(b) * a.R + i) * 3 + tab.axis[d]] : tab.axis[d];
         tabw[i * 64 + d] = sd_rope_cs(static_cast<float>(pc), d, tab);
       }
-    }
-    tc_fence_before();
-    __syncthreads();
-    tc_fence_after();
-    const uint32_t tmem = *tmem_slot;
-    const uint32_t tmem_o = tmem + 3 * C::kSStride;
-    ranges(*s_len);
-    const bool has_new = valid && last_rank;
+    };
+    // the rows, rotated (fused), into the operand layouts; on the second of two runs
+    // the append too
+    auto store_rows = [&](bool has_kv, int it) {
+#pragma unroll
+      for (int u = 0; u < kQc; ++u) {
+        const int idx = st + u * kSoftThreads, row = idx / kChunks, c = idx % kChunks, p = mblock * kR + row;
+        if (idx >= kR * kChunks) break;
+        uint32_t w[4] = {qv[u].x, qv[u].y, qv[u].z, qv[u].w};
+        if (kFused && p < a.M) {
+          const float2* cs = cs_tab + gdiv(p) * 64 + c * 4;
+#pragma unroll
+          for (int j = 0; j < 4; ++j) w[j] = sd_rope_pair(w[j], cs[j].x, cs[j].y);
+        }
+        st_shared_v4(qs + swz(row, c, C::kQHalf), w[0], w[1], w[2], w[3]);
+      }
+      if (last_rank && st < C::kMaxNew * kChunks) {
+        // new key (rotated) and value rows, zero past R
+        const int i = st / kChunks, c = st % kChunks;
+        uint32_t w[4] = {kv.x, kv.y, kv.z, kv.w};
+        if (kFused && has_kv) {
+          const float2* cs = cs_tab + i * 64 + c * 4;
+#pragma unroll
+          for (int j = 0; j < 4; ++j) w[j] = sd_rope_pair(w[j], cs[j].x, cs[j].y);
+        }
+        const uint32_t off = swz(i, c, C::kNewHalf);
+        st_shared_v4(base + C::kOffNewK + off, w[0], w[1], w[2], w[3]);
+        st_shared_v4(base + C::kOffNewV + off, vv.x, vv.y, vv.z, vv.w);
+        if (kFused && has_kv && it == 1 && mblock == 0) {
+          // the append: cache rows L_pre .. L_pre + R - 1, which no CTA of
+          // this launch reads; and, when this cluster alone reads the head's
+          // raw key rows, their rotation in place
+          *reinterpret_cast<uint4*>(a.kc + cache_row()) = make_uint4(w[0], w[1], w[2], w[3]);
+          *reinterpret_cast<uint4*>(a.vc + cache_row()) = vv;
+          if (a.n_mblocks == 1) *reinterpret_cast<uint4*>(a.k_new + kv_row) = make_uint4(w[0], w[1], w[2], w[3]);
+        }
+      }
+    };
     // rank c merges packed rows [c * rpc, ...) of the m-block's rows_in rows
     const int rows_in = max(1, min(kR, a.M - mblock * kR));
     const int rpc = (rows_in + csize - 1) / csize;
     auto rows_of = [&](int c) { return max(0, min(rpc, rows_in - c * rpc)); };
     const int my_rows = rows_of(rank);
     const int mrow0 = rank * rpc;
-    {
-      // The rows, rotated (fused) and into the operand layouts. Iteration 0 runs
-      // BEFORE the dependency wait on whatever the rows hold: it brings this code
-      // into the instruction cache and the rows into L2, and iteration 1
-      // overwrites everything it stored (.cg loads: no stale L1 line).
+    uint32_t tmem;
+    bool has_new;
+    auto cta_barrier = [&] {
+      tc_fence_before();
+      __syncthreads();
+      tc_fence_after();
+      tmem = *tmem_slot;
+      ranges(*s_len);
+      has_new = valid && last_rank;
+    };
+    // Two runs, the first BEFORE the dependency wait on whatever the rows hold: it
+    // brings this code into the instruction cache (and, with the early prefix, the
+    // rows into L2), and the second overwrites everything it stored (.cg loads: no
+    // stale L1 line). The cluster launched last has no time for it. Without the early
+    // prefix the dry run and its table took the draft step from 6.14 to 5.93 us and the
+    // tiny layer from 6.9 to 6.6; as one loop for both kinds of launch the target layer
+    // lost 0.15 us, so each has its own.
+    const int it0 = last_cluster ? 1 : 0;
+    if (early) {
+      if (kFused) make_table(true);
+      cta_barrier();
       const bool has_kv = new_kv && valid;
 #pragma unroll 1
-      for (int it = early && !last_cluster ? 0 : 1; it < 2; ++it) {
-        if (early) {
-          if (it == 1) griddep_wait();
-          load_q();
-          if (kFused && has_kv) load_kv(a.k_new, a.v_new, kv_row);
-        }
-        if (!kFused && early && has_kv) load_kv(a.kc, a.vc, cache_row());
-#pragma unroll
-        for (int u = 0; u < kQc; ++u) {
-          const int idx = st + u * kSoftThreads, row = idx / kChunks, c = idx % kChunks, p = mblock * kR + row;
-          if (idx >= kR * kChunks) break;
-          uint32_t w[4] = {qv[u].x, qv[u].y, qv[u].z, qv[u].w};
-          if (kFused && p < a.M) {
-            const float2* cs = cs_tab + gdiv(p) * 64 + c * 4;
-#pragma unroll
-            for (int j = 0; j < 4; ++j) w[j] = sd_rope_pair(w[j], cs[j].x, cs[j].y);
-          }
-          st_shared_v4(qs + swz(row, c, C::kQHalf), w[0], w[1], w[2], w[3]);
-        }
-        if (last_rank && st < C::kMaxNew * kChunks) {
-          // new key (rotated) and value rows, zero past R
-          const int i = st / kChunks, c = st % kChunks;
-          uint32_t w[4] = {kv.x, kv.y, kv.z, kv.w};
-          if (kFused && has_kv) {
-            const float2* cs = cs_tab + i * 64 + c * 4;
-#pragma unroll
-            for (int j = 0; j < 4; ++j) w[j] = sd_rope_pair(w[j], cs[j].x, cs[j].y);
-          }
-          const uint32_t off = swz(i, c, C::kNewHalf);
-          st_shared_v4(base + C::kOffNewK + off, w[0], w[1], w[2], w[3]);
-          st_shared_v4(base + C::kOffNewV + off, vv.x, vv.y, vv.z, vv.w);
-          if (kFused && has_kv && it == 1 && mblock == 0) {
-            // the append: cache rows L_pre .. L_pre + R - 1, which no CTA of
-            // this launch reads; and, when this cluster alone reads the head's
-            // raw key rows, their rotation in place
-            *reinterpret_cast<uint4*>(a.kc + cache_row()) = make_uint4(w[0], w[1], w[2], w[3]);
-            *reinterpret_cast<uint4*>(a.vc + cache_row()) = vv;
-            if (a.n_mblocks == 1) *reinterpret_cast<uint4*>(a.k_new + kv_row) = make_uint4(w[0], w[1], w[2], w[3]);
-          }
-        }
+      for (int it = it0; it < 2; ++it) {
+        if (it == 1) griddep_wait();
+        load_q();
+        if (kFused && has_kv) load_kv(a.k_new, a.v_new, kv_row);
+        if (!kFused && has_kv) load_kv(a.kc, a.vc, cache_row());
+        store_rows(has_kv, it);
       }
+    } else {
+      // Without the early prefix the rows are read together with the length and the
+      // positions: one global round trip before the tiles, not two. The attention's
+      // new rows need the length: the last rank's threads read it themselves rather
+      // than wait for the producer's at the CTA barrier (one scene, L = 4096, K = 7:
+      // 7.8 -> 7.4 us; head dim 64, L = 4099: 9.5 -> 8.9)
+      valid = false;
+#pragma unroll 1
+      for (int it = it0; it < 2; ++it) {
+        if (it == 1) {
+          griddep_wait();
+          load_q();
+          if (kFused && new_kv) load_kv(a.k_new, a.v_new, kv_row);
+          if (!kFused && new_kv) {
+            ranges(__ldcg(a.len + b));
+            if (valid) load_kv(a.kc, a.vc, cache_row());
+          }
+        }
+        if (kFused) make_table(it == 1);
+        if (it == 1) cta_barrier();
+        store_rows(new_kv && valid, it);
+      }
+    }
+    {
       if (st < kR) row_nref[st] = 0.f;
       asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
       named_bar_sync(3, kSoftThreads + 32);  // Q is complete; the rotation table is no longer read
@@ -1005,13 +1029,13 @@ __global__ void __launch_bounds__(kThreads, 1)
 #pragma unroll
       for (int j0 = 0; j0 + 8 <= kOr; j0 += 8) {
         uint32_t x8[8];
-        tmem_ld(tmem_o + orow0 + j0 + lane_off, x8);
+        tmem_ld(tmem + 3 * C::kSStride + orow0 + j0 + lane_off, x8);
 #pragma unroll
         for (int j = 0; j < 8; ++j) o[j0 + j] = x8[j];
       }
       if constexpr (kOr % 8 != 0) {
         uint32_t x4[4];
-        tmem_ld(tmem_o + orow0 + kOr - 4 + lane_off, x4);
+        tmem_ld(tmem + 3 * C::kSStride + orow0 + kOr - 4 + lane_off, x4);
 #pragma unroll
         for (int j = 0; j < 4; ++j) o[kOr - 4 + j] = x4[j];
       }
