@@ -112,10 +112,10 @@ __device__ __forceinline__ void mma_bf16(float (&c)[4], const uint32_t (&a)[4], 
 // independent product chains), takes their maximum once and folds them without a
 // running one; the sums merge over lanes, warps and CTAs by a common maximum, one
 // rescale and plain additions; and every CTA finishes 32 / S rows of the cluster.
-// One scene, 32 rows on each of 8 KV heads, 4096 keys: 7.9 us (14.9 with a running
+// One scene, 32 rows on each of 8 KV heads, 4096 keys: 7.8 us (14.9 with a running
 // maximum per thread, query fragments read from global memory before the keys, and one
 // CTA merging the cluster); of it the length takes 1.0 us, the keys 2.5, the products
-// 1.4, the fold 1.0, the merges and the exchange 2.2. Eight scenes 44.8 us (64.7).
+// 1.4, the fold 1.0, the merges and the exchange 2.2. Eight scenes 44.1 us (64.7).
 constexpr int kTiles = 2;
 constexpr int kPassRows = 16 * kTiles;
 constexpr int kChunkKeys = 320;  // keys a CTA stages at once (10 boxes of 32)
@@ -289,8 +289,9 @@ __global__ void __launch_bounds__(kThreads, 2)
           }
         }
       }
-      // scores in log2 units, -inf where masked, and their maximum per row over
-      // the quad of lanes that holds the row. A block's 8 keys are mostly of one
+      // products, -inf where masked, and their maximum per row over the quad of lanes
+      // that holds the row (a score is the product in log2 units: one fma with the
+      // maximum, which rounds once). A block's 8 keys are mostly of one
       // segment and all visible (the packed rows past M, never written, need no
       // mask): what it costs is instructions, so such blocks skip the tests.
       const int kb0 = c0 + 8 * warp, full = min(k_hi, L);
@@ -306,17 +307,14 @@ __global__ void __launch_bounds__(kThreads, 2)
 #pragma unroll
           for (int u = 0; u < kTiles; ++u)
 #pragma unroll
-            for (int e = 0; e < 4; ++e) {
-              c[u][j][e] *= scale_log2;
-              bm[u][e >> 1] = fmaxf(bm[u][e >> 1], c[u][j][e]);
-            }
+            for (int e = 0; e < 4; ++e) bm[u][e >> 1] = fmaxf(bm[u][e >> 1], c[u][j][e]);
         } else {
 #pragma unroll
           for (int u = 0; u < kTiles; ++u)
 #pragma unroll
             for (int e = 0; e < 4; ++e) {
               const int key = kb + 2 * tq + (e & 1);
-              c[u][j][e] = key < k_hi && key <= lim[u][e >> 1] ? c[u][j][e] * scale_log2 : -INFINITY;
+              c[u][j][e] = key < k_hi && key <= lim[u][e >> 1] ? c[u][j][e] : -INFINITY;
               bm[u][e >> 1] = fmaxf(bm[u][e >> 1], c[u][j][e]);
             }
         }
@@ -328,7 +326,7 @@ __global__ void __launch_bounds__(kThreads, 2)
         for (int h2 = 0; h2 < 2; ++h2) {
 #pragma unroll
           for (int o = 1; o < 4; o <<= 1) bm[u][h2] = fmaxf(bm[u][h2], __shfl_xor_sync(0xffffffffu, bm[u][h2], o));
-          const float m = fmaxf(mx[u][h2], bm[u][h2]);
+          const float m = fmaxf(mx[u][h2], bm[u][h2] * scale_log2);
           row_rescale(st[u][h2], mx[u][h2], m);
           mx[u][h2] = m;
           ref[u][h2] = m == -INFINITY ? 0.f : m;
@@ -341,14 +339,14 @@ __global__ void __launch_bounds__(kThreads, 2)
 #pragma unroll
           for (int u = 0; u < kTiles; ++u)
 #pragma unroll
-            for (int e = 0; e < 4; ++e) st[u][e >> 1].v += ex2f(c[u][j][e] - ref[u][e >> 1]);
+            for (int e = 0; e < 4; ++e) st[u][e >> 1].v += ex2f(fmaf(c[u][j][e], scale_log2, -ref[u][e >> 1]));
         } else if (kb >= nv && kb + 8 <= full) {  // trajectory / prompt-text keys
 #pragma unroll
           for (int u = 0; u < kTiles; ++u)
 #pragma unroll
             for (int e = 0; e < 4; ++e) {
               RowSums& s = st[u][e >> 1];
-              const float d = c[u][j][e] - ref[u][e >> 1], w = ex2f(d);
+              const float d = fmaf(c[u][j][e], scale_log2, -ref[u][e >> 1]), w = ex2f(d);
               s.t += w;
               if (w > 0.f) s.n = fmaf(w, d, s.n);
             }
@@ -359,7 +357,7 @@ __global__ void __launch_bounds__(kThreads, 2)
             for (int e = 0; e < 4; ++e) {
               RowSums& s = st[u][e >> 1];
               const int key = kb + 2 * tq + (e & 1);
-              const float d = c[u][j][e] - ref[u][e >> 1], w = ex2f(d);  // masked: ex2(-inf) = 0
+              const float d = fmaf(c[u][j][e], scale_log2, -ref[u][e >> 1]), w = ex2f(d);  // masked: ex2(-inf) = 0
               const bool vis = key < nv, txt = key < L;
               s.v += vis ? w : 0.f;
               s.t += !vis && txt ? w : 0.f;
