@@ -39,7 +39,7 @@ cudaError_t sd_take_error_sample(uint32_t* bits);
 cudaError_t sd_take_error_budget(uint32_t* bits);
 
 // Verify attention on the tcgen05 path (attention_tc.cu). Sets *handled when
-// the shape is one it serves (head_dim 128, G * R <= 128) and it launched.
+// the shape is one it serves (G * R <= 128; head_dim 64 with up to 31 new rows) and it launched.
 sd_status sd_internal_verify_attention_tc(const void* q, const sd_kv_cache* cache, void* out,
                                           int R, int Hq, float scale_log2, int flags, cudaStream_t stream,
                                           bool* handled);
