@@ -71,8 +71,9 @@ struct Fold<__nv_bfloat16> {
   __device__ __forceinline__ float value() const { return fmaxf(sd_bf16_lo(m), sd_bf16_hi(m)); }
 };
 
-__device__ __forceinline__ float load_one(const float* p) { return __ldg(p); }
-__device__ __forceinline__ float load_one(const __nv_bfloat16* p) { return __bfloat162float(__ldg(p)); }
+// (loads past the read-only path: the kernel is resident while its inputs are written)
+__device__ __forceinline__ float load_one(const float* p) { return __ldcg(p); }
+__device__ __forceinline__ float load_one(const __nv_bfloat16* p) { return sd_ldcg_bf16(p); }
 
 // First element of a vector that equals best (a value it holds), as its offset.
 __device__ __forceinline__ int first_equal(const float*, const uint4& w, float best) {
@@ -98,8 +99,8 @@ __device__ __forceinline__ int first_equal(const __nv_bfloat16*, const uint4& w,
 // segments of vps; segment 0 also takes the elements before the first boundary,
 // the last one those after the last.
 template <typename T>
-__global__ void __launch_bounds__(kThreads) greedy_kernel(const T* __restrict__ logits, int R, int V, int vps,
-                                                          const int32_t* __restrict__ draft,
+__global__ void __launch_bounds__(kThreads) greedy_kernel(const T* logits, int R, int V, int vps,
+                                                          const int32_t* draft,
                                                           int32_t* __restrict__ n_emit,
                                                           int32_t* __restrict__ tokens,
                                                           int32_t* __restrict__ argmax_out,
@@ -126,13 +127,13 @@ __global__ void __launch_bounds__(kThreads) greedy_kernel(const T* __restrict__ 
     if (v + (kStep - 1) * kThreads < v1) {
       uint4 w[kStep];
 #pragma unroll
-      for (int k = 0; k < kStep; ++k) w[k] = __ldg(vec + v + k * kThreads);
+      for (int k = 0; k < kStep; ++k) w[k] = __ldcg(vec + v + k * kThreads);
 #pragma unroll
       for (int k = 0; k < kStep; ++k) f.add(w[k]);
     } else {
 #pragma unroll
       for (int k = 0; k < kStep; ++k)
-        if (v + k * kThreads < v1) f.add(__ldg(vec + v + k * kThreads));
+        if (v + k * kThreads < v1) f.add(__ldcg(vec + v + k * kThreads));
     }
     const float m = f.value();
     if (m > best) {
@@ -165,7 +166,7 @@ __global__ void __launch_bounds__(kThreads) greedy_kernel(const T* __restrict__ 
     for (int k = kStep - 1; k >= 0; --k) {
       const int v = step + k * kThreads;
       if (v >= v1) continue;
-      const int e = first_equal(row, __ldg(vec + v), best);
+      const int e = first_equal(row, __ldcg(vec + v), best);
       if (e != 0x7fffffff) at = min(static_cast<uint32_t>(head + v * kPer + e), at);
     }
   }
@@ -193,7 +194,7 @@ __global__ void __launch_bounds__(kThreads) greedy_kernel(const T* __restrict__ 
     if (j < R) {
       unsigned long long* key = keys + static_cast<long long>(b) * R + j;
       star = static_cast<int>(0xffffffffu - static_cast<uint32_t>(__ldcg(key)));
-      if (j < K) d = __ldg(draft + static_cast<long long>(b) * K + j);
+      if (j < K) d = __ldcg(draft + static_cast<long long>(b) * K + j);
       *key = 0ull;  // re-armed for the next call
       s_star[j] = star;
       if (argmax_out) argmax_out[static_cast<long long>(b) * R + j] = star;

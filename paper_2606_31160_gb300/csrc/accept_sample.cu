@@ -88,8 +88,8 @@ constexpr int kScalarChunk = kThreads * kScalarPer;
 
 template <bool kVec>
 __global__ void __launch_bounds__(kVec ? kVecThreads : kThreads)
-    sample_stats_kernel(const float* __restrict__ zt, const float* __restrict__ zd, int K, int V,
-                        float c2, int chunk, int n_chunks, const int32_t* __restrict__ draft,
+    sample_stats_kernel(const float* zt, const float* zd, int K, int V,
+                        float c2, int chunk, int n_chunks, const int32_t* draft,
                         float2* __restrict__ part, float* __restrict__ dlogit) {
   constexpr int kT = kVec ? kVecThreads : kThreads;
   const int c = blockIdx.x, rr = blockIdx.y, b = blockIdx.z;
@@ -100,8 +100,8 @@ __global__ void __launch_bounds__(kVec ? kVecThreads : kThreads)
   // the CTA whose chunk holds the draft token of its row records that logit
   if (threadIdx.x == 0 && rr != K) {
     const int j = rr < K ? rr : rr - K - 1;
-    const int x = __ldg(draft + static_cast<long long>(b) * K + j);
-    if (x >= lo && x < hi) dlogit[static_cast<long long>(b) * rows + rr] = __ldg(row + x);
+    const int x = __ldcg(draft + static_cast<long long>(b) * K + j);
+    if (x >= lo && x < hi) dlogit[static_cast<long long>(b) * rows + rr] = __ldcg(row + x);
   }
   float m = -INFINITY, s = 0.f;
   if (kVec) {
@@ -110,7 +110,7 @@ __global__ void __launch_bounds__(kVec ? kVecThreads : kThreads)
 #pragma unroll
     for (int k = 0; k < kVecPer / 4; ++k) {
       const int i = lo + 4 * (threadIdx.x + kT * k);
-      const float4 v = i < hi ? __ldg(reinterpret_cast<const float4*>(row + i))
+      const float4 v = i < hi ? __ldcg(reinterpret_cast<const float4*>(row + i))
                               : make_float4(-INFINITY, -INFINITY, -INFINITY, -INFINITY);
       x[4 * k + 0] = v.x;
       x[4 * k + 1] = v.y;
@@ -128,7 +128,7 @@ __global__ void __launch_bounds__(kVec ? kVecThreads : kThreads)
 #pragma unroll
     for (int k = 0; k < kScalarPer; ++k) {
       const int i = lo + threadIdx.x + kT * k;
-      x[k] = i < hi ? __ldg(row + i) : -INFINITY;
+      x[k] = i < hi ? __ldcg(row + i) : -INFINITY;
     }
 #pragma unroll
     for (int k = 0; k < kScalarPer; ++k) m = fmaxf(m, x[k]);
@@ -187,8 +187,8 @@ __device__ __forceinline__ bool st_wait(uint32_t bar, uint32_t parity) {
 
 template <int kStreamStages>
 __global__ void __launch_bounds__(kStreamThreads)
-    sample_stats_stream_kernel(const float* __restrict__ zt, const float* __restrict__ zd, int K, int V,
-                               float c2, int seg, int n_seg, const int32_t* __restrict__ draft,
+    sample_stats_stream_kernel(const float* zt, const float* zd, int K, int V,
+                               float c2, int seg, int n_seg, const int32_t* draft,
                                float2* __restrict__ part, float* __restrict__ dlogit) {
   extern __shared__ __align__(128) float stage_raw[];  // [kStreamStages][kStageFloats]
   float (*stage)[kStageFloats] = reinterpret_cast<float (*)[kStageFloats]>(stage_raw);
@@ -235,8 +235,8 @@ __global__ void __launch_bounds__(kStreamThreads)
       }
       if (rr != K) {
         const int j = rr < K ? rr : rr - K - 1;
-        const int x = __ldg(draft + static_cast<long long>(b) * K + j);
-        if (x >= lo && x < hi) dlogit[static_cast<long long>(b) * rows + rr] = __ldg(row + x);
+        const int x = __ldcg(draft + static_cast<long long>(b) * K + j);
+        if (x >= lo && x < hi) dlogit[static_cast<long long>(b) * rows + rr] = __ldcg(row + x);
       }
     }
   } else {
@@ -305,8 +305,8 @@ __global__ void __launch_bounds__(kStreamThreads)
 // the row to draw from. The CTA that publishes also writes n_emit and the
 // accepted tokens (all but token l, which the draw writes).
 __device__ __forceinline__ DrawInfo accept_scene(int K, int V, float c2, int n_chunks, int b,
-                                                 const int32_t* __restrict__ draft, const float* __restrict__ u,
-                                                 const float2* __restrict__ part, const float* __restrict__ dlogit,
+                                                 const int32_t* draft, const float* u,
+                                                 const float2* part, const float* dlogit,
                                                  bool publish, int32_t* __restrict__ n_emit,
                                                  int32_t* __restrict__ tokens) {
   const int rows = 2 * K + 1;
@@ -320,14 +320,14 @@ __device__ __forceinline__ DrawInfo accept_scene(int K, int V, float c2, int n_c
   __shared__ int s_x[128];
   __shared__ DrawInfo s_info;
   for (int j = threadIdx.x; j < K; j += kThreads) {
-    const int x = __ldg(draft + static_cast<long long>(b) * K + j);
+    const int x = __ldcg(draft + static_cast<long long>(b) * K + j);
     const bool ok = x >= 0 && x < V;  // out of range: no CTA has recorded a logit
     const float lt = __ldcg(dlogit + static_cast<long long>(b) * rows + j);
     const float ld = __ldcg(dlogit + static_cast<long long>(b) * rows + K + 1 + j);
     s_x[j] = x;
     s_zt[j] = ok ? lt : 0.f;
     s_zd[j] = ok ? ld : 0.f;
-    s_u[j] = __ldg(u + static_cast<long long>(b) * (K + 1) + j);
+    s_u[j] = __ldcg(u + static_cast<long long>(b) * (K + 1) + j);
   }
   constexpr int nw = kThreads / 32;
   const int first = n_chunks > 16 ? 16 : (1 << (31 - __clz(2 * n_chunks - 1))) / 2;  // lanes past the chunks hold nothing
@@ -443,25 +443,25 @@ __device__ __forceinline__ void draw_load(const float* rt, const float* rd, int 
   if (vec && v0 + kDrawPer <= V) {
 #pragma unroll
     for (int q = 0; q < kDrawPer / 4; ++q) {
-      const float4 a = __ldg(reinterpret_cast<const float4*>(rt + v0) + q);
+      const float4 a = __ldcg(reinterpret_cast<const float4*>(rt + v0) + q);
       xt[4 * q] = a.x, xt[4 * q + 1] = a.y, xt[4 * q + 2] = a.z, xt[4 * q + 3] = a.w;
-      const float4 d = rd ? __ldg(reinterpret_cast<const float4*>(rd + v0) + q) : make_float4(0.f, 0.f, 0.f, 0.f);
+      const float4 d = rd ? __ldcg(reinterpret_cast<const float4*>(rd + v0) + q) : make_float4(0.f, 0.f, 0.f, 0.f);
       xd[4 * q] = d.x, xd[4 * q + 1] = d.y, xd[4 * q + 2] = d.z, xd[4 * q + 3] = d.w;
     }
   } else if (vec) {
 #pragma unroll
     for (int e = 0; e < kDrawPer; ++e) {
       const bool in = v0 + e < V;
-      xt[e] = in ? __ldg(rt + v0 + e) : -INFINITY;
-      xd[e] = (in && rd) ? __ldg(rd + v0 + e) : 0.f;
+      xt[e] = in ? __ldcg(rt + v0 + e) : -INFINITY;
+      xd[e] = (in && rd) ? __ldcg(rd + v0 + e) : 0.f;
     }
   } else {
 #pragma unroll
     for (int k = 0; k < kDrawPer; ++k) {
       const int i = threadIdx.x + kThreads * k;
       const bool in = c0 + i < V;
-      xt[k] = in ? __ldg(rt + c0 + i) : -INFINITY;
-      xd[k] = (in && rd) ? __ldg(rd + c0 + i) : 0.f;
+      xt[k] = in ? __ldcg(rt + c0 + i) : -INFINITY;
+      xd[k] = (in && rd) ? __ldcg(rd + c0 + i) : 0.f;
     }
 #pragma unroll
     for (int k = 0; k < kDrawPer; ++k) {
@@ -500,10 +500,10 @@ __device__ __forceinline__ float2 block_sum2(float x, float y) {
 // (c + 1) * kDrawChunk), thread t the kDrawPer consecutive values from
 // c * kDrawChunk + t * kDrawPer, summed in order.
 __global__ void __launch_bounds__(kThreads)
-    sample_draw_kernel(const float* __restrict__ zt, const float* __restrict__ zd, int K, int V,
-                       float c2, int n_chunks, bool vec, int n_parts, const int32_t* __restrict__ draft,
-                       const float* __restrict__ u, int32_t* __restrict__ n_emit, int32_t* __restrict__ tokens,
-                       const float2* __restrict__ part, const float* __restrict__ dlogit,
+    sample_draw_kernel(const float* zt, const float* zd, int K, int V,
+                       float c2, int n_chunks, bool vec, int n_parts, const int32_t* draft,
+                       const float* u, int32_t* __restrict__ n_emit, int32_t* __restrict__ tokens,
+                       const float2* part, const float* dlogit,
                        float2* __restrict__ sums, uint32_t* __restrict__ ticket) {
   const int c = blockIdx.x, b = blockIdx.y;
   // a programmatic dependent launch: resident while the statistics finish,
@@ -567,7 +567,7 @@ __global__ void __launch_bounds__(kThreads)
     const float tot_p = __shfl_sync(0xffffffffu, ip, 31);
     const int use_res = (di.ell < K && tot_r > 0.f) ? 1 : 0;
     const float total = use_res ? tot_r : tot_p;
-    const float target = __fmul_rn(u[static_cast<long long>(b) * (K + 1) + K], total);
+    const float target = __fmul_rn(__ldcg(u + static_cast<long long>(b) * (K + 1) + K), total);
     const float incl = use_res ? ir : ip;
     float run = __shfl_up_sync(0xffffffffu, incl, 1);
     if (lane == 0) run = 0.f;

@@ -125,8 +125,8 @@ constexpr int kBlocks = kChunkKeys / (8 * kWarps);  // 8-key blocks a warp takes
 // need only 8 SMs of a GPC and every cluster of a launch fits in one wave
 template <int D>
 __global__ void __launch_bounds__(kThreads, 2)
-    budget_kernel(const __grid_constant__ CUtensorMap tm_k, const __nv_bfloat16* __restrict__ q,
-                  const int32_t* __restrict__ len, const int32_t* __restrict__ n_visual, int R, int Hq,
+    budget_kernel(const __grid_constant__ CUtensorMap tm_k, const __nv_bfloat16* q,
+                  const int32_t* len, const int32_t* n_visual, int R, int Hq,
                   int Hkv, int cap, float scale_log2, bool q_vec, float* __restrict__ mass, float* __restrict__ entropy) {
   static_assert(kPassRows == 32 && kPassRows * kWarps == kThreads, "one thread a (row, warp) in the merge");
   constexpr int kRowChunks = D / 8;  // 16-byte chunks of a query row
@@ -167,17 +167,17 @@ __global__ void __launch_bounds__(kThreads, 2)
       if (p < M) {
         const __nv_bfloat16* src = q + ((static_cast<long long>(b) * R + i) * Hq + kvh * G + (p - i * G)) * D + chunk * 8;
         if (q_vec) {
-          x = *reinterpret_cast<const uint4*>(src);
+          x = __ldcg(reinterpret_cast<const uint4*>(src));
         } else {
           const uint32_t* s4 = reinterpret_cast<const uint32_t*>(src);
-          x = make_uint4(s4[0], s4[1], s4[2], s4[3]);
+          x = make_uint4(__ldcg(s4), __ldcg(s4 + 1), __ldcg(s4 + 2), __ldcg(s4 + 3));
         }
       }
       qs[row * kRowChunks + (chunk ^ (row & 7))] = x;
     }
   };
-  const int n_keys = len[b], L = n_keys - R;
-  int nv = n_visual[b];
+  const int n_keys = __ldcg(len + b), L = n_keys - R;
+  int nv = __ldcg(n_visual + b);
   // every CTA of a cluster runs the same barriers, so a bad length only
   // empties the key ranges (and writes nothing)
   const bool ok = L >= 0 && n_keys <= cap;

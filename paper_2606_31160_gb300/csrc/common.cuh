@@ -118,6 +118,16 @@ __device__ __forceinline__ void sd_pdl_enter() {
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
 
+// Loads of what an earlier kernel may write, in a kernel that is resident while
+// that kernel runs: through L2, coherent (__ldcg). The read-only path (__ldg, and
+// what the compiler makes of a const __restrict__ parameter) is for memory that
+// nobody writes while the kernel lives, and such a kernel lives from before its
+// wait. CUDA's __ldcg of a bf16 is an asm that the compiler may move across the
+// wait; the 16-bit one is volatile.
+__device__ __forceinline__ float sd_ldcg_bf16(const __nv_bfloat16* p) {
+  return __uint_as_float(static_cast<uint32_t>(__ldcg(reinterpret_cast<const unsigned short*>(p))) << 16);
+}
+
 __device__ __forceinline__ float sd_bf16_lo(uint32_t w) { return __uint_as_float(w << 16); }
 __device__ __forceinline__ float sd_bf16_hi(uint32_t w) { return __uint_as_float(w & 0xffff0000u); }
 

@@ -17,8 +17,7 @@ namespace {
 
 __global__ void __launch_bounds__(512) kv_append_kernel(uint4* __restrict__ kc, uint4* __restrict__ vc,
                                                         int32_t* __restrict__ len,
-                                                        const uint4* __restrict__ kn,
-                                                        const uint4* __restrict__ vn, int R, int hkv,
+                                                        const uint4* kn, const uint4* vn, int R, int hkv,
                                                         int cap, int vec_per_row) {
   sd_pdl_enter();
   const int b = blockIdx.x;
@@ -33,15 +32,28 @@ __global__ void __launch_bounds__(512) kv_append_kernel(uint4* __restrict__ kc, 
   const int l0 = s_len;
   if (l0 < 0) return;
   const int per_scene = R * hkv * vec_per_row;
-  for (int i = threadIdx.x; i < per_scene; i += blockDim.x) {
-    const int vec = i % vec_per_row;
-    const int t = i / vec_per_row;
-    const int g = t % hkv;
-    const int r = t / hkv;
-    const long long src = ((long long)b * per_scene) + i;                 // [b][r][g][vec]
-    const long long dst = (((long long)b * hkv + g) * cap + (l0 + r)) * vec_per_row + vec;
-    kc[dst] = kn[src];
-    vc[dst] = vn[src];
+  kn += static_cast<long long>(b) * per_scene;  // [b][r][g][vec]
+  vn += static_cast<long long>(b) * per_scene;
+  constexpr int kBatch = 4;  // chunks a thread has in flight
+  for (int i0 = threadIdx.x; i0 < per_scene; i0 += kBatch * blockDim.x) {
+    uint4 k[kBatch], v[kBatch];
+#pragma unroll
+    for (int u = 0; u < kBatch; ++u) {
+      const int i = i0 + u * blockDim.x;
+      if (i < per_scene) k[u] = __ldcg(kn + i), v[u] = __ldcg(vn + i);
+    }
+#pragma unroll
+    for (int u = 0; u < kBatch; ++u) {
+      const int i = i0 + u * blockDim.x;
+      if (i >= per_scene) break;
+      const int vec = i % vec_per_row;
+      const int t = i / vec_per_row;
+      const int g = t % hkv;
+      const int r = t / hkv;
+      const long long dst = (((long long)b * hkv + g) * cap + (l0 + r)) * vec_per_row + vec;
+      kc[dst] = k[u];
+      vc[dst] = v[u];
+    }
   }
   __syncthreads();
   if (threadIdx.x == 0) len[b] = l0 + R;
@@ -55,7 +67,7 @@ __global__ void __launch_bounds__(512) kv_append_kernel(uint4* __restrict__ kc, 
 // together, the rotation's table is read before the wait.
 template <int D>
 __global__ void __launch_bounds__(512) rope_append_kernel(uint4* __restrict__ q, uint4* __restrict__ kn,
-                                                          const uint4* __restrict__ vn, const int32_t* __restrict__ pos,
+                                                          const uint4* vn, const int32_t* pos,
                                                           uint4* __restrict__ kc, uint4* __restrict__ vc,
                                                           int32_t* __restrict__ len, int R, int hq, int hkv, int cap,
                                                           const __grid_constant__ RopeTable tab) {
@@ -69,7 +81,7 @@ __global__ void __launch_bounds__(512) rope_append_kernel(uint4* __restrict__ q,
     if (i >= n) return;
     const int32_t* p3 = pos + i / (kVec * hq) * 3;
     uint4* x = q + b * n + i;
-    *x = sd_rope_rotate8(*x, p3[0], p3[1], p3[2], chunk);
+    *x = sd_rope_rotate8(*x, __ldcg(p3), __ldcg(p3 + 1), __ldcg(p3 + 2), chunk);
     return;
   }
   const int l0 = len[b], n = R * hkv * kVec;
@@ -77,8 +89,8 @@ __global__ void __launch_bounds__(512) rope_append_kernel(uint4* __restrict__ q,
   for (int i = threadIdx.x; i < n; i += 512) {
     const int t = i / kVec, g = t % hkv, r = t / hkv;
     const long long src = static_cast<long long>(b) * n + i;  // [b][r][g][vec]
-    const uint4 k = kn[src], v = vn[src];
-    const uint4 kr = sd_rope_rotate8(k, pos[r * 3], pos[r * 3 + 1], pos[r * 3 + 2], chunk);
+    const uint4 k = kn[src], v = __ldcg(vn + src);
+    const uint4 kr = sd_rope_rotate8(k, __ldcg(pos + r * 3), __ldcg(pos + r * 3 + 1), __ldcg(pos + r * 3 + 2), chunk);
     kn[src] = kr;
     if (ok) {
       const long long dst = ((static_cast<long long>(b) * hkv + g) * cap + (l0 + r)) * kVec + vec;
@@ -94,11 +106,11 @@ __global__ void __launch_bounds__(512) rope_append_kernel(uint4* __restrict__ q,
 }
 
 __global__ void kv_rollback_kernel(int32_t* __restrict__ len, int count, int B,
-                                   const int32_t* __restrict__ committed, int n_appended) {
+                                   const int32_t* committed, int n_appended) {
   sd_pdl_enter();
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= count) return;
-  const int c = committed[i % B];
+  const int c = __ldcg(committed + i % B);
   const int l = len[i];
   const int nl = l - n_appended + c;
   if (c < 0 || c > n_appended || nl < 0) {

@@ -26,7 +26,7 @@ template <int D, bool kFlat>
 __global__ void __launch_bounds__(256) rope_kernel(__nv_bfloat16* __restrict__ q,
                                                    __nv_bfloat16* __restrict__ k,
                                                    int rows, int hq, int hkv,
-                                                   const int32_t* __restrict__ pos,
+                                                   const int32_t* pos,
                                                    RopeTable tab) {
   constexpr int kVecPerHead = D / 8;
   // every chunk of a thread is the same one of its head: the stride is a multiple of D / 8
@@ -45,7 +45,8 @@ __global__ void __launch_bounds__(256) rope_kernel(__nv_bfloat16* __restrict__ q
     uint4* ptr = reinterpret_cast<uint4*>(base) + vec;
     const uint4 v = *ptr;
     const int32_t* pr = pos + (kFlat ? row : row * 3);
-    *ptr = sd_rope_rotate8(v, pr[0], pr[kFlat ? 0 : 1], pr[kFlat ? 0 : 2], chunk);
+    const int pt = __ldcg(pr), ph = kFlat ? pt : __ldcg(pr + 1), pw = kFlat ? pt : __ldcg(pr + 2);
+    *ptr = sd_rope_rotate8(v, pt, ph, pw, chunk);
   }
 }
 
