@@ -25,7 +25,9 @@
 //
 // The new rows stay out of the loop: the cluster's last rank holds the R (rotated)
 // new keys and values in shared memory, scores them by mma.sync, 8 rows by 16 keys a
-// warp, and adds one PV product of 16 or 32 keys. Scored on the CUDA cores by the
+// warp, and adds one PV product of 16 or 32 keys, its weights to 16 bits in two bf16
+// terms: with one term the error at an empty prefix was 2.1e-3 against the 1.66e-3 of
+// the output's rounding. Scored on the CUDA cores by the
 // rows a CTA merges instead, rows x new keys took 26 us a launch at one CTA a head
 // and K = 16.
 //
@@ -100,8 +102,10 @@ struct Cfg {
   static constexpr bool kNewFirst = kR == 32;
   static constexpr int kOffPNew = kOffP + (kNewFirst ? kPBuf : 2 * kPBuf);
   static constexpr int kPNewGroup = kNewFirst ? kPGroup : kMaxNew * 32;
-  static constexpr int kPNewLow = kNewFirst ? kP : (kR / 16) * kPNewGroup;  // from the high to the low terms
-  static constexpr int kOffBar = kNewFirst ? kOffP + 2 * kPBuf : kOffPNew + (kSplit ? 2 : 1) * kPNewLow;
+  // from the high to the low terms (two for head dim 128 too: these weights were fp32 where
+  // the new keys were merged on the CUDA cores): in P buffer 1 the 16 keys after the 16 new ones
+  static constexpr int kPNewLow = kNewFirst ? kMaxNew * 32 : (kR / 16) * kPNewGroup;
+  static constexpr int kOffBar = kNewFirst ? kOffP + 2 * kPBuf : kOffPNew + 2 * kPNewLow;
   // full_k[S] full_v[S] p_full[2] s_ready[3] s_free[3] pv_done[S] p_new new_done recv decide maxima tmem_done
   static constexpr int kNumBars = 3 * kStages + 14;
   static constexpr int kOffMisc = round_up(kOffBar + kNumBars * 8, 16);
@@ -578,7 +582,7 @@ __global__ void __launch_bounds__(kThreads, 1)
           for (int kk = 0; kk < C::kMaxNew / 16; ++kk)
             if (kk * 16 < a.R) {
               umma(tmem_o, dN + (kk * 2048 >> 4), dpn + (kk * 512 >> 4), kIdescO, kk > 0 || add ? 1 : 0);
-              if (C::kSplit) umma(tmem_o, dN + (kk * 2048 >> 4), dpn + ((C::kPNewLow + kk * 512) >> 4), kIdescO, 1);
+              umma(tmem_o, dN + (kk * 2048 >> 4), dpn + ((C::kPNewLow + kk * 512) >> 4), kIdescO, 1);
             }
           umma_commit(NEWDONE);
         }
@@ -850,15 +854,13 @@ __global__ void __launch_bounds__(kThreads, 1)
           const float e1 = key <= lim1 ? ex2(fmaf(c[2 * h + 1] + c1[2 * h + 1], sl, nr.y)) : 0.f;
           uint32_t hi, lo = 0;
           uint64_t l;
-          weight_terms<C::kSplit>(e0, e1, hi, lo, l);
-          float x0, x1;
-          unpack2(l, x0, x1);
-          l0 += x0;
-          l1 += x1;
+          weight_terms<true>(e0, e1, hi, lo, l);
+          l0 += e0;
+          l1 += e1;
           const uint32_t dst = base + C::kOffPNew + (unit >> 1) * C::kPNewGroup + key * 32 +
                                (((unit & 1) ^ ((key >> 2) & 1)) << 4) + (lane & 3) * 4;
           asm volatile("st.shared.u32 [%0], %1;" ::"r"(dst), "r"(hi) : "memory");
-          if (C::kSplit) asm volatile("st.shared.u32 [%0], %1;" ::"r"(dst + C::kPNewLow), "r"(lo) : "memory");
+          asm volatile("st.shared.u32 [%0], %1;" ::"r"(dst + C::kPNewLow), "r"(lo) : "memory");
         }
       }
       asm volatile("fence.proxy.async.shared::cta;" ::: "memory");

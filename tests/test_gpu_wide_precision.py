@@ -1,0 +1,69 @@
+"""Error of the row-tile attention against 64 bits where few keys hold the mass.
+
+Every bound is the rounding of an exact output to bf16 on the same inputs, with 1% for
+the weights (2^-17 each, beside the output's 2^-9) and the fp32 scores."""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+from paper_2606_31160_gb300 import sd, workloads
+from tests.helpers import ensure_lib, to64
+
+pytestmark = pytest.mark.gpu
+# packed rows 1, 32 | 48 | 64 | 68, 80 | 96 (two m-blocks)
+SHAPES = [(1, 1), (4, 8), (2, 16), (4, 12), (4, 16), (4, 17), (5, 16), (6, 16)]
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _lib():
+    ensure_lib()
+
+
+def _bf(x):
+    return to64(workloads.to_bf16(x))
+
+
+def _inputs(seed, B, G, R, Hkv, cap, D, v_scale=1.0):
+    rng = np.random.default_rng(seed)
+    draw = lambda *s: rng.standard_normal(s).astype(np.float32)  # noqa: E731
+    return [draw(B, R, Hkv * G, D), draw(B, Hkv, cap, D), draw(B, Hkv, cap, D) * np.float32(v_scale), draw(B, R, Hkv, D),
+            draw(B, R, Hkv, D) * np.float32(v_scale)]
+
+
+def _call(q, k, v, k_new, v_new, prefix, fused):
+    """Position-0 new rows (an identity rotation); returns (out, q, keys, values, lengths) in 64 bits."""
+    B, R, Hq, D = q.shape
+    bf = workloads.to_bf16
+    kc, vc = k.copy(), v.copy()
+    for b, n in enumerate(prefix):
+        if not fused:
+            kc[b, :, n:n + R] = k_new[b].transpose(1, 0, 2)
+            vc[b, :, n:n + R] = v_new[b].transpose(1, 0, 2)
+    cache = sd.KVCache(bf(kc).cuda(), bf(vc).cuda(),
+                       torch.tensor([n + (0 if fused else R) for n in prefix], dtype=torch.int32).cuda())
+    qd = bf(q).cuda()
+    if fused:
+        sections = (16, 24, 24) if D == 128 else (8, 12, 12)
+        out = sd.verify_layer(qd, bf(k_new).cuda(), bf(v_new).cuda(), torch.zeros((B, R, 3), dtype=torch.int32).cuda(),
+                              sections, cache, 0, 1e6)
+    else:
+        out = sd.verify_attention(qd, cache)
+    torch.cuda.synchronize()
+    assert sd.get_device_error() == 0
+    return to64(out), to64(qd), to64(cache.k), to64(cache.v), cache.len.cpu().numpy()
+
+
+def _rel(x, ref):
+    return float(np.sqrt(((x - ref) ** 2).sum() / (ref ** 2).sum()))
+
+
+@pytest.mark.parametrize("G,R", SHAPES)
+@pytest.mark.parametrize("fused", [True, False])
+def test_new_keys_alone(G, R, fused):
+    """Without a prefix the weights are those of the new keys, 16 bits and more: what is left
+    is the rounding of the output."""
+    q, k, v, k_new, v_new = _inputs(31 * G + R, 6, G, R, 2, 40, 128)
+    out, *rest = _call(q, k, v, k_new, v_new, [0] * 6, fused)
+    ref = oracle.verify_attention(*rest)
+    assert _rel(out, ref) <= 1.01 * _rel(_bf(ref.astype(np.float32)), ref) + 1e-6
