@@ -837,9 +837,11 @@ static bool tc_enabled() {
 }
 
 // How the tcgen05 path runs a shape: row tile, its packed rows, m-blocks (row
-// tiles per KV head) and cluster size; cs == 0: not served.
+// tiles per KV head), cluster size and whether the weights are two bf16 terms
+// where the tile has both forms; cs == 0: not served.
 struct TcPlan {
   int tile = kWide32, rows = 0, mblocks = 0, cs = 0;
+  bool split = false;
 };
 
 // Cluster size forced by sd_set_cluster_size (0: chosen per call).
@@ -861,7 +863,8 @@ extern "C" sd_status sd_set_cluster_size(int cluster_size) {
 // The tile and cluster size of a shape: up to 31 new rows beside the prefix loop
 // on the smallest wide tile that holds the packed rows in one m-block (every key
 // read once), above 80 rows on two; more new rows with every key in the loop
-// (all_keys). The 32-row tile holds 16 new rows.
+// (all_keys). The 32-row tile holds 16 new rows; 17 to 31 of one query head each
+// take the 48-row tile with the weights in two terms.
 static TcPlan tc_plan(int B, int R, int Hq, int Hkv, int D, int cap, bool all_keys) {
   TcPlan p;
   if (!tc_enabled() || (D != kD && (D != 64 || all_keys)) || Hkv <= 0 || Hq % Hkv || R <= 0) return p;
@@ -871,6 +874,7 @@ static TcPlan tc_plan(int B, int R, int Hq, int Hkv, int D, int cap, bool all_ke
     p.tile = kAll64;
   } else {
     if (R > 31) return p;
+    p.split = M <= 32 && R > 16;
     p.tile = M <= 32 && R <= 16 ? kWide32 : (M <= 48 ? kWide48 : (M <= 64 ? kWide64 : (M <= 80 ? kWide80 : (M <= 96 ? kWide48 : kWide64))));
   }
   p.rows = all_keys ? 64 : kTileRows[p.tile];
@@ -955,7 +959,7 @@ sd_status sd_internal_verify_attention_tc(const void* q, const sd_kv_cache* cach
     // a programmatic dependent launch either way: without the flag the kernel
     // waits before its first global access, so only its launch and set-up
     // (barriers, tensor memory) overlap the kernel before it
-    return sd_internal_wide_launch(cache, a, tab, plan.rows, plan.cs, false, stream);
+    return sd_internal_wide_launch(cache, a, tab, plan.rows, plan.split, plan.cs, false, stream);
   }
   a.early = block ? 1 : 0;  // the all-keys kernel's block mask
   return launch_tc<64>(cache, a, plan, stream);
@@ -997,5 +1001,5 @@ sd_status sd_internal_verify_layer_tc(void* q, void* k_new, const void* v_new, c
   // without the early prefix a dependent launch as well: the wait comes before any
   // global access (the draft's single-row steps, each reading the length the step
   // before advanced)
-  return sd_internal_wide_launch(cache, a, tab, plan.rows, plan.cs, true, stream);
+  return sd_internal_wide_launch(cache, a, tab, plan.rows, plan.split, plan.cs, true, stream);
 }

@@ -65,7 +65,7 @@ constexpr int kSoft0 = 32 * kFirstSoft;  // the first softmax thread
 constexpr int kThreads = kSoft0 + kSoftThreads;
 constexpr float kHigh = 18446744073709551616.f;          // 2^64: a larger row sum runs the range again
 constexpr float kLow = 8.271806125530277e-25f;           // 2^-80: a smaller one too
-template <int kR, int kDim>
+template <int kR, int kDim, bool kSplitWeights>
 struct Cfg {
   static_assert(kR == 32 || kR == 48 || kR == 64 || kR == 80, "row tile");
   static_assert(kDim == 64 || kDim == 128, "head dim");
@@ -85,10 +85,13 @@ struct Cfg {
   // 16-row groups kPGroup apart
   static constexpr int kPGroup = kStageKeys * 32;
   static constexpr int kP = (kR / 16) * kPGroup;
-  // head dim 64 keeps the weights to 16 bits as two bf16 terms (two PV products): the
-  // mma.sync kernel that served it rounds weights below a running maximum, which is
-  // 14% closer to 64 bits than one term without a reference (2.1e-3 against 2.4e-3)
-  static constexpr bool kSplit = kDim == 64;
+  // whether the weights are kept to 16 bits as two bf16 terms (two PV products). Head
+  // dim 64 is: the mma.sync kernel that served it rounds weights below a running maximum,
+  // which is 14% closer to 64 bits than one term without a reference (2.1e-3 against
+  // 2.4e-3). So are 17 to 31 packed rows of a query head each at head dim 128, which ran
+  // with their first tile's maximum as reference (largest weight exact: 1.8e-3 against
+  // 2.1e-3 at a prefix of one tile)
+  static constexpr bool kSplit = kSplitWeights;
   static constexpr int kPBuf = kSplit ? 2 * kP : kP;  // a group's P buffer: the high terms, then the low ones
   static constexpr int kSStride = kR == 32 ? 32 : (kR <= 64 ? 64 : 128);  // columns between S0 | S1 | S2 | O
   static constexpr int kTmemCols = 4 * kSStride;
@@ -277,11 +280,11 @@ __device__ __noinline__ float new_key_max(const uint8_t* q, int row, int q_half,
 // and pos may be read before the dependency wait; bit 1: the block mask. Grid:
 // (cluster size, Hkv * n_mblocks, B); m-block mb takes packed rows mb * kR ..
 // mb * kR + kR - 1.
-template <int kR, int kDim, bool kFused>
+template <int kR, int kDim, bool kFused, bool kSplitWeights>
 __global__ void __launch_bounds__(kThreads, 1)
     verify_wide_kernel(const __grid_constant__ CUtensorMap tm_k128, const __grid_constant__ CUtensorMap tm_v128,
                        const TcArgs a, const RopeTable tab) {
-  using C = Cfg<kR, kDim>;
+  using C = Cfg<kR, kDim, kSplitWeights>;
   constexpr int kHalves = C::kHalves, kChunks = C::kChunks, kKV = C::kKV;
   constexpr int kRowL = C::kRowL, kRowM = C::kRowM, kRowF = C::kRowF, kRowBytes = C::kRowBytes;
   constexpr int kS = C::kStages;
@@ -1186,12 +1189,12 @@ __global__ void __launch_bounds__(kThreads, 1)
 }
 
 // ------------------------------------------------------------------ host
-template <int kR, int kDim>
+template <int kR, int kDim, bool kSplitWeights>
 bool set_attributes(const int* sizes, int n, int* active) {
   // (head dim 64 layers run as the rotation, append and attention kernels)
-  const void* kerns[2] = {reinterpret_cast<const void*>(verify_wide_kernel<kR, kDim, false>),
-                          reinterpret_cast<const void*>(verify_wide_kernel<kR, kDim, kDim == 128>)};
-  constexpr int smem = Cfg<kR, kDim>::kSmemBytes;
+  const void* kerns[2] = {reinterpret_cast<const void*>(verify_wide_kernel<kR, kDim, false, kSplitWeights>),
+                          reinterpret_cast<const void*>(verify_wide_kernel<kR, kDim, kDim == 128, kSplitWeights>)};
+  constexpr int smem = Cfg<kR, kDim, kSplitWeights>::kSmemBytes;
   for (const void* k : kerns)
     if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess ||
         cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) {
@@ -1220,7 +1223,7 @@ bool set_attributes(const int* sizes, int n, int* active) {
   return true;
 }
 
-template <int kR, int kDim, bool kFused>
+template <int kR, int kDim, bool kFused, bool kSplitWeights>
 sd_status launch(const sd_kv_cache* cache, const TcArgs& a, const RopeTable& tab, int cs, cudaStream_t stream) {
   const int B = cache->batch, Hkv = cache->n_kv_heads, cap = cache->capacity;
   CUtensorMap k128, v128;
@@ -1236,11 +1239,11 @@ sd_status launch(const sd_kv_cache* cache, const TcArgs& a, const RopeTable& tab
   attr[1].val.programmaticStreamSerializationAllowed = 1;
   cfg.gridDim = dim3(cs, Hkv * a.n_mblocks, B);
   cfg.blockDim = dim3(kThreads, 1, 1);
-  cfg.dynamicSmemBytes = Cfg<kR, kDim>::kSmemBytes;
+  cfg.dynamicSmemBytes = Cfg<kR, kDim, kSplitWeights>::kSmemBytes;
   cfg.stream = stream;
   cfg.attrs = attr;
   cfg.numAttrs = 2;
-  if (cudaLaunchKernelEx(&cfg, verify_wide_kernel<kR, kDim, kFused>, k128, v128, a, tab) != cudaSuccess) {
+  if (cudaLaunchKernelEx(&cfg, verify_wide_kernel<kR, kDim, kFused, kSplitWeights>, k128, v128, a, tab) != cudaSuccess) {
     (void)cudaGetLastError();
     return SD_ERR_CUDA;
   }
@@ -1248,20 +1251,23 @@ sd_status launch(const sd_kv_cache* cache, const TcArgs& a, const RopeTable& tab
 }
 
 template <int kDim, bool kFused>
-sd_status launch_rows(const sd_kv_cache* cache, const TcArgs& a, const RopeTable& tab, int rows, int cs,
+sd_status launch_rows(const sd_kv_cache* cache, const TcArgs& a, const RopeTable& tab, int rows, bool split, int cs,
                       cudaStream_t stream) {
-  if (rows == 32) return launch<32, kDim, kFused>(cache, a, tab, cs, stream);
-  if (rows == 48) return launch<48, kDim, kFused>(cache, a, tab, cs, stream);
-  if (rows == 64) return launch<64, kDim, kFused>(cache, a, tab, cs, stream);
-  return launch<80, kDim, kFused>(cache, a, tab, cs, stream);
+  constexpr bool kAll = kDim == 64;  // two terms on every tile
+  if (rows == 32) return launch<32, kDim, kFused, kAll>(cache, a, tab, cs, stream);
+  if (rows == 48 && split) return launch<48, kDim, kFused, true>(cache, a, tab, cs, stream);
+  if (rows == 48) return launch<48, kDim, kFused, kAll>(cache, a, tab, cs, stream);
+  if (rows == 64) return launch<64, kDim, kFused, kAll>(cache, a, tab, cs, stream);
+  return launch<80, kDim, kFused, kAll>(cache, a, tab, cs, stream);
 }
 
 template <int kDim>
 bool active_of(int rows, const int* sizes, int n, int* active) {
-  if (rows == 32) return set_attributes<32, kDim>(sizes, n, active);
-  if (rows == 48) return set_attributes<48, kDim>(sizes, n, active);
-  if (rows == 64) return set_attributes<64, kDim>(sizes, n, active);
-  return set_attributes<80, kDim>(sizes, n, active);
+  constexpr bool kAll = kDim == 64;
+  if (rows == 32) return set_attributes<32, kDim, kAll>(sizes, n, active);
+  if (rows == 48) return set_attributes<48, kDim, true>(sizes, n, active) && set_attributes<48, kDim, kAll>(sizes, n, active);
+  if (rows == 64) return set_attributes<64, kDim, kAll>(sizes, n, active);
+  return set_attributes<80, kDim, kAll>(sizes, n, active);
 }
 
 }  // namespace
@@ -1270,9 +1276,9 @@ bool sd_internal_wide_active(int rows, int D, const int* sizes, int n, int* acti
   return D == 64 ? active_of<64>(rows, sizes, n, active) : active_of<128>(rows, sizes, n, active);
 }
 
-sd_status sd_internal_wide_launch(const sd_kv_cache* cache, const TcArgs& a, const RopeTable& tab, int rows, int cs,
-                                  bool fused, cudaStream_t stream) {
-  if (cache->head_dim == 64) return launch_rows<64, false>(cache, a, tab, rows, cs, stream);
-  return fused ? launch_rows<128, true>(cache, a, tab, rows, cs, stream)
-               : launch_rows<128, false>(cache, a, tab, rows, cs, stream);
+sd_status sd_internal_wide_launch(const sd_kv_cache* cache, const TcArgs& a, const RopeTable& tab, int rows, bool split,
+                                  int cs, bool fused, cudaStream_t stream) {
+  if (cache->head_dim == 64) return launch_rows<64, false>(cache, a, tab, rows, split, cs, stream);
+  return fused ? launch_rows<128, true>(cache, a, tab, rows, split, cs, stream)
+               : launch_rows<128, false>(cache, a, tab, rows, split, cs, stream);
 }

@@ -36,8 +36,8 @@ struct TcArgs {
 // attention_wide.cu: clusters of each size that fit at once (false: not
 // available here), and the launch on row tiles of `rows` (32, 48, 64, 80).
 bool sd_internal_wide_active(int rows, int D, const int* sizes, int n, int* active);
-sd_status sd_internal_wide_launch(const sd_kv_cache* cache, const TcArgs& a, const RopeTable& tab, int rows, int cs,
-                                  bool fused, cudaStream_t stream);
+sd_status sd_internal_wide_launch(const sd_kv_cache* cache, const TcArgs& a, const RopeTable& tab, int rows, bool split,
+                                  int cs, bool fused, cudaStream_t stream);
 
 namespace {
 
