@@ -191,8 +191,8 @@ sd_status sd_verify_attention(const void* q, const sd_kv_cache* cache, void* out
  * SD_ATTN_PREFIX_EARLY declares that the kernel issued just before this call
  * on the stream writes neither this cache (its K / V rows, the new rows
  * included) nor its len (true when a step's layers are issued back to back
- * after their appends). For head_dim 128 and up to 31 new rows
- * the call is then a programmatic dependent launch that reads len
+ * after their appends). For head_dim 128 and up to 31 new rows (32 with one
+ * query head a KV head) the call is then a programmatic dependent launch that reads len
  * and streams the whole cache while its predecessor still runs, and reads q
  * only after the predecessor has completed; other shapes ignore the flag.
  * Without the flag those shapes are programmatic dependent launches too, but

@@ -3,10 +3,10 @@
 // cached prefix (Eq. verify, Sec. 3.2) and the fused verify layer (M-RoPE of
 // Sec. 3.3 / Sec. 4.2 + the KV append of Eq. commit + the attention).
 //
-// Up to 31 new rows take the row tiles of attention_wide.cu, whose loop covers the
-// prefix and whose new rows enter beside it. With more (32 to 128, so at most 4
-// query heads a KV head) the attention runs here, every key in the loop, in
-// m-blocks of 64 packed rows:
+// Up to 31 new rows (32 with one query head a KV head) take the row tiles of
+// attention_wide.cu, whose loop covers the prefix and whose new rows enter beside it.
+// With more (32 to 128, so at most 4 query heads a KV head) the attention runs here,
+// every key in the loop, in m-blocks of 64 packed rows:
 //     S^T[128 keys][64 rows] = K_tile[128 keys][128 d] . Q^T      (K-major A, B)
 //     O^T[128 d][64 rows]   += V_tile^T[128 d][128 keys] . P^T     (MN-major A, B)
 // Both accumulators live in tensor memory, S triple-buffered.
@@ -863,9 +863,11 @@ extern "C" sd_status sd_set_cluster_size(int cluster_size) {
 // The tile and cluster size of a shape: up to 31 new rows beside the prefix loop
 // on the smallest wide tile that holds the packed rows in one m-block (every key
 // read once), above 80 rows on two; more new rows with every key in the loop
-// (all_keys). The 32-row tile holds 16 new rows; 17 to 31 of one query head each
-// take the 48-row tile with the weights in two terms.
-static TcPlan tc_plan(int B, int R, int Hq, int Hkv, int D, int cap, bool all_keys) {
+// (all_keys). The 32-row tile holds 16 new rows; 17 to 32 of one query head each
+// take the 48-row tile with the weights in two terms (32 of them, 32 scenes of 8 heads,
+// L = 2048: 45.1 us, against 60.7 on the all-keys kernel's 64 rows; 4 scenes, L = 700:
+// 7.7 against 14.2). A layer of 32 new rows stays three kernels.
+static TcPlan tc_plan(int B, int R, int Hq, int Hkv, int D, int cap, bool all_keys, bool layer = false) {
   TcPlan p;
   if (!tc_enabled() || (D != kD && (D != 64 || all_keys)) || Hkv <= 0 || Hq % Hkv || R <= 0) return p;
   const int M = (Hq / Hkv) * R;
@@ -873,7 +875,7 @@ static TcPlan tc_plan(int B, int R, int Hq, int Hkv, int D, int cap, bool all_ke
   if (all_keys) {
     p.tile = kAll64;
   } else {
-    if (R > 31) return p;
+    if (R > 31 && !(R == 32 && M == 32 && D == kD && !layer)) return p;
     p.split = M <= 32 && R > 16;
     p.tile = M <= 32 && R <= 16 ? kWide32 : (M <= 48 ? kWide48 : (M <= 64 ? kWide64 : (M <= 80 ? kWide80 : (M <= 96 ? kWide48 : kWide64))));
   }
@@ -895,7 +897,7 @@ bool sd_internal_tc_serves(int B, int R, int Hq, int Hkv, int D, int cap) {
 }
 
 bool sd_internal_tc_serves_layer(int B, int R, int Hq, int Hkv, int D, int cap) {
-  return D == kD && tc_plan(B, R, Hq, Hkv, D, cap, false).cs > 0;
+  return D == kD && tc_plan(B, R, Hq, Hkv, D, cap, false, true).cs > 0;
 }
 
 template <int kR>
@@ -923,7 +925,8 @@ static sd_status launch_tc(const sd_kv_cache* cache, const TcArgs& a, const TcPl
   return SD_OK;
 }
 
-// Routed here by sd_verify_attention for G * R <= 128. Up to 31 new rows take the wide tiles, whose loop covers the prefix only, with the
+// Routed here by sd_verify_attention for G * R <= 128. Up to 31 new rows (32 of one
+// query head each) take the wide tiles, whose loop covers the prefix only, with the
 // prefix optionally streamed before the dependency wait (SD_ATTN_PREFIX_EARLY);
 // more take the kernel whose loop covers every key (the flag is then a promise it
 // does not need).
@@ -973,7 +976,7 @@ sd_status sd_internal_verify_layer_tc(void* q, void* k_new, const void* v_new, c
   *handled = false;
   const int B = cache->batch, Hkv = cache->n_kv_heads;
   if (cache->head_dim != kD) return SD_OK;
-  const TcPlan plan = tc_plan(B, R, Hq, Hkv, cache->head_dim, cache->capacity, false);
+  const TcPlan plan = tc_plan(B, R, Hq, Hkv, cache->head_dim, cache->capacity, false, true);
   if (plan.cs <= 0) return SD_OK;
   TcArgs a = {};
   a.q = static_cast<const __nv_bfloat16*>(q);

@@ -88,7 +88,7 @@ struct Cfg {
   // whether the weights are kept to 16 bits as two bf16 terms (two PV products). Head
   // dim 64 is: the mma.sync kernel that served it rounds weights below a running maximum,
   // which is 14% closer to 64 bits than one term without a reference (2.1e-3 against
-  // 2.4e-3). So are 17 to 31 packed rows of a query head each at head dim 128, which ran
+  // 2.4e-3). So are 17 to 32 packed rows of a query head each at head dim 128, which ran
   // with their first tile's maximum as reference (largest weight exact: 1.8e-3 against
   // 2.1e-3 at a prefix of one tile)
   static constexpr bool kSplit = kSplitWeights;

@@ -69,11 +69,11 @@ def test_new_keys_alone(G, R, fused):
     assert _rel(out, ref) <= 1.01 * _rel(_bf(ref.astype(np.float32)), ref) + 1e-6
 
 
-@pytest.mark.parametrize("R", [17, 24, 31])
+@pytest.mark.parametrize("R", [17, 24, 31, 32])
 @pytest.mark.parametrize("fused", [True, False])
 @pytest.mark.parametrize("csize,prefix", [(1, [1, 7, 32, 100, 128, 200]), (4, [200, 320, 500, 512, 600, 700])])
 def test_many_rows_of_one_head(R, fused, csize, prefix):
-    """17 to 31 new rows of one query head a KV head: the weights of the prefix to 16 bits too."""
+    """17 to 32 new rows of one query head a KV head: the weights of the prefix to 16 bits too."""
     q, k, v, k_new, v_new = _inputs(7 + R + csize, len(prefix), 1, R, 2, 760, 128)
     sd.set_cluster_size(csize)
     try:
