@@ -15,7 +15,7 @@
 // 153 -> 142 us, K = 8 165 -> 143, 1.0 of the measured copy). With one scene the
 // dependent path behind the previous kernel: rows, rotation, S(0), the tiles at
 // ~0.4 us of products each, the exchange (~0.7 us), the merge (target layer
-// 6.77 -> 6.24 us, K = 8 10.0 -> 7.2, K = 16 block 15.9 -> 10.4, draft step 6.8 -> 5.9
+// 6.77 -> 6.45 us, K = 8 10.0 -> 7.4, K = 16 block 15.9 -> 10.7, draft step 6.8 -> 6.0
 // on one cache).
 //
 // Head dim 64 (the attention; its layers run as the rotation, append and attention
@@ -27,16 +27,20 @@
 // new keys and values in shared memory, scores them by mma.sync, 8 rows by 16 keys a
 // warp, and adds one PV product of 16 or 32 keys, its weights to 16 bits in two bf16
 // terms: with one term the error at an empty prefix was 2.1e-3 against the 1.66e-3 of
-// the output's rounding. Scored on the CUDA cores by the
-// rows a CTA merges instead, rows x new keys took 26 us a launch at one CTA a head
-// and K = 16.
+// the output's rounding. Scored on the CUDA cores by the rows a CTA merges instead,
+// rows x new keys took 26 us a launch at one CTA a head and K = 16.
 //
-// Fixed reference. Weights are 2^(score * scale) with no reference subtracted: a
-// floating-point weight keeps its relative precision at any size, so only overflow
-// and underflow matter. A row sum above 2^64, or no lane of a warp with every sum
-// above 2^-80, sends the CTA through its range again with each row's exact maximum
-// as its reference: one pass for the maxima, one for the weights. No reduction and
-// no reference product stands between S and P.
+// Fixed reference. Weights are 2^(score * scale - ref) with the row's score against its
+// own new key as its reference on every CTA of the cluster: the row's sum is about 1 or
+// more, scores may have any common offset, and the CTAs' partials add as they are. (Row
+// and key turn by the same angles, so the unrotated ones give it, while they are in
+// registers; nothing stands between S and P.) A floating-point weight keeps its relative
+// precision at any size, so only overflow matters: a row sum above 2^64 sends the CTA
+// through its range again with each row's exact maximum as its reference, one pass for
+// the maxima and one for the weights. Without a reference scores 40 away from 0 took
+// those passes (8 scenes, L = 8192, K = 7: 38 -> 102 us), and values far from 1 left
+// fp32's range in the product; the references cost a chained layer 0.2 us, the others
+// nothing.
 //
 // Warps (608 threads): 0 the TMA producer, whose first tiles go out before the CTA's
 // set-up is over; 1 issues S and owns tensor memory; 2 issues PV; 3..18 two softmax
@@ -64,7 +68,6 @@ constexpr int kFirstSoft = 3;            // the first softmax warp
 constexpr int kSoft0 = 32 * kFirstSoft;  // the first softmax thread
 constexpr int kThreads = kSoft0 + kSoftThreads;
 constexpr float kHigh = 18446744073709551616.f;          // 2^64: a larger row sum runs the range again
-constexpr float kLow = 8.271806125530277e-25f;           // 2^-80: a smaller one too
 template <int kR, int kDim, bool kSplitWeights>
 struct Cfg {
   static_assert(kR == 32 || kR == 48 || kR == 64 || kR == 80, "row tile");
@@ -244,6 +247,11 @@ __device__ __forceinline__ void ldmatrix4(uint32_t addr, uint32_t (&r)[4]) {
                : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
                : "r"(addr)
                : "memory");
+}
+// The dot product of 8 bf16 pairs
+__device__ __forceinline__ float dot8(const uint4& x, const uint4& y) {
+  auto dot2 = [](uint32_t a, uint32_t b) { return fmaf(sd_bf16_hi(a), sd_bf16_hi(b), sd_bf16_lo(a) * sd_bf16_lo(b)); };
+  return (dot2(x.x, y.x) + dot2(x.y, y.y)) + (dot2(x.z, y.z) + dot2(x.w, y.w));
 }
 // Byte offset of 16-byte chunk c of row r in a 128-byte-swizzled pair of
 // 64-column halves, `half` bytes each.
@@ -635,7 +643,8 @@ __global__ void __launch_bounds__(kThreads, 1)
     };
     const bool new_kv = last_rank && st < a.R * kChunks;
     const long long kv_row = ((static_cast<long long>(b) * a.R + (st / kChunks)) * a.Hkv + kvh) * kDim + (st % kChunks) * 8;
-    uint4 qv[kQc] = {}, kv = make_uint4(0, 0, 0, 0), vv = make_uint4(0, 0, 0, 0);
+    uint4 qv[kQc] = {}, own[kQc] = {};  // the row's chunk, and its own new key's
+    uint4 kv = make_uint4(0, 0, 0, 0), vv = make_uint4(0, 0, 0, 0);
     auto load_q = [&] {
 #pragma unroll
       for (int u = 0; u < kQc; ++u) {
@@ -643,6 +652,15 @@ __global__ void __launch_bounds__(kThreads, 1)
         qv[u] = idx < kR * kChunks && p < a.M
                     ? __ldcg(reinterpret_cast<const uint4*>((kFused ? a.qw : a.q) + q_off(p) + (idx % kChunks) * 8))
                     : make_uint4(0, 0, 0, 0);
+      }
+    };
+    auto load_own = [&] {
+#pragma unroll
+      for (int u = 0; u < kQc; ++u) {
+        const int idx = st + u * kSoftThreads, p = mblock * kR + (idx / kChunks), i = gdiv(p);
+        const __nv_bfloat16* src = kFused ? a.k_new + ((static_cast<long long>(b) * a.R + i) * a.Hkv + kvh) * kDim
+                                          : a.kc + ((static_cast<long long>(b) * a.Hkv + kvh) * a.cap + L_pre + i) * kDim;
+        if (idx < kR * kChunks && p < a.M) own[u] = __ldcg(reinterpret_cast<const uint4*>(src + (idx % kChunks) * 8));
       }
     };
     auto load_kv = [&](const __nv_bfloat16* k, const __nv_bfloat16* v, long long src) {
@@ -681,6 +699,17 @@ __global__ void __launch_bounds__(kThreads, 1)
         }
         st_shared_v4(qs + swz(row, c, C::kQHalf), w[0], w[1], w[2], w[3]);
       }
+      // the rows' references; a score that is not a number or infinite: 0
+#pragma unroll
+      for (int u = 0; u < kQc; ++u) {
+        const int idx = st + u * kSoftThreads;
+        if (idx >= kR * kChunks) break;  // warp-uniform
+        float d = dot8(qv[u], own[u]);
+#pragma unroll
+        for (int o = kChunks / 2; o > 0; o >>= 1) d += __shfl_xor_sync(0xffffffffu, d, o);
+        d *= sl;
+        if (idx % kChunks == 0) row_nref[idx / kChunks] = fabsf(d) < INFINITY ? -d : 0.f;
+      }
       if (last_rank && st < C::kMaxNew * kChunks) {
         // new key (rotated) and value rows, zero past R
         const int i = st / kChunks, c = st % kChunks;
@@ -695,11 +724,9 @@ __global__ void __launch_bounds__(kThreads, 1)
         st_shared_v4(base + C::kOffNewV + off, vv.x, vv.y, vv.z, vv.w);
         if (kFused && has_kv && it == 1 && mblock == 0) {
           // the append: cache rows L_pre .. L_pre + R - 1, which no CTA of
-          // this launch reads; and, when this cluster alone reads the head's
-          // raw key rows, their rotation in place
+          // this launch reads
           *reinterpret_cast<uint4*>(a.kc + cache_row()) = make_uint4(w[0], w[1], w[2], w[3]);
           *reinterpret_cast<uint4*>(a.vc + cache_row()) = vv;
-          if (a.n_mblocks == 1) *reinterpret_cast<uint4*>(a.k_new + kv_row) = make_uint4(w[0], w[1], w[2], w[3]);
         }
       }
     };
@@ -735,6 +762,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       for (int it = it0; it < 2; ++it) {
         if (it == 1) griddep_wait();
         load_q();
+        if (kFused || valid) load_own();
         if (kFused && has_kv) load_kv(a.k_new, a.v_new, kv_row);
         if (!kFused && has_kv) load_kv(a.kc, a.vc, cache_row());
         store_rows(has_kv, it);
@@ -742,7 +770,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     } else {
       // Without the early prefix the rows are read together with the length and the
       // positions: one global round trip before the tiles, not two. The attention's
-      // new rows need the length: the last rank's threads read it themselves rather
+      // new rows need the length: the threads read it themselves rather
       // than wait for the producer's at the CTA barrier (one scene, L = 4096, K = 7:
       // 7.8 -> 7.4 us; head dim 64, L = 4099: 9.5 -> 8.9)
       valid = false;
@@ -751,32 +779,19 @@ __global__ void __launch_bounds__(kThreads, 1)
         if (it == 1) {
           griddep_wait();
           load_q();
+          if (!kFused) ranges(__ldcg(a.len + b));
+          if (kFused || valid) load_own();
           if (kFused && new_kv) load_kv(a.k_new, a.v_new, kv_row);
-          if (!kFused && new_kv) {
-            ranges(__ldcg(a.len + b));
-            if (valid) load_kv(a.kc, a.vc, cache_row());
-          }
+          if (!kFused && new_kv && valid) load_kv(a.kc, a.vc, cache_row());
         }
         if (kFused) make_table(it == 1);
         if (it == 1) cta_barrier();
         store_rows(new_kv && valid, it);
       }
     }
-    {
-      if (st < kR) row_nref[st] = 0.f;
-      asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-      named_bar_sync(3, kSoftThreads + 32);  // Q is complete; the rotation table is no longer read
-      if (st == 0) {
-        griddep_launch();  // every older kernel has finished: the next layer may launch
-        // with several m-blocks the head's raw key rows are read by the last
-        // rank of each: the last of them writes the rotated rows back (the
-        // fence orders this CTA's reads before its ticket)
-        if (kFused && has_new && a.n_mblocks > 1) {
-          __threadfence();
-          *s_kvlast = atomicAdd(&a.kv_ticket[b * a.Hkv + kvh], 1u) == static_cast<uint32_t>(a.n_mblocks - 1);
-        }
-      }
-    }
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+    named_bar_sync(3, kSoftThreads + 32);  // Q and the references are complete; the rotation table is no longer read
+    if (st == 0) griddep_launch();         // every older kernel has finished: the next layer may launch
 
     const uint64_t sl2 = pack2f(sl, sl);
     uint64_t lp2[kRpt / 2];  // this key lane's row sums, in pairs
@@ -874,7 +889,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         l0 += __shfl_xor_sync(0xffffffffu, l0, o);
         l1 += __shfl_xor_sync(0xffffffffu, l1, o);
       }
-      out_of_range |= fmaxf(l0, l1) > kHigh || fminf(l0, l1) < kLow;
+      out_of_range |= fmaxf(l0, l1) > kHigh;
       if (lane < 4) *reinterpret_cast<float2*>(row_new + r8 + 2 * lane) = make_float2(l0, l1);
     };
     while (true) {
@@ -884,18 +899,16 @@ __global__ void __launch_bounds__(kThreads, 1)
       if (C::kNewFirst && has_new && kSoftWarps - 1 - sw < kR / 8) new_keys(kSoftWarps - 1 - sw);
       // ---- this group's prefix tiles
 #pragma unroll
-      for (int j = 0; j < kRpt / 2; ++j) lp2[j] = skips && row0 >= rows_in ? pack2f(1.f, 1.f) : 0ull;
+      for (int j = 0; j < kRpt / 2; ++j) lp2[j] = 0ull;
       const int t_first = ((pass * n_pre) ^ group) & 1;
       const int T1 = pass * n_pre + t_first, V1 = T1 + 2 * kS - 2;  // PV(T - 2) as a phase of its ring, T >= 0
       int sb = T1 % 3, vb = V1 % kS;
       uint32_t spar = (T1 / 3) & 1, vpar = (V1 / kS) & 1;
       int key0 = key_begin + t_first * kStageKeys;
-      bool seen = false;  // this warp has had a prefix key
 #pragma unroll 1
       for (int t = t_first; t < n_pre; t += 2) {
         const int T = pass * n_pre + t;
         const bool key_ok = key0 + kl < key_end;
-        seen |= key0 + quarter * 32 < key_end;
         key0 += 2 * kStageKeys;
         mbar_wait(SREADY(sb), spar);
         tc_fence_after();
@@ -930,20 +943,16 @@ __global__ void __launch_bounds__(kThreads, 1)
       if (!C::kNewFirst && has_new && group == (n_pre & 1))
 #pragma unroll 1
         for (int unit = sw & 7; unit < kR / 8; unit += 8) new_keys(unit);
-      // ---- whether a row sum left the range that weights without a reference are
-      // exact in: a thread's sum too large, or a warp (with a key of its own) none of
-      // whose lanes has every row's sum large enough
+      // ---- whether a row's scores rose too far above its reference
       {
-        float lo = INFINITY, hi = 0.f;
+        float hi = 0.f;
 #pragma unroll
         for (int j = 0; j < kRpt / 2; ++j) {
           float x, y;
           unpack2(lp2[j], x, y);
-          lo = fminf(lo, fminf(x, y));
           hi = fmaxf(hi, fmaxf(x, y));
         }
-        const bool some = __any_sync(0xffffffffu, lo >= kLow);  // by every lane, whatever the others find
-        out_of_range |= hi > kHigh || (seen && !some);
+        out_of_range |= hi > kHigh;
       }
       const bool again = named_bar_or(2, kSoftThreads, out_of_range);
       if (pass == 2) break;
@@ -1097,8 +1106,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     if (kFused && valid) {
       // while the partials travel: every CTA of the cluster has read the raw
       // rows (its tiles came after), so the rotated query rows this CTA merges
-      // go back to q, and with several m-blocks the head's last reader of the
-      // raw key rows writes the rotated ones back to k_new
+      // go back to q
 #pragma unroll 1
       for (int idx = st; idx < my_rows * kChunks; idx += kSoftThreads) {
         const int row = mrow0 + (idx / kChunks), c = idx % kChunks, p = mblock * kR + row;
@@ -1106,17 +1114,11 @@ __global__ void __launch_bounds__(kThreads, 1)
         *reinterpret_cast<uint4*>(a.qw + q_off(p) + c * 8) =
             *reinterpret_cast<const uint4*>(smem + C::kOffQ + swz(row, c, C::kQHalf));
       }
-      if (last_rank && a.n_mblocks > 1 && *s_kvlast != 0) {
-        if (st < a.R * kChunks)
-          *reinterpret_cast<uint4*>(a.k_new + kv_row) =
-              *reinterpret_cast<const uint4*>(smem + C::kOffNewK + swz(st / kChunks, st % kChunks, C::kNewHalf));
-        if (st == 0) a.kv_ticket[b * a.Hkv + kvh] = 0;  // re-armed
-      }
     }
     if (merge) {
       // ---- merge of the rows this CTA owns, a warp a row, kDim / 32 d a lane; slot
-      // c * rpc + r came from rank c. Unless some rank ran its range again all
-      // references are 0 and the partials add.
+      // c * rpc + r came from rank c. Unless some rank ran its range again all have
+      // the row's one reference and the partials add.
       const float* recv = reinterpret_cast<const float*>(smem);
       const int cstep = rpc * kRowF;
       constexpr int kPer = kDim / 32;
@@ -1131,6 +1133,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         if (r == sw) mbar_wait(RECV, 0);
         Row ov = {};
         float l = 0.f;
+        const float ref0 = part[kRowM];
         // the ranks' row sums and references, one a lane: element lane & 15 of every
         // second rank (8: the reference; 0..7 and 9: sums)
         const int e = lane & 15;
@@ -1138,7 +1141,7 @@ __global__ void __launch_bounds__(kThreads, 1)
 #pragma unroll 2
         for (int c = lane >> 4; c < csize; c += 2) {
           const float x = part[c * cstep + kRowL + (e < 10 ? e : 0)];
-          moved |= e == 8 && x != 0.f;
+          moved |= e == 8 && x != ref0;
           l += e < 10 && e != 8 ? x : 0.f;
         }
 #pragma unroll 4
@@ -1183,6 +1186,26 @@ __global__ void __launch_bounds__(kThreads, 1)
       }
       if (elect_one()) asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
       __syncwarp();
+    }
+    if (kFused && valid && last_rank) {
+      // every CTA of the cluster has read the raw key rows: the rotated ones go back to
+      // k_new, by the warps that merge least. With several m-blocks each one's cluster
+      // reads them: the last to come here writes (the fence orders the reads before its
+      // ticket)
+      bool write = true;
+      if (a.n_mblocks > 1) {
+        if (st == 0) {
+          __threadfence();
+          *s_kvlast = atomicAdd(&a.kv_ticket[b * a.Hkv + kvh], 1u) == static_cast<uint32_t>(a.n_mblocks - 1);
+          if (*s_kvlast) a.kv_ticket[b * a.Hkv + kvh] = 0;  // re-armed
+        }
+        named_bar_sync(2, kSoftThreads);
+        write = *s_kvlast != 0;
+      }
+      const int idx = kSoftThreads - 1 - st, i = idx / kChunks, c = idx % kChunks;
+      if (write && i < a.R)
+        *reinterpret_cast<uint4*>(a.k_new + ((static_cast<long long>(b) * a.R + i) * a.Hkv + kvh) * kDim + c * 8) =
+            *reinterpret_cast<const uint4*>(smem + C::kOffNewK + swz(i, c, C::kNewHalf));
     }
   }
   // no CTA-wide barrier at the end: every warp leaves when its own work is done

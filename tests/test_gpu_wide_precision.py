@@ -1,6 +1,7 @@
-"""Error of the row-tile attention against 64 bits where few keys hold the mass.
+"""Error of the row-tile attention against 64 bits where few keys hold the mass, and
+where scores and values are far from 1.
 
-Every bound is the rounding of an exact output to bf16 on the same inputs, with 1% for
+Every bound on few keys is the rounding of an exact output to bf16 on the same inputs, with 1% for
 the weights (2^-17 each, beside the output's 2^-9) and the fp32 scores."""
 import numpy as np
 import pytest
@@ -8,7 +9,7 @@ import torch
 
 import oracle
 from paper_2606_31160_gb300 import sd, workloads
-from tests.helpers import ensure_lib, to64
+from tests.helpers import attn_within, ensure_lib, to64
 
 pytestmark = pytest.mark.gpu
 # packed rows 1, 32 | 48 | 64 | 68, 80 | 96 (two m-blocks)
@@ -82,3 +83,22 @@ def test_many_rows_of_one_head(R, fused, csize, prefix):
         sd.set_cluster_size(0)
     ref = oracle.verify_attention(*rest)
     assert _rel(out, ref) <= 1.01 * _rel(_bf(ref.astype(np.float32)), ref)
+
+
+# (log2 of every score, log2 of the values): with weights that are not relative to one of
+# the row's own scores their products leave the range of fp32
+@pytest.mark.parametrize("level,scale", [(-60.0, -90), (-75.0, -60), (50.0, 90), (55.0, 75), (-20.0, -110), (0.0, -100), (0.0, 100)])
+@pytest.mark.parametrize("G,R", [(4, 1), (4, 8), (4, 12), (4, 17)])
+@pytest.mark.parametrize("fused,cluster,D", [(True, 0, 128), (True, 1, 128), (False, 0, 128), (False, 4, 64)])
+def test_values_far_from_one(level, scale, G, R, fused, cluster, D):
+    prefix = [0, 5, 700, 1500]
+    q, k, v, k_new, v_new = _inputs(int(1000 + level + scale) + G * R, len(prefix), G, R, 1, 1540, D, 2.0 ** scale)
+    beta = level / (8.0 * 1.4426950408889634 / np.sqrt(D))
+    q[..., 5], k[..., 5], k_new[..., 5] = 8.0, beta, beta
+    sd.set_cluster_size(cluster)
+    try:
+        out, qd, kd, vd, lens = _call(q, k, v, k_new, v_new, prefix, fused)
+    finally:
+        sd.set_cluster_size(0)
+    ref = oracle.verify_attention(qd, kd, vd * 2.0 ** -scale, lens)
+    assert attn_within(out * 2.0 ** -scale, ref), np.abs(out * 2.0 ** -scale - ref).max()

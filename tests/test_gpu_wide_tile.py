@@ -1,8 +1,9 @@
 """The row tiles (32, 48, 64 and 80 packed query rows per KV head, two m-blocks
 above 80) against the float64 oracle: every edge of the tile choice, prefixes
 around the 32-key split and the 128-key tile, causal and block masks, the fused
-layer and the attention; and the second pass of a CTA whose row sums leave the
-range of weights taken without a reference (2^-80 .. 2^64)."""
+layer and the attention; and scores far from 0 and from each other: a row's reference
+is its score against new key 0, and a CTA with a row sum above 2^64 runs its range a
+second time."""
 import numpy as np
 import pytest
 import torch
