@@ -223,12 +223,20 @@ sd_status sd_set_cluster_size(int cluster_size);
 /*
  * Which kernel serves a shape on the CURRENT device: "tcgen05" or
  * "mma.sync" for sd_verify_attention (layer = 0), and for
- * sd_verify_layer (layer = 1, or 2 with SD_LAYER_BLOCK_MASK; "three kernels"
- * when the layer runs as the rotation, append and attention kernels in
- * sequence); "unsupported" for a shape neither call takes. Host-only, no
+ * sd_verify_layer (layer nonzero: 1, or 2 with SD_LAYER_BLOCK_MASK, whose
+ * kernel is the same; "three kernels" when the layer runs as the rotation,
+ * append and attention kernels in sequence); "unsupported" for a shape neither call takes. Host-only, no
  * device work; a static string.
  */
 const char* sd_verify_kernel(int B, int R, int Hq, int Hkv, int D, int capacity, int layer);
+
+/*
+ * CTAs a thread-block cluster that the next sd_verify_attention (layer = 0) or
+ * sd_verify_layer (layer = 1) call of this shape takes on the CURRENT device,
+ * the forced size of sd_set_cluster_size included; 0 when no tcgen05 kernel
+ * serves it (sd_verify_kernel). Host-only, no device work.
+ */
+int sd_verify_cluster_size(int B, int R, int Hq, int Hkv, int D, int capacity, int layer);
 
 /*
  * Attention budget of the verify rows (Sec. 4.2 "Empirical confirmation",

@@ -791,16 +791,22 @@ DevState* state() {
 // count a quarter more. Sizes above 8 cost more a wave (their set-up and exchange),
 // and one that leaves no room for the next layer's clusters loses the overlap of its
 // stream when layers are chained (the choice is the same with and without the early
-// prefix, so that both give the same bits); both weigh less on the wider row tiles,
-// whose 128 keys take longer. The weights are fitted to 60 measured shapes (1 to 256
-// (scene, head) pairs, L = 512 to 16384): the choice is within 2% of the best size on
-// 51 of them and 15% on the rest. Measured, one scene, 8 KV heads, us a launch at sizes
-// 8 / 10 / 12 (sizes 7, 9, 11 lie between or above; 13 and more do not fit in one wave):
+// prefix, so that both give the same bits). On the wider row tiles, whose 128 keys take
+// longer, these weigh less, but for size 10's charge: it is what the measurements below
+// give on 32 and on 80 rows alike, and leaves 10 the shapes between 8 and 12 (8 heads:
+// 5 of the next layer's clusters still fit) and those of 9 to 12 heads.
+// The weights are fitted to 70 measured shapes (1 to 256 (scene, head) pairs, L = 512 to
+// 16384): the choice is within 2.5% of the best size on 62 of them. The others (pairs, L:
+// chosen / best, us): 80 rows 8, 4096: 8 / 12, 10.97 / 10.53; 32 rows 4, 4096: 12 / 16,
+// 7.0 / 6.4; 12, 2048: 6 / 8, 7.3 / 6.8; 24, 512: 2 / 4, 6.1 / 5.6; 32, 512: 2 / 4,
+// 6.3 / 5.9; 16, 2048: 5 / 4, 6.2 / 5.75; 24, 2048: 5 / 4, 7.6 / 7.2; 64, 512: 2 / 1,
+// 6.8 / 6.4. Measured, one scene, 8 KV heads, us a launch at
+// sizes 8 / 10 / 12 (7, 9, 11 lie between or above; 13 and more do not fit in one wave):
 //   chained, 32 rows: L = 4096 6.3 / 6.6 / 7.8, 8192 9.4 / 8.9 / 9.8, 16384 14.8 / 14.6 / 13.7
 //   chained, 80 rows: L = 4096 10.7 / 11.1 / 11.5, 8192 14.6 / 14.2 / 14.2, 16384 20.9 / 19.9 / 18.6
 // 4 KV heads at 8 / 10 / 12 / 16: draft step L = 4096 6.9 / 6.6 / 6.1 / 6.2, chained 5.5 /
 // 5.6 / 5.2 / 5.6. 20 pairs, L = 4099, 48 rows, at 5 / 6 / 8: 11.2 / 11.0 / 16.9. 24 pairs,
-// L = 8192, 32 rows, at 4 / 5: 18.0 / 17.7.
+// L = 8192, 32 rows, at 4 / 5: 18.0 / 17.7. (All measured before the rows had references.)
 int pick_cluster(const int* active, long long units, int cap, int rows) {
   const double nblk = (cap + 31) / 32, wide = rows <= 32 ? 1.0 : (rows <= 48 ? 0.8 : 0.5);
   double best_cost = -1;
@@ -898,6 +904,12 @@ bool sd_internal_tc_serves(int B, int R, int Hq, int Hkv, int D, int cap) {
 
 bool sd_internal_tc_serves_layer(int B, int R, int Hq, int Hkv, int D, int cap) {
   return D == kD && tc_plan(B, R, Hq, Hkv, D, cap, false, true).cs > 0;
+}
+
+int sd_internal_tc_cluster(int B, int R, int Hq, int Hkv, int D, int cap, bool layer) {
+  if (layer) return D == kD ? tc_plan(B, R, Hq, Hkv, D, cap, false, true).cs : 0;
+  const TcPlan p = tc_plan(B, R, Hq, Hkv, D, cap, false);
+  return p.cs > 0 ? p.cs : tc_plan(B, R, Hq, Hkv, D, cap, true).cs;
 }
 
 template <int kR>

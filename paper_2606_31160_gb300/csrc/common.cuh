@@ -47,6 +47,8 @@ sd_status sd_internal_verify_attention_tc(const void* q, const sd_kv_cache* cach
 // attention, and the fused layer.
 bool sd_internal_tc_serves(int B, int R, int Hq, int Hkv, int D, int cap);
 bool sd_internal_tc_serves_layer(int B, int R, int Hq, int Hkv, int D, int cap);
+// Their cluster sizes, 0 where not served.
+int sd_internal_tc_cluster(int B, int R, int Hq, int Hkv, int D, int cap, bool layer);
 
 struct RopeTable;
 // The fused verify layer on the tcgen05 path (attention_tc.cu); *handled is

@@ -80,10 +80,18 @@ extern "C" sd_status sd_verify_layer(void* q, void* k_new, const void* v_new, co
                                 ws_bytes - kTicketBytes(B, Hkv), stream);
 }
 
+// (sd_verify_attention's limits)
+static bool shape_ok(int B, int R, int Hq, int Hkv, int D, int capacity) {
+  return B > 0 && R > 0 && Hq > 0 && Hkv > 0 && capacity > 0 && Hq % Hkv == 0 && (D == 64 || D == 128) &&
+         static_cast<long long>(Hq / Hkv) * R <= 128;
+}
+
 extern "C" const char* sd_verify_kernel(int B, int R, int Hq, int Hkv, int D, int capacity, int layer) {
-  if (B <= 0 || R <= 0 || Hq <= 0 || Hkv <= 0 || capacity <= 0 || Hq % Hkv || (D != 64 && D != 128) ||
-      static_cast<long long>(Hq / Hkv) * R > 128)
-    return "unsupported";
+  if (!shape_ok(B, R, Hq, Hkv, D, capacity)) return "unsupported";
   if (layer) return sd_internal_tc_serves_layer(B, R, Hq, Hkv, D, capacity) ? "tcgen05" : "three kernels";
   return sd_internal_tc_serves(B, R, Hq, Hkv, D, capacity) ? "tcgen05" : "mma.sync";
+}
+
+extern "C" int sd_verify_cluster_size(int B, int R, int Hq, int Hkv, int D, int capacity, int layer) {
+  return shape_ok(B, R, Hq, Hkv, D, capacity) ? sd_internal_tc_cluster(B, R, Hq, Hkv, D, capacity, layer != 0) : 0;
 }

@@ -63,6 +63,7 @@ _SIGNATURES = {
     "sd_get_device_error": ([_vp, ctypes.POINTER(ctypes.c_uint32)], _i),
     "sd_set_cluster_size": ([_i], _i),
     "sd_verify_kernel": ([_i, _i, _i, _i, _i, _i, _i], ctypes.c_char_p),
+    "sd_verify_cluster_size": ([_i, _i, _i, _i, _i, _i, _i], _i),
     "sd_attention_budget": ([_vp, ctypes.POINTER(KVCacheStruct), _i, _i, _f, _vp, _vp, _vp, _vp], _i),
 }
 
@@ -389,6 +390,11 @@ def verify_kernel(B, R, Hq, Hkv, D, capacity, layer=False):
     """Name of the kernel that serves this shape on the current device
     (sd_verify_kernel): "tcgen05", "mma.sync" or "three kernels"."""
     return lib().sd_verify_kernel(B, R, Hq, Hkv, D, capacity, 1 if layer else 0).decode()
+
+
+def verify_cluster_size(B, R, Hq, Hkv, D, capacity, layer=False):
+    """CTAs a cluster that this shape's next call takes (sd_verify_cluster_size); 0 off the tcgen05 path."""
+    return lib().sd_verify_cluster_size(B, R, Hq, Hkv, D, capacity, 1 if layer else 0)
 
 
 def get_device_error():

@@ -88,8 +88,8 @@ def test_row_sums_out_of_range(G, R, level, part, cluster, D):
         sd.set_cluster_size(0)
 
 
-# (scenes, KV heads, capacity) whose clusters are of 5, 12, 12, 16 and 10 CTAs: a scene that
-# leaves most of them without a key, and one whose last 32-key split is partial
+# prefixes that leave most CTAs of a cluster without a key, or end in a partial 32-key
+# split, on capacities that get large clusters (which ones: test_sizes_that_only_the_rule_chooses)
 @pytest.mark.parametrize("prefix,Hkv,cap", [([0, 37, 4099], 8, 4112), ([70, 4099], 2, 4112), ([4088], 4, 4112), ([16390], 4, 16400), ([8189], 8, 8206)])
 @pytest.mark.parametrize("G,R", [(4, 1), (4, 8), (8, 8), (5, 12)])
 @pytest.mark.parametrize("fused,D", [(True, 128), (False, 64)])
@@ -100,3 +100,34 @@ def test_cluster_sizes(prefix, Hkv, cap, G, R, fused, D):
     prefix = [min(n, cap - R) for n in prefix]
     _run(draw(B, R, Hkv * G, D), draw(B, Hkv, cap, D), draw(B, Hkv, cap, D), draw(B, R, Hkv, D), draw(B, R, Hkv, D),
          prefix, fused, False)
+
+
+# The sizes that sd_set_cluster_size does not force, and 16, on every row tile that the
+# rule gives them on 152 SMs: 32, 48, 64, 80 rows, 48 with two-term weights, two m-blocks
+@pytest.mark.parametrize("cs,Hkv,cap,G,R", [(cs, Hkv, cap, G, R) for cs, Hkv, cap in ((5, 14, 600), (10, 9, 8200), (12, 8, 12300), (16, 1, 4112))
+                                            for G, R in ((4, 8), (4, 12), (4, 16), (5, 16), (1, 20))]
+                         + [(5, 12, 2100, 6, 16), (12, 4, 8200, 6, 16), (16, 1, 4112, 6, 16)])
+@pytest.mark.parametrize("fused,D", [(True, 128), (False, 128), (False, 64)])
+def test_sizes_that_only_the_rule_chooses(cs, Hkv, cap, G, R, fused, D):
+    if torch.cuda.get_device_properties(0).multi_processor_count != 152:
+        pytest.skip("the rule's choice is that of 152 SMs")
+    assert sd.verify_cluster_size(1, R, G * Hkv, Hkv, D, cap, fused) == cs
+    rng = np.random.default_rng(cap + 10 * G + R)
+    draw = lambda *s: rng.standard_normal(s, dtype=np.float32)  # noqa: E731
+    prefix = [min(701, cap - R)]
+    _run(draw(1, R, Hkv * G, D), draw(1, Hkv, cap, D), draw(1, Hkv, cap, D), draw(1, R, Hkv, D), draw(1, R, Hkv, D),
+         prefix, fused, False)
+
+
+def test_forced_size_is_the_size():
+    for cs in (1, 2, 4, 6, 8, 16):
+        sd.set_cluster_size(cs)
+        try:
+            assert sd.verify_cluster_size(1, 8, 32, 8, 128, 4112) == cs
+            assert sd.verify_cluster_size(1, 17, 32, 8, 128, 4112, True) == cs
+            assert sd.verify_cluster_size(1, 8, 32, 8, 64, 4112) == cs
+            assert sd.verify_cluster_size(1, 40, 8, 8, 128, 4112) == cs     # every key in the loop
+        finally:
+            sd.set_cluster_size(0)
+    assert sd.verify_cluster_size(1, 40, 8, 8, 64, 4112) == 0               # mma.sync
+    assert sd.verify_cluster_size(1, 8, 32, 8, 64, 4112, True) == 0         # three kernels
