@@ -105,10 +105,17 @@ def _check(status, what):
         raise SDError(what, status)
 
 
+# private to torch: looked up once, and done without where a torch has them not
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+_raw_device = getattr(torch._C, "_cuda_getDevice", None)
+
+
 def _stream():
-    """Handle of torch's current stream on the current device (without the Stream
-    object that torch.cuda.current_stream() builds, ~1 us a call)."""
-    return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
+    """Handle of torch's current stream on the current device (where torch offers it
+    without the Stream object that torch.cuda.current_stream() builds, ~1 us a call)."""
+    if _raw_stream is None or _raw_device is None:
+        return torch.cuda.current_stream().cuda_stream
+    return _raw_stream(_raw_device())
 
 
 def _dev(t, name, dtype=None, ndim=None):
