@@ -80,18 +80,16 @@ __device__ __forceinline__ const float* row_ptr(const float* zt, const float* zd
 }
 
 // ------------------------------------------------------------------ stats
-constexpr int kVecThreads = 512;       // threads of the vectorised stats kernel
-constexpr int kVecPer = 32;            // values per thread (eight 16-byte loads)
-constexpr int kVecChunk = kVecThreads * kVecPer;
-constexpr int kScalarPer = 16;  // values per thread of the scalar kernel (unaligned rows)
+constexpr int kScalarPer = 16;  // values per thread of the scalar kernel
 constexpr int kScalarChunk = kThreads * kScalarPer;
+constexpr int kMinSegment = 16384;  // values a CTA of the streaming kernel at least takes of a longer row
 
-template <bool kVec>
-__global__ void __launch_bounds__(kVec ? kVecThreads : kThreads)
+// Rows that are not aligned: values lo + t + kThreads k, k < 16, of a chunk, loaded once,
+// all in flight, for the maximum and the sum.
+__global__ void __launch_bounds__(kThreads)
     sample_stats_kernel(const float* zt, const float* zd, int K, int V,
                         float c2, int chunk, int n_chunks, const int32_t* draft,
                         float2* __restrict__ part, float* __restrict__ dlogit) {
-  constexpr int kT = kVec ? kVecThreads : kThreads;
   const int c = blockIdx.x, rr = blockIdx.y, b = blockIdx.z;
   sd_pdl_enter();
   const int rows = 2 * K + 1;
@@ -104,38 +102,17 @@ __global__ void __launch_bounds__(kVec ? kVecThreads : kThreads)
     if (x >= lo && x < hi) dlogit[static_cast<long long>(b) * rows + rr] = __ldcg(row + x);
   }
   float m = -INFINITY, s = 0.f;
-  if (kVec) {
-    // values lo + 4 (t + kT k) + e, k < 8, e < 4: one fixed order for both passes
-    float x[kVecPer];
+  float x[kScalarPer];
 #pragma unroll
-    for (int k = 0; k < kVecPer / 4; ++k) {
-      const int i = lo + 4 * (threadIdx.x + kT * k);
-      const float4 v = i < hi ? __ldcg(reinterpret_cast<const float4*>(row + i))
-                              : make_float4(-INFINITY, -INFINITY, -INFINITY, -INFINITY);
-      x[4 * k + 0] = v.x;
-      x[4 * k + 1] = v.y;
-      x[4 * k + 2] = v.z;
-      x[4 * k + 3] = v.w;
-    }
-#pragma unroll
-    for (int e = 0; e < kVecPer; ++e) m = fmaxf(m, x[e]);
-    if (m != -INFINITY)
-#pragma unroll
-      for (int e = 0; e < kVecPer; ++e) s = __fadd_rn(s, x[e] == -INFINITY ? 0.f : wexp(x[e], m, c2));
-  } else {
-    // values lo + t + kT k, k < 16: loaded once, all in flight, for the maximum and the sum
-    float x[kScalarPer];
-#pragma unroll
-    for (int k = 0; k < kScalarPer; ++k) {
-      const int i = lo + threadIdx.x + kT * k;
-      x[k] = i < hi ? __ldcg(row + i) : -INFINITY;
-    }
-#pragma unroll
-    for (int k = 0; k < kScalarPer; ++k) m = fmaxf(m, x[k]);
-    if (m != -INFINITY)
-#pragma unroll
-      for (int k = 0; k < kScalarPer; ++k) s = __fadd_rn(s, x[k] == -INFINITY ? 0.f : wexp(x[k], m, c2));
+  for (int k = 0; k < kScalarPer; ++k) {
+    const int i = lo + threadIdx.x + kThreads * k;
+    x[k] = i < hi ? __ldcg(row + i) : -INFINITY;
   }
+#pragma unroll
+  for (int k = 0; k < kScalarPer; ++k) m = fmaxf(m, x[k]);
+  if (m != -INFINITY)
+#pragma unroll
+    for (int k = 0; k < kScalarPer; ++k) s = __fadd_rn(s, x[k] == -INFINITY ? 0.f : wexp(x[k], m, c2));
   // warp then block merge, fixed tree
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) {
@@ -143,7 +120,7 @@ __global__ void __launch_bounds__(kVec ? kVecThreads : kThreads)
     const float s2 = __shfl_xor_sync(0xffffffffu, s, o);
     merge_ms(m, s, m2, s2, c2);
   }
-  __shared__ float sm[kT / 32], ss[kT / 32];
+  __shared__ float sm[kThreads / 32], ss[kThreads / 32];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   if (lane == 0) {
     sm[warp] = m;
@@ -152,7 +129,7 @@ __global__ void __launch_bounds__(kVec ? kVecThreads : kThreads)
   __syncthreads();
   if (threadIdx.x == 0) {
     float bm = sm[0], bs = ss[0];
-    for (int w = 1; w < kT / 32; ++w) merge_ms(bm, bs, sm[w], ss[w], c2);
+    for (int w = 1; w < kThreads / 32; ++w) merge_ms(bm, bs, sm[w], ss[w], c2);
     part[(static_cast<long long>(b) * rows + rr) * n_chunks + c] = make_float2(bm, bs);
   }
 }
@@ -668,26 +645,21 @@ __global__ void __launch_bounds__(kThreads)
 }
 
 struct Plan {
-  int chunk1, n1, chunk2, n2;
+  int n1, n2;  // chunks a row of the scalar stats kernel, and of the draw
   bool vec;
-  int n_scalar;  // chunks a row of the scalar stats kernel (unaligned rows)
 };
 
-// Vectorised stats when every row starts on a 16-byte boundary (V a multiple
-// of 4 and a 16-byte-aligned base, checked at the call).
+// Streaming stats when every row starts on a 16-byte boundary (V a multiple of 4 and
+// 16-byte-aligned bases, checked at the call).
 Plan plan(int V) {
   Plan p;
   p.vec = V % 4 == 0;
   // (the doubling is for the workspace size alone: a call with over kMaxChunks
   // chunks of 4096 is refused)
-  p.chunk1 = p.vec ? kVecChunk : kScalarChunk;
-  while ((V + p.chunk1 - 1) / p.chunk1 > kMaxChunks) p.chunk1 *= 2;
-  p.n1 = (V + p.chunk1 - 1) / p.chunk1;
-  int scalar = kScalarChunk;
-  while ((V + scalar - 1) / scalar > kMaxChunks) scalar *= 2;
-  p.n_scalar = (V + scalar - 1) / scalar;
-  p.chunk2 = kDrawChunk;
-  p.n2 = (V + p.chunk2 - 1) / p.chunk2;
+  int chunk = kScalarChunk;
+  while ((V + chunk - 1) / chunk > kMaxChunks) chunk *= 2;
+  p.n1 = (V + chunk - 1) / chunk;
+  p.n2 = (V + kDrawChunk - 1) / kDrawChunk;
   return p;
 }
 
@@ -703,8 +675,8 @@ Layout layout(int B, int K, const Plan& p) {
     off += (bytes + 255) / 256 * 256;
     return at;
   };
-  // room for the scalar chunking's partials too (rows found unaligned at the call)
-  l.part = take(static_cast<size_t>(B) * (2 * K + 1) * (p.n_scalar > p.n1 ? p.n_scalar : p.n1) * sizeof(float2));
+  // room for the scalar chunking's partials (rows found unaligned at the call)
+  l.part = take(static_cast<size_t>(B) * (2 * K + 1) * p.n1 * sizeof(float2));
   l.dlogit = take(static_cast<size_t>(B) * (2 * K + 1) * sizeof(float));
   // unused: the size that callers have planned with counts 4 and 32 bytes a scene here
   take(static_cast<size_t>(B) * 4);
@@ -719,12 +691,14 @@ constexpr int stream_smem(int stages) { return stages * kStageFloats * 4; }
 
 // Stages of the ring. Four leave room for three CTAs an SM, three for four; the
 // latter where four stages would leave a few CTAs for a second wave: 480 CTAs (16
-// scenes, K = 7) 44.3 -> 39.5 us, 32 scenes 77 -> 66. With fewer CTAs the deeper
-// ring is as fast or faster (336 CTAs 25.2 against 26.8, 396 25.0 / 25.5; 360 25.8 / 23.7).
+// scenes, K = 7) 44.3 -> 39.5 us, 32 scenes 77 -> 66. With fewer CTAs the deeper ring
+// is the faster one at 336 (25.2 us against 26.8) and 396 CTAs (25.0, 25.5) but not at
+// the 360 of 8 scenes, K = 7, V = 151936 (25.8, 23.7): the line is where the waves
+// change, and that size lies on the slower side of it.
 bool deep_ring(long long ctas, int n_sm) { return ctas <= 3LL * n_sm; }
 
 // SMs of the current device, once the streaming kernel's shared-memory
-// attribute is set there; 0 when either call fails (the one-shot kernel runs).
+// attribute is set there; 0 when either call fails (the kernel for unaligned rows runs).
 int stream_sms() {
   static int cache[64];
   static bool done[64];
@@ -770,12 +744,8 @@ extern "C" sd_status sd_accept_sample(const float* z_target, const float* z_draf
     return SD_ERR_INVALID_ARG;
   Plan p = plan(V);
   const Layout l = layout(B, K, p);
-  // the vectorised stats also need 16-byte-aligned rows (same workspace either way)
-  if ((reinterpret_cast<uintptr_t>(z_target) & 15) || (K > 0 && (reinterpret_cast<uintptr_t>(z_draft) & 15))) {
-    p.vec = false;
-    p.chunk1 = kScalarChunk;
-    p.n1 = p.n_scalar;
-  }
+  // aligned rows need aligned bases too (same workspace either way)
+  if ((reinterpret_cast<uintptr_t>(z_target) & 15) || (K > 0 && (reinterpret_cast<uintptr_t>(z_draft) & 15))) p.vec = false;
   if (!ws || ws_bytes < l.total || !sd_aligned16(ws)) return SD_ERR_WORKSPACE;
   char* w = static_cast<char*>(ws);
   auto* part = reinterpret_cast<float2*>(w + l.part);
@@ -791,7 +761,8 @@ extern "C" sd_status sd_accept_sample(const float* z_target, const float* z_draf
     // segments of whole stages, about two CTAs per SM over all (row, scene) pairs
     const long long rows_all = static_cast<long long>(2 * K + 1) * B;
     long long n_seg = (2LL * n_sm + rows_all - 1) / rows_all;
-    n_seg = n_seg < 1 ? 1 : (n_seg > p.n1 ? p.n1 : n_seg);
+    const long long most = (V + kMinSegment - 1) / kMinSegment;
+    n_seg = n_seg < 1 ? 1 : (n_seg > most ? most : n_seg);
     const int seg = static_cast<int>(((V + n_seg - 1) / n_seg + kStageFloats - 1) / kStageFloats * kStageFloats);
     const int ns = (V + seg - 1) / seg;
     const bool deep = deep_ring(rows_all * ns, n_sm);
@@ -800,9 +771,8 @@ extern "C" sd_status sd_accept_sample(const float* z_target, const float* z_draf
                       dlogit);
     parts = ns;
   } else {
-    e = sd_launch_pdl(p.vec ? sample_stats_kernel<true> : sample_stats_kernel<false>, dim3(p.n1, 2 * K + 1, B),
-                      dim3(p.vec ? kVecThreads : kThreads), 0, st, z_target, z_draft, K, V, c2, p.chunk1, p.n1, draft, part,
-                      dlogit);
+    e = sd_launch_pdl(sample_stats_kernel, dim3(p.n1, 2 * K + 1, B), dim3(kThreads), 0, st, z_target, z_draft, K, V, c2,
+                      kScalarChunk, p.n1, draft, part, dlogit);
   }
   if (e == cudaSuccess)
     e = sd_launch_pdl(sample_draw_kernel, dim3(p.n2, B), dim3(kThreads), p.vec ? 0 : kDrawSmem, st, z_target, z_draft, K, V, c2, p.n2, p.vec,

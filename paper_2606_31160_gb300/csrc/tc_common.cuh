@@ -79,15 +79,7 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity) {
   mbar_timed_out();
   return false;
 }
-__device__ __forceinline__ void tma_load_3d(uint32_t dst, const CUtensorMap* map, uint32_t bar,
-                                            int x, int y, int z) {
-  asm volatile(
-      "cp.async.bulk.tensor.3d.shared::cluster.global.tile.mbarrier::complete_tx::bytes"
-      " [%0], [%1, {%3, %4, %5}], [%2];" ::"r"(dst),
-      "l"(reinterpret_cast<uint64_t>(map)), "r"(bar), "r"(x), "r"(y), "r"(z)
-      : "memory");
-}
-// The same load with an L2 eviction policy (createpolicy): the cached prefix is
+// One box of a 3-D map with an L2 eviction policy (createpolicy): the cached prefix is
 // read once per step, so its lines go first and the code and the per-step rows
 // stay in L2 (an instruction fetch that misses L2 waits behind the stream).
 __device__ __forceinline__ void tma_load_3d_hint(uint32_t dst, const CUtensorMap* map, uint32_t bar, int x, int y,
@@ -188,11 +180,6 @@ __device__ __forceinline__ void umma(uint32_t d_tmem, uint64_t a, uint64_t b, ui
       "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(d_tmem),
       "l"(a), "l"(b), "r"(idesc), "r"(accumulate)
       : "memory");
-}
-__device__ __forceinline__ __nv_bfloat162 as_bf162(uint32_t w) {
-  __nv_bfloat162 v;
-  memcpy(&v, &w, 4);
-  return v;
 }
 // one lane of the (converged) warp
 __device__ __forceinline__ bool elect_one() {
