@@ -82,10 +82,17 @@ def measured_peaks():
         return 6800.0, "fallback"
 
 
+# what decides the dominant kernel's DRAM traffic: its source, the copies, tensor maps
+# and cache policies it is built from, and the tile and cluster choice
+KERNEL_SOURCES = ("attention_wide.cu", "tc_common.cuh", "common.cuh", "attention_tc.cu")
+
+
 def kernel_source_hash():
-    path = os.path.join(ROOT, "paper_2606_31160_gb300", "csrc", "attention_wide.cu")
-    with open(path, "rb") as f:
-        return hashlib.sha256(f.read()).hexdigest()
+    h = hashlib.sha256()
+    for name in KERNEL_SOURCES:
+        with open(os.path.join(ROOT, "paper_2606_31160_gb300", "csrc", name), "rb") as f:
+            h.update(hashlib.sha256(f.read()).digest())
+    return h.hexdigest()
 
 
 def ncu_traffic(kernel="verify_layer"):
