@@ -1,6 +1,7 @@
 // The verify attention and the fused verify layer (Eq. verify, Sec. 3.2; the
-// rotations of Sec. 3.3 / 4.2, the append of Eq. commit) for up to 31 new rows, head
-// dim 128 and (the attention) 64, on the 5th-generation tensor cores (tcgen05 + TMEM).
+// rotations of Sec. 3.3 / 4.2, the append of Eq. commit) for up to 31 new rows (the
+// attention of one query head a KV head: 32), head dim 128 and (the attention) 64, on
+// the 5th-generation tensor cores (tcgen05 + TMEM).
 //
 // The packed query rows of a KV head (G * R) are few, so both products run
 // transposed, the 128-wide dimension on the MMA's M side:
@@ -15,7 +16,7 @@
 // 153 -> 142 us, K = 8 165 -> 143, 1.0 of the measured copy). With one scene the
 // dependent path behind the previous kernel: rows, rotation, S(0), the tiles at
 // ~0.4 us of products each, the exchange (~0.7 us), the merge (target layer
-// 6.77 -> 6.45 us, K = 8 10.0 -> 7.4, K = 16 block 15.9 -> 10.7, draft step 6.8 -> 6.0
+// 6.77 -> 6.35 us, K = 8 10.0 -> 7.5, K = 16 block 15.9 -> 10.65, draft step 6.8 -> 6.05
 // on one cache).
 //
 // Head dim 64 (the attention; its layers run as the rotation, append and attention
@@ -39,8 +40,7 @@
 // through its range again with each row's exact maximum as its reference, one pass for
 // the maxima and one for the weights. Without a reference scores 40 away from 0 took
 // those passes (8 scenes, L = 8192, K = 7: 38 -> 102 us), and values far from 1 left
-// fp32's range in the product; the references cost a chained layer 0.2 us, the others
-// nothing.
+// fp32's range in the product; the references cost 0.1 to 0.2 us a layer.
 //
 // Warps (608 threads): 0 the TMA producer, whose first tiles go out before the CTA's
 // set-up is over; 1 issues S and owns tensor memory; 2 issues PV; 3..18 two softmax
@@ -692,8 +692,8 @@ __global__ void __launch_bounds__(kThreads, 1)
         const int idx = st + u * kSoftThreads, row = idx / kChunks, c = idx % kChunks, p = mblock * kR + row;
         if (idx >= kR * kChunks) break;
         uint32_t w[4] = {qv[u].x, qv[u].y, qv[u].z, qv[u].w};
-        if (kFused && p < a.M) {
-          const float2* cs = cs_tab + gdiv(p) * 64 + c * 4;
+        if (kFused) {  // (rows past M, zero, turn by the last row's angles: a branch cost 0.1 us a layer)
+          const float2* cs = cs_tab + gdiv(min(p, a.M - 1)) * 64 + c * 4;
 #pragma unroll
           for (int j = 0; j < 4; ++j) w[j] = sd_rope_pair(w[j], cs[j].x, cs[j].y);
         }
