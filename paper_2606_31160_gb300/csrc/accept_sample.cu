@@ -26,8 +26,8 @@
 // The logits stream once; beside that it is latency. Acceptance in every CTA of
 // the draw, rather than by the last CTA of the statistics, takes a fence, an
 // atomic and two round trips off the path; with the launches overlapped, 8 scenes,
-// K = 7, V = 151936: 28.7 -> 25.2 us, one scene 15.7 -> 12.0. Rows that are not
-// aligned, 8 scenes, V = 50257: 29.6 -> 19.8 with the statistics'
+// K = 7, V = 151936: 28.7 -> 25.5 us, one scene 15.7 -> 12.2. Rows that are not
+// aligned, 8 scenes, V = 50257: 29.6 -> 20.3 with the statistics'
 // values in registers and the draw's rows read in order through shared memory.
 // All reductions run in a fixed order (deterministic), the weight formula
 // uses non-contractible intrinsics so both passes of the draw evaluate
@@ -412,7 +412,8 @@ constexpr int kDrawStage = kDrawChunk + kDrawChunk / kDrawPer;
 constexpr int kDrawSmem = 2 * kDrawStage * 4;
 
 // This thread's kDrawPer logits of both rows (missing values: -inf, weight 0) of
-// the chunk that begins at c0. Aligned rows: 16-byte loads. Others: a warp would
+// the chunk that begins at c0. Aligned rows: 16-byte loads, through L1 (a load of a warp
+// takes half of 32 sectors; past L1 each came twice: 16 scenes 39.3 -> 44.5 us). Others: a warp would
 // touch 32 lines a load, so the block reads the chunk in order through `stage`.
 __device__ __forceinline__ void draw_load(const float* rt, const float* rd, int c0, int V, bool vec, float* stage,
                                           float (&xt)[kDrawPer], float (&xd)[kDrawPer]) {
@@ -420,9 +421,9 @@ __device__ __forceinline__ void draw_load(const float* rt, const float* rd, int 
   if (vec && v0 + kDrawPer <= V) {
 #pragma unroll
     for (int q = 0; q < kDrawPer / 4; ++q) {
-      const float4 a = __ldcg(reinterpret_cast<const float4*>(rt + v0) + q);
+      const float4 a = sd_ld4(rt + v0 + 4 * q);
       xt[4 * q] = a.x, xt[4 * q + 1] = a.y, xt[4 * q + 2] = a.z, xt[4 * q + 3] = a.w;
-      const float4 d = rd ? __ldcg(reinterpret_cast<const float4*>(rd + v0) + q) : make_float4(0.f, 0.f, 0.f, 0.f);
+      const float4 d = rd ? sd_ld4(rd + v0 + 4 * q) : make_float4(0.f, 0.f, 0.f, 0.f);
       xd[4 * q] = d.x, xd[4 * q + 1] = d.y, xd[4 * q + 2] = d.z, xd[4 * q + 3] = d.w;
     }
   } else if (vec) {

@@ -130,6 +130,14 @@ __device__ __forceinline__ float sd_ldcg_bf16(const __nv_bfloat16* p) {
   return __uint_as_float(static_cast<uint32_t>(__ldcg(reinterpret_cast<const unsigned short*>(p))) << 16);
 }
 
+// The same through L1, for what a warp reads in pieces of its sectors (after the wait
+// an ordinary load sees all that the earlier kernels wrote).
+__device__ __forceinline__ float4 sd_ld4(const float* p) {
+  float4 v;
+  asm volatile("ld.global.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "l"(p));
+  return v;
+}
+
 __device__ __forceinline__ float sd_bf16_lo(uint32_t w) { return __uint_as_float(w << 16); }
 __device__ __forceinline__ float sd_bf16_hi(uint32_t w) { return __uint_as_float(w & 0xffff0000u); }
 
