@@ -908,10 +908,9 @@ def sweep(args):
                 torch.cuda.empty_cache()
 
 
-# A launch shape like the 32-row fused layer kernel's (8 heads x a cluster of 8
-# CTAs; that kernel has 608 threads and 231,888 bytes of dynamic shared memory):
-# 352 threads, 230,976 bytes, 256 tensor-memory columns.
-FLOOR_SHAPE = {"ctas": 64, "cluster": 8, "threads": 352, "smem": 230976, "tmem_cols": 256}
+# The launch shape of the 32-row fused layer kernel (8 heads x a cluster of 8 CTAs):
+# 608 threads, 231,888 bytes of dynamic shared memory, 128 tensor-memory columns.
+FLOOR_SHAPE = {"ctas": 64, "cluster": 8, "threads": 608, "smem": 231888, "tmem_cols": 128}
 
 
 def floor(args):

@@ -254,8 +254,8 @@ int sd_verify_cluster_size(int B, int R, int Hq, int Hkv, int D, int capacity, i
  *   n_visual: int32 [B] device, mass: fp32 [B][R][Hq][3] device,
  *   entropy: fp32 [B][R][Hq] device; scale: 0 selects 1/sqrt(D).
  * One pass over the keys: bf16 tensor-core scores with fp32 accumulation,
- * fp32 sums with a running maximum per row (within 1e-4 of a float64 reference
- * on the target layer).
+ * fp32 sums relative to a row's maximum over 320 keys at a time (within 1e-4 of
+ * a float64 reference on the target layer).
  * D in {64, 128}, Hq % Hkv == 0. A scene with len[b] < R or len[b] >
  * capacity sets SD_DEVERR_LENGTH and is left unwritten; n_visual[b] outside
  * [0, L_b] sets it too and is clamped.
@@ -303,10 +303,10 @@ size_t sd_verify_layer_workspace(int B, int R, int Hq, int Hkv, int D, int capac
  *   SD_LAYER_BLOCK_MASK: the attention uses the block mask (as
  *   SD_ATTN_BLOCK_MASK of sd_verify_attention_ex).
  * For head_dim 128 this is one kernel: the tcgen05 kernel for G * R <= 128
- * and R <= 31;
- * other shapes run the three kernels in sequence (sd_verify_kernel names the
- * choice), the first two as one launch where the new rows are few. A scene whose append would pass the
- * capacity sets SD_DEVERR_KV_OVERFLOW and is left untouched.
+ * and R <= 31; other shapes run the three kernels in sequence (sd_verify_kernel
+ * names the choice), the first two as one launch where the new rows are few. A
+ * scene whose append would pass the capacity sets SD_DEVERR_KV_OVERFLOW and
+ * keeps its cache and length.
  */
 sd_status sd_verify_layer(void* q, void* k_new, const void* v_new, const int32_t* pos,
                           const int32_t sections[3], int interleaved, float base,
@@ -344,9 +344,11 @@ sd_status sd_accept_greedy(const void* logits, sd_dtype dtype, int B, int K, int
  * Same arguments, results and rules as sd_accept_greedy minus ws / ws_bytes.
  * Its scratch is a fixed array inside the library of
  * sd_accept_greedy_noalloc_max_bytes() bytes (1 MiB: per-scene tickets for up
- * to 4096 scenes, then B * (K + 1) * ceil(V / 4096) partials of 8 bytes), held
- * on every device that loads the library until the process exits. Larger
- * shapes return SD_ERR_WORKSPACE. Allocates nothing. The first call on a
+ * to 4096 scenes, then 8 bytes a row for its maximum), held on every device
+ * that loads the library until the process exits. Shapes of more than 4096
+ * scenes, or for which 8 bytes per 4096 values (sd_accept_greedy_workspace's
+ * measure, larger than the kernel's need) pass the rest, return
+ * SD_ERR_WORKSPACE. Allocates nothing. The first call on a
  * device resolves the array's device address (make it before any stream
  * capture). All calls share the array: calls that overlap on the device race
  * and must not be issued; every completed call leaves it ready for the next.
@@ -376,7 +378,11 @@ size_t sd_accept_sample_workspace(int B, int K, int V);
  * Outputs: n_emit [B] = l + 1 and tokens [B][K+1] (draft[0..l-1], the drawn
  * token, then -1). fp32 arithmetic with fixed-order reductions: the result is
  * a deterministic function of the inputs.
- * ws: as for sd_accept_greedy (zero-filled before first use, left zeroed).
+ * ws: device scratch of sd_accept_sample_workspace() bytes, zero-filled before
+ * its first use with a (B, K, V); a call leaves it ready for the next of the
+ * same (B, K, V), not zeroed: sharing it with another shape or with
+ * sd_accept_greedy takes a zero-fill in between. Calls that share it must not
+ * overlap on the device.
  */
 sd_status sd_accept_sample(const float* z_target, const float* z_draft, int B, int K,
                            int V, float temperature, const int32_t* draft,

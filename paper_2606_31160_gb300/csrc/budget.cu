@@ -112,10 +112,10 @@ __device__ __forceinline__ void mma_bf16(float (&c)[4], const uint32_t (&a)[4], 
 // independent product chains), takes their maximum once and folds them without a
 // running one; the sums merge over lanes, warps and CTAs by a common maximum, one
 // rescale and plain additions; and every CTA finishes 32 / S rows of the cluster.
-// One scene, 32 rows on each of 8 KV heads, 4096 keys: 7.8 us (14.9 with a running
+// One scene, 32 rows on each of 8 KV heads, 4096 keys: 7.9 us (14.9 with a running
 // maximum per thread, query fragments read from global memory before the keys, and one
 // CTA merging the cluster); of it the length takes 1.0 us, the keys 2.5, the products
-// 1.4, the fold 1.0, the merges and the exchange 2.2. Eight scenes 44.1 us (64.7).
+// 1.4, the fold 1.0, the merges and the exchange 2.2. Eight scenes 44.0 us (64.7).
 constexpr int kTiles = 2;
 constexpr int kPassRows = 16 * kTiles;
 constexpr int kChunkKeys = 320;  // keys a CTA stages at once (10 boxes of 32)

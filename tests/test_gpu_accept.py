@@ -45,9 +45,8 @@ def test_greedy_workloads(make):
 
 
 @pytest.mark.parametrize("dtype", [torch.bfloat16, torch.float32])
-# V * element size a multiple of 16 bytes takes the cluster kernel (V = 151936
-# fp32 with K = 16: 17 rows in four passes over 37,984-byte slices); other V
-# the chunked kernel
+# rows that all start on 16-byte boundaries (V * element size a multiple of 16), and
+# rows that do not
 @pytest.mark.parametrize("B,K,V", [(1, 0, 5), (3, 1, 4097), (8, 7, 151936), (2, 16, 32000), (5, 3, 123457),
                                    (2, 16, 151936)])
 def test_greedy_random(dtype, B, K, V):

@@ -150,9 +150,8 @@ def _fused_case(R, prefix, layer):
                                  layer=layer, tail_fill=float("nan"))
 
 
-# R = 8: 32 packed rows (32-row tile); R = 9 and 16: 36 and 64 rows (64-row
-# tile); R = 17: 68 rows, two 64-row m-blocks (the fused layer caps the
-# cluster size at 32 - R, so a forced 16 falls back to the automatic choice)
+# R = 8: 32 packed rows (32-row tile); R = 9 and 16: 36 and 64 rows (48- and 64-row
+# tiles); R = 17: 68 rows (80-row tile)
 @pytest.mark.parametrize("cluster", [1, 2, 4, 6, 8, 16])
 @pytest.mark.parametrize("R", [8, 9, 16, 17])
 def test_every_cluster_size(cluster, R):
