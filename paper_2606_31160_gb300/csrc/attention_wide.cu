@@ -33,12 +33,13 @@
 //
 // Fixed reference. Weights are 2^(score * scale - ref) with the row's score against its
 // own new key as its reference on every CTA of the cluster: the row's sum is about 1 or
-// more, scores may have any common offset, and the CTAs' partials add as they are. (Row
-// and key turn by the same angles, so the unrotated ones give it, while they are in
-// registers; nothing stands between S and P.) A floating-point weight keeps its relative
-// precision at any size, so only overflow matters: a row sum above 2^64 sends the CTA
-// through its range again with each row's exact maximum as its reference, one pass for
-// the maxima and one for the weights. Without a reference scores 40 away from 0 took
+// more, scores may have any common offset, and the CTAs' partials add as they are. (Both
+// turn by the same angles, in registers, on the way to shared memory: nothing stands
+// between S and P. Their score before the rotation would do but for its rounding to
+// bf16, which underflows every weight at scores of 1e4; it saved 0.07 us a layer.) A
+// floating-point weight keeps its relative precision at any size, so only overflow
+// matters: a row sum above 2^64 sends the CTA through its range again with each row's
+// exact maximum as its reference, one pass for the maxima and one for the weights. Without a reference scores 40 away from 0 took
 // those passes (8 scenes, L = 8192, K = 7: 38 -> 102 us), and values far from 1 left
 // fp32's range in the product; the references cost 0.1 to 0.2 us a layer.
 //
@@ -249,9 +250,9 @@ __device__ __forceinline__ void ldmatrix4(uint32_t addr, uint32_t (&r)[4]) {
                : "memory");
 }
 // The dot product of 8 bf16 pairs
-__device__ __forceinline__ float dot8(const uint4& x, const uint4& y) {
+__device__ __forceinline__ float dot8(const uint32_t (&x)[4], const uint32_t (&y)[4]) {
   auto dot2 = [](uint32_t a, uint32_t b) { return fmaf(sd_bf16_hi(a), sd_bf16_hi(b), sd_bf16_lo(a) * sd_bf16_lo(b)); };
-  return (dot2(x.x, y.x) + dot2(x.y, y.y)) + (dot2(x.z, y.z) + dot2(x.w, y.w));
+  return (dot2(x[0], y[0]) + dot2(x[1], y[1])) + (dot2(x[2], y[2]) + dot2(x[3], y[3]));
 }
 // Byte offset of 16-byte chunk c of row r in a 128-byte-swizzled pair of
 // 64-column halves, `half` bytes each.
@@ -690,25 +691,23 @@ __global__ void __launch_bounds__(kThreads, 1)
 #pragma unroll
       for (int u = 0; u < kQc; ++u) {
         const int idx = st + u * kSoftThreads, row = idx / kChunks, c = idx % kChunks, p = mblock * kR + row;
-        if (idx >= kR * kChunks) break;
-        uint32_t w[4] = {qv[u].x, qv[u].y, qv[u].z, qv[u].w};
+        if (idx >= kR * kChunks) break;  // warp-uniform
+        uint32_t w[4] = {qv[u].x, qv[u].y, qv[u].z, qv[u].w}, o[4] = {own[u].x, own[u].y, own[u].z, own[u].w};
         if (kFused) {  // (rows past M, zero, turn by the last row's angles: a branch cost 0.1 us a layer)
           const float2* cs = cs_tab + gdiv(min(p, a.M - 1)) * 64 + c * 4;
 #pragma unroll
-          for (int j = 0; j < 4; ++j) w[j] = sd_rope_pair(w[j], cs[j].x, cs[j].y);
+          for (int j = 0; j < 4; ++j) {
+            w[j] = sd_rope_pair(w[j], cs[j].x, cs[j].y);
+            o[j] = sd_rope_pair(o[j], cs[j].x, cs[j].y);
+          }
         }
         st_shared_v4(qs + swz(row, c, C::kQHalf), w[0], w[1], w[2], w[3]);
-      }
-      // the rows' references; a score that is not a number or infinite: 0
+        // the row's reference; a score that is not a number or infinite: 0
+        float d = dot8(w, o);
 #pragma unroll
-      for (int u = 0; u < kQc; ++u) {
-        const int idx = st + u * kSoftThreads;
-        if (idx >= kR * kChunks) break;  // warp-uniform
-        float d = dot8(qv[u], own[u]);
-#pragma unroll
-        for (int o = kChunks / 2; o > 0; o >>= 1) d += __shfl_xor_sync(0xffffffffu, d, o);
+        for (int x = kChunks / 2; x > 0; x >>= 1) d += __shfl_xor_sync(0xffffffffu, d, x);
         d *= sl;
-        if (idx % kChunks == 0) row_nref[idx / kChunks] = fabsf(d) < INFINITY ? -d : 0.f;
+        if (c == 0) row_nref[row] = fabsf(d) < INFINITY ? -d : 0.f;
       }
       if (last_rank && st < C::kMaxNew * kChunks) {
         // new key (rotated) and value rows, zero past R

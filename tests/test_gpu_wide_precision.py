@@ -102,3 +102,25 @@ def test_values_far_from_one(level, scale, G, R, fused, cluster, D):
         sd.set_cluster_size(0)
     ref = oracle.verify_attention(qd, kd, vd * 2.0 ** -scale, lens)
     assert attn_within(out * 2.0 ** -scale, ref), np.abs(out * 2.0 ** -scale - ref).max()
+
+
+@pytest.mark.parametrize("G,R", [(4, 1), (4, 8), (4, 12), (4, 17), (6, 16)])
+def test_scores_of_tens_of_thousands(G, R):
+    """Rotated rows whose one pair makes scores of 3e4: fp32 sums are off by some 2^-24 of
+    them there, 2% of a weight, and a row's reference has to be its rotated score (rounding
+    the rotated rows to bf16 moves it by 2^-8: 100 and more)."""
+    prefix = [0, 5, 700, 1500]
+    B, D = len(prefix), 128
+    q, k, v, k_new, v_new = _inputs(G * R, B, G, R, 2, 1540, D)
+    for x in (q, k, k_new):
+        x[..., 6], x[..., 7] = 500.0, 300.0
+    bf = workloads.to_bf16
+    cache = sd.KVCache(bf(k).cuda(), bf(v).cuda(), torch.tensor(prefix, dtype=torch.int32).cuda())
+    qd = bf(q).cuda()
+    pos = (37 + torch.arange(R, dtype=torch.int32))[None, :, None].expand(B, R, 3).contiguous().cuda()
+    out = torch.full_like(qd, float("nan"))
+    sd.verify_layer(qd, bf(k_new).cuda(), bf(v_new).cuda(), pos, (16, 24, 24), cache, 0, 1e6, out=out)
+    torch.cuda.synchronize()
+    assert sd.get_device_error() == 0
+    ref = oracle.verify_attention(to64(qd), to64(cache.k), to64(cache.v), cache.len.cpu().numpy())
+    assert np.isfinite(to64(out)).all() and np.abs(to64(out) - ref).max() < 0.2
