@@ -16,7 +16,7 @@
 // 153 -> 142 us, K = 8 165 -> 143, 1.0 of the measured copy). With one scene the
 // dependent path behind the previous kernel: rows, rotation, S(0), the tiles at
 // ~0.4 us of products each, the exchange (~0.7 us), the merge (target layer
-// 6.77 -> 6.35 us, K = 8 10.0 -> 7.5, K = 16 block 15.9 -> 10.65, draft step 6.8 -> 6.05
+// 6.77 -> 6.42 us, K = 8 10.0 -> 7.5, K = 16 block 15.9 -> 10.6, draft step 6.8 -> 6.1
 // on one cache).
 //
 // Head dim 64 (the attention; its layers run as the rotation, append and attention
